@@ -152,8 +152,6 @@ sap_status upload(sap_handle h, SweepState &sw, const double *U0)
     }
     WCK(cudaMemcpy(sw.Uhi, hi.data(), hi.size() * 2, cudaMemcpyHostToDevice));
     WCK(cudaMemcpy(sw.Ulo, lo.data(), lo.size() * 2, cudaMemcpyHostToDevice));
-    WCK(cudaMemset(sw.Y, 0, (size_t)sw.KY * r.Npad * sizeof(float)));
-    WCK(cudaMemset(sw.Yd, 0, (size_t)sw.KY * r.Npad * 2 * sizeof(float)));
     return SAP_OK;
 }
 
