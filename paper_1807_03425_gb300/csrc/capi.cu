@@ -320,6 +320,7 @@ sap_status enqueue_iteration(sap_handle h, double alpha, int eval_only, Partial 
             restructured_fuse_args(h, bv, u);
         }
         Timed t(h, K_UPDATE);
+        h->launches += select_update_launches(u) - 1;
         CK(launch_select_update(u, s));
     }
     return SAP_OK;
@@ -1168,6 +1169,7 @@ sap_status sap_shard_step(sap_handle h, double alpha, const sap_record *recs, in
     u.seeds_in_product = 1;  // a split handle is restructured: its product evaluates them
     {
         Timed t(h, K_UPDATE);
+        h->launches += select_update_launches(u) - 1;
         CK(launch_select_update(u, h->stream));
     }
     h->shard_steps++;
@@ -1204,9 +1206,13 @@ static sap_status graph_for(sap_handle h, double alpha, int eval_only, int chunk
     return SAP_OK;
 }
 
-static int kernels_per_iteration(sap_handle h)
+static int kernels_per_iteration(sap_handle h, bool update)
 {
-    return h->path == SAP_PLAIN ? 2 : restructured_kernels_per_iteration(h) + 1;
+    const bool plain = h->path == SAP_PLAIN;
+    // the recheck and the update of a large basis are two launches, unless
+    // the pass evaluated its candidates itself (second tier 5)
+    const bool two = update && update_is_cluster(h->dt == SAP_F64, h->n, h->k) && (plain || restructured_tier(h) != 5);
+    return (plain ? 2 : restructured_kernels_per_iteration(h) + 1) + (two ? 1 : 0);
 }
 
 sap_status sap_run(sap_handle h, double alpha, int32_t iters, double *hist, int64_t *argmins)
@@ -1227,7 +1233,7 @@ sap_status sap_run(sap_handle h, double alpha, int32_t iters, double *hist, int6
         if (s != SAP_OK) return s;
     } else {
         const int chunk = std::min(iters, 32);
-        const int kpi = kernels_per_iteration(h);
+        const int kpi = kernels_per_iteration(h, true);
         if (chunk > 0) {
             cudaGraphExec_t g;
             s = graph_for(h, alpha, 0, chunk, &g);
@@ -1248,7 +1254,7 @@ sap_status sap_run(sap_handle h, double alpha, int32_t iters, double *hist, int6
         s = graph_for(h, 0.0, 1, 1, &ge);
         if (s != SAP_OK) return s;
         CK(cudaGraphLaunch(ge, h->stream));
-        h->launches += kpi;
+        h->launches += kernels_per_iteration(h, false);
     }
     h->last_iters = iters;
     if (hist || argmins) return sap_get_history(h, hist, argmins, iters + 1);

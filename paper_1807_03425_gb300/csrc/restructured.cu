@@ -23,6 +23,7 @@
 // and near pairs hold NaN.
 #include "restructured.cuh"
 #include "tc_ptx.cuh"
+#include "update_cluster.cuh"
 
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -1763,6 +1764,7 @@ sap_status restructured_prepare(sap_handle h)
         RCK(cudaMalloc(&r.near_w, (size_t)r.near_cap * sizeof(float)));
         RCK(cudaMalloc(&r.xn, r.Npad * sizeof(float)));
         RCK(gemm_configure());
+        RCK(update_cluster_configure());
         RCK(configure_pass_kernels());
     }
     const int sms = handle_sms(h);

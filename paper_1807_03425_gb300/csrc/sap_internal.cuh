@@ -357,6 +357,20 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int *scratch, int *to
     return (w > 0 ? scratch[w - 1] : 0) + x - v;
 }
 
+// An approximate 1/sqrt(x) for x > 0 used as a column scale: the FP32
+// hardware estimate (relative error ~2^-23), widened.  A scale s applied to
+// column 0 of the Gram matrix (G' = S G S, S = diag(s, 1, ...)) and to row 0
+// of the Cholesky factor's inverse gives the same orthonormal basis for any
+// s; it only has to bring G'_00 within the series' 1e-5 of one, and this
+// estimate leaves it within ~5e-7.  (Each dependent FP64 operation costs
+// about 0.12 us here, so Newton steps toward full precision are not taken.)
+__device__ __forceinline__ double rsqrt_scale(double x)
+{
+    const float xf = (float)x;
+    if (!(xf > 1e-30f && xf < 1e30f)) return 1.0 / sqrt(x);
+    return (double)rsqrtf(xf);
+}
+
 // Extended-precision FP32 arithmetic for the explicit-difference tiers:
 // s + e = a + b exactly (Knuth's two-sum; the _rn intrinsics keep the
 // compiler from contracting the steps into FMAs).
@@ -593,7 +607,17 @@ struct SelectUpdateArgs {
     // blocks' best pairs in partials[0 .. pass_parts - 1]; one block takes
     // the argmin and updates (no list is read)
     int pass_parts = 0;
+    // 1: only the recheck; the blocks' best pairs stay in partials[] for the
+    // update by a cluster (update_cluster.cu)
+    int recheck_only = 0;
 };
 cudaError_t launch_select_update(const SelectUpdateArgs &a, cudaStream_t s);
+// Kernels that call launches: an update of FP32/BF16 data with k > 8 or
+// n > 128 is a launch of its own (update_cluster.cu) after the recheck.
+bool update_is_cluster(int x_is_f64, int n, int k);
+inline int select_update_launches(const SelectUpdateArgs &a)
+{
+    return (!a.eval_only && a.pass_parts == 0 && update_is_cluster(a.x_is_f64, a.n, a.k)) ? 2 : 1;
+}
 
 } // namespace sap

@@ -35,6 +35,7 @@
 // Steps 2-4 run in the data's precision (FP32 for FP32 data, FP64 for FP64
 // data); the recheck and the re-orthonormalisation are FP64.
 #include "sap_internal.cuh"
+#include "update_cluster.cuh"
 
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -56,20 +57,6 @@ __device__ __forceinline__ void seed_bar() { asm volatile("bar.sync 2, %0;" ::"n
 // 1/sqrt(x) in the working precision (FP32: the hardware approximation)
 __device__ __forceinline__ float rsq(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double rsq(double x) { return 1.0 / sqrt(x); }
-
-// An approximate 1/sqrt(x) for x > 0 used as a column scale: the FP32
-// hardware estimate (relative error ~2^-23), widened.  A scale s applied to
-// column 0 of the Gram matrix (G' = S G S, S = diag(s, 1, ...)) and to row 0
-// of the Cholesky factor's inverse gives the same orthonormal basis for any
-// s; it only has to bring G'_00 within the series' 1e-5 of one, and this
-// estimate leaves it within ~5e-7.  (Each dependent FP64 operation costs
-// about 0.12 us here, so Newton steps toward full precision are not taken.)
-__device__ __forceinline__ double rsqrt_scale(double x)
-{
-    const float xf = (float)x;
-    if (!(xf > 1e-30f && xf < 1e30f)) return 1.0 / sqrt(x);
-    return (double)rsqrtf(xf);
-}
 
 template <typename TX>
 __device__ __forceinline__ TX ld_x(const void *X, size_t idx)
@@ -97,8 +84,8 @@ __device__ __forceinline__ void block_sum_multi(V (&v)[M], V *scratch /* NW*M */
     __syncthreads();
 }
 
-// Dynamic shared memory of phase 2 when the basis fits: U' (FP64), D (data
-// precision, padded to 8 bytes) and the FP32 final basis.
+// Dynamic shared memory of the large-basis update (FP64 data) when it fits:
+// U' and D.
 template <typename TX>
 __host__ __device__ inline size_t su_dyn_bytes(int n, int K)
 {
@@ -625,9 +612,12 @@ __global__ void __launch_bounds__(SB) select_update_kernel(SelectUpdateArgs a)
         for (int q = 1; q < NW; ++q)
             if (better_q(sh.wb[q].r, sh.wb[q].i, sh.wb[q].j, b.r, b.i, b.j)) b = sh.wb[q];
         a.partials[blockIdx.x] = b;
-        __threadfence();
-        const unsigned int t = atomicAdd(&st->ticket, 1u);
-        sh.last = (t == gridDim.x - 1) ? 1 : 0;
+        sh.last = 0;
+        if (!a.recheck_only) {
+            __threadfence();
+            const unsigned int t = atomicAdd(&st->ticket, 1u);
+            sh.last = (t == gridDim.x - 1) ? 1 : 0;
+        }
     }
     __syncthreads();
     if (!sh.last) return;
@@ -1039,26 +1029,14 @@ __global__ void __launch_bounds__(SB) select_update_kernel(SelectUpdateArgs a)
     const Partial b = sh.wb[0];
     if (!(b.r < INFINITY) || a.eval_only) return;
 
-    // the watch pairs' coordinates, loaded now and used at the very end
+    // FP32 data: update_cluster.cu updates (the launch picks this kernel for
+    // such data's recheck and evaluations only)
+    if constexpr (sizeof(TX) == 8) {
     const int nwatch = sh.watch_n;
-    const bool prefetch = n <= 32 * kSeedRegs;
-    float wxi[kSeedRegs], wxj[kSeedRegs];
-    if (prefetch && w < nwatch && !a.seeds_in_product && SAP_PAIR_OK(st, sh.watch[w], a.N)) {
-        const int2 pr = sh.watch[w];
-#pragma unroll
-        for (int q = 0; q < kSeedRegs; ++q) {
-            const int l = lane + 32 * q;
-            wxi[q] = l < n ? (float)ld_x<TX>(a.X, (size_t)pr.x * n + l) : 0.f;
-            wxj[q] = l < n ? (float)ld_x<TX>(a.X, (size_t)pr.y * n + l) : 0.f;
-        }
-    }
-
-    float *Uf = nullptr;  // FP32 copy of the final basis (n x K) for the seeds
     {
         const bool in_smem = K <= 8 && su_dyn_bytes<TX>(n, K) <= kDynSmem;
         double *Up = in_smem ? dyn : a.work;           // n x K: the new basis before QR
         WT *Ds = reinterpret_cast<WT *>(Up + (size_t)n * K);  // n
-        if (in_smem) Uf = reinterpret_cast<float *>(dyn + (size_t)n * K + ((size_t)n * sizeof(WT) + 7) / 8);
 
         // 2. D = x_i - x_j, |D|^2 and U^T D in one multi-value reduction
         {
@@ -1255,7 +1233,7 @@ __global__ void __launch_bounds__(SB) select_update_kernel(SelectUpdateArgs a)
             double row[K];
 #pragma unroll
             for (int m = 0; m < K; ++m) row[m] = m < kk ? Up[(size_t)l * K + m] : 0.0;
-            write_row<TX, K>(a, sh, kk, l, row, Uf);
+            write_row<TX, K>(a, sh, kk, l, row, nullptr);
         }
         __syncthreads();
     }
@@ -1265,66 +1243,31 @@ __global__ void __launch_bounds__(SB) select_update_kernel(SelectUpdateArgs a)
         return;
     }
 
-    // seeds: the recent argmin pairs under the new basis
+    // seeds: the recent argmin pairs under the new basis, in FP64
     if (w < nwatch && SAP_PAIR_OK(st, sh.watch[w], a.N)) {
         const int2 pr = sh.watch[w];
-        float seed = INFINITY;
-        if (sizeof(TX) == 8) {
-            double v[K + 1];
+        double v[K + 1];
 #pragma unroll
-            for (int q = 0; q <= K; ++q) v[q] = 0.0;
-            for (int l = lane; l < n; l += 32) {
-                const double D = (double)ld_x<TX>(a.X, (size_t)pr.x * n + l) - (double)ld_x<TX>(a.X, (size_t)pr.y * n + l);
-                v[K] = fma(D, D, v[K]);
+        for (int q = 0; q <= K; ++q) v[q] = 0.0;
+        for (int l = lane; l < n; l += 32) {
+            const double D = (double)ld_x<TX>(a.X, (size_t)pr.x * n + l) - (double)ld_x<TX>(a.X, (size_t)pr.y * n + l);
+            v[K] = fma(D, D, v[K]);
 #pragma unroll
-                for (int c = 0; c < K; ++c)
-                    if (c < kk) v[c] = fma(a.U64[(size_t)c * n + l], D, v[c]);
-            }
-            warp_sum_multi<double, K + 1>(v);
-            double zz = 0.0;
-#pragma unroll
-            for (int c = 0; c < K; ++c) zz = fma(v[c], v[c], zz);
-            if (v[K] > 0.0) seed = __double2float_ru(sqrt(zz / v[K])) * 1.000001f;
-        } else {
-            float v[K + 1];
-#pragma unroll
-            for (int q = 0; q <= K; ++q) v[q] = 0.f;
-            if (prefetch) {
-#pragma unroll
-                for (int q = 0; q < kSeedRegs; ++q) {
-                    const int l = lane + 32 * q;
-                    if (l < n) {
-                        const float D = wxi[q] - wxj[q];
-                        v[K] = fmaf(D, D, v[K]);
-                        const float *ur_ = Uf ? Uf + (size_t)l * K : a.U32 + (size_t)l * a.KP;
-#pragma unroll
-                        for (int c = 0; c < K; ++c)
-                            if (c < kk) v[c] = fmaf(ur_[c], D, v[c]);
-                    }
-                }
-            } else {
-                for (int l = lane; l < n; l += 32) {
-                    const float D = (float)ld_x<TX>(a.X, (size_t)pr.x * n + l) - (float)ld_x<TX>(a.X, (size_t)pr.y * n + l);
-                    v[K] = fmaf(D, D, v[K]);
-                    const float *ur_ = Uf ? Uf + (size_t)l * K : a.U32 + (size_t)l * a.KP;
-#pragma unroll
-                    for (int c = 0; c < K; ++c)
-                        if (c < kk) v[c] = fmaf(ur_[c], D, v[c]);
-                }
-            }
-            warp_sum_multi<float, K + 1>(v);
-            float zz = 0.f;
-#pragma unroll
-            for (int c = 0; c < K; ++c) zz = fmaf(v[c], v[c], zz);
-            if (v[K] > 1e-30f) seed = cert_upper(sqrtf(zz / v[K]), a.seed_cert);
+            for (int c = 0; c < K; ++c)
+                if (c < kk) v[c] = fma(a.U64[(size_t)c * n + l], D, v[c]);
         }
-        if (lane == 0) sh.seed[w] = seed;
+        warp_sum_multi<double, K + 1>(v);
+        double zz = 0.0;
+#pragma unroll
+        for (int c = 0; c < K; ++c) zz = fma(v[c], v[c], zz);
+        if (lane == 0) sh.seed[w] = v[K] > 0.0 ? __double2float_ru(sqrt(zz / v[K])) * 1.000001f : INFINITY;
     }
     __syncthreads();
     if (tid == 0) {
         float m = INFINITY;
         for (int q = 0; q < nwatch; ++q) m = fminf(m, sh.seed[q]);
         st->seed_ub = __float_as_uint(m);
+    }
     }
 }
 
@@ -1365,8 +1308,24 @@ cudaError_t launch_su_t(const SelectUpdateArgs &a, cudaStream_t s)
 
 } // namespace
 
+// The small-basis form keeps a basis row in one thread's registers (warps
+// 0-3: n <= 128, k <= 8).  Beyond it FP32 and BF16 data take the cluster;
+// FP64 data stays with the last block of the recheck.
+bool update_is_cluster(int x_is_f64, int n, int k) { return !x_is_f64 && (k > 8 || n > 32 * kQW); }
+
 cudaError_t launch_select_update(const SelectUpdateArgs &a, cudaStream_t s)
 {
+    if (!a.eval_only && update_is_cluster(a.x_is_f64, a.n, a.k)) {
+        int nparts = a.pass_parts;
+        if (nparts == 0) {
+            SelectUpdateArgs r = a;
+            r.recheck_only = 1;
+            const cudaError_t e = launch_su_t<float>(r, s);
+            if (e != cudaSuccess) return e;
+            nparts = a.grid;
+        }
+        return launch_update_cluster(a, nparts, s);
+    }
     return a.x_is_f64 ? launch_su_t<double>(a, s) : launch_su_t<float>(a, s);
 }
 

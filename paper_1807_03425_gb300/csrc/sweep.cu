@@ -230,6 +230,7 @@ sap_status enqueue_iteration(sap_handle h, SweepState &sw, double alpha, int eva
         const SelectUpdateArgs u = update_args(h, sw, b, alpha, eval_only);
         cudaEvent_t ea, eb;
         handle_count_launch(h, 5, &ea, &eb);
+        handle_add_launches(h, select_update_launches(u) - 1);
         if (ea) cudaEventRecord(ea, b.stream);
         WCK(launch_select_update(u, b.stream));
         if (eb) cudaEventRecord(eb, b.stream);
