@@ -591,23 +591,10 @@ __global__ void __launch_bounds__(kPassThreads, 1) restr_pass_kernel(PassArgs a)
         if constexpr (EXPL) {
             if (!SAP_PAIR_OK(a.st, ij, a.N)) return;
             if (lane == 0) atomicAdd((unsigned int *)&a.st->cnt2, 1u);
-            // FP64: |D|^2 and U^T D with D = x_i - x_j (the FP64 recheck's sums)
-            // (the FP64 recheck's compute width for this k, so its sums
-            // are the same in the same order: the same q = r^2 bits)
+            // the FP64 recheck's compute width for this k
             constexpr int KS = K <= 8 ? K : K <= 12 ? 12 : K <= 16 ? 16 : K <= 24 ? 24 : 32;
-            double v[KS + 1];
-#pragma unroll
-            for (int q = 0; q <= KS; ++q) v[q] = 0.0;
-#pragma unroll 4
-            for (int l = lane; l < a.n; l += 32) {
-                const double D = (double)__ldg(a.X + (size_t)ij.x * a.n + l) - (double)__ldg(a.X + (size_t)ij.y * a.n + l);
-                v[KS] = fma(D, D, v[KS]);
-#pragma unroll
-                for (int c = 0; c < KS; ++c)
-                    if (c < a.k) v[c] = fma(__ldg(a.U64 + (size_t)c * a.n + l), D, v[c]);
-            }
             double zz, d2;
-            warp_ratio_parts<KS>(v, lane, zz, d2);
+            fp64_pair_parts<float, KS, true>(a.X, a.U64, a.n, a.k, ij, lane, zz, d2);
             if (d2 == 0.0 || d2 < a.eps2) return;
             const double q = zz / d2;
             if (better_q(q, ij.x, ij.y, best.r, best.i, best.j)) best = Partial{q, ij.x, ij.y};
@@ -1374,7 +1361,7 @@ struct RefineArgs {
     int n_near;
     Cert cert;               // rho (A unused: each pair has its own bound)
     ProbState *st;
-    int2 *cand2;
+    unsigned long long *cand2;  // packed (i, j, lower bound of the ratio)
     long long cap2;
     int pdl;
 };
@@ -1458,7 +1445,10 @@ __global__ void __launch_bounds__(256) refine_kernel(RefineArgs a)
                 b = __shfl_sync(0xffffffffu, b, 0);
                 if (emit) {
                     const long long pos = (long long)b + __popc(m & ((1u << lane) - 1u));
-                    if (pos < a.cap2) a.cand2[pos] = pr;
+                    // with a lower bound on its ratio, against which the FP64
+                    // recheck filters once the bound is final (rounded down)
+                    const float lb = code == 2 ? 0.f : fmaxf((r - bnd) / (1.0f + rho) * 0.999998f, 0.f);
+                    if (pos < a.cap2) a.cand2[pos] = pack_cand(pr.x, pr.y, lb, code == 2);
                     else atomicOr(&a.st->status, ST_OVERFLOW);
                 }
             }
@@ -2017,7 +2007,7 @@ sap_status restructured_enqueue_basis(sap_handle h, const BasisView &b, cudaStre
         x.n_near = r.n_near;
         x.cert = cert_refine(n, b.k);
         x.st = b.st;
-        x.cand2 = b.cand2;
+        x.cand2 = reinterpret_cast<unsigned long long *>(b.cand2);
         x.cap2 = b.cap;
         x.pdl = handle_tune(h).pdl;
         const int sms = handle_sms(h);
@@ -2209,6 +2199,15 @@ void restructured_fuse_args(sap_handle h, const BasisView &b, SelectUpdateArgs &
         u.list = b.cand2;
         u.which = 2;
         u.cert2 = cert_explicit_df(handle_n_dim(h), b.k);
+        return;
+    }
+    if (tier == 1) {
+        // the refine tier's packed list: the entries are lower bounds on the
+        // ratios, so the final bound itself is the threshold
+        u.fused = 4;
+        u.list = b.cand2;
+        u.which = 2;
+        u.cert2 = Cert{0.f, 0.f};
         return;
     }
     if (tier != 2 && tier != 3) return;

@@ -280,6 +280,96 @@ __device__ __forceinline__ void warp_ratio_parts(double (&v)[K + 1], int lane, d
     }
 }
 
+// FP64 sums of one pair by a warp: D = x_i - x_j, d2 = |D|^2 and zz =
+// |U^T D|^2 from explicit FP64 differences, delivered to every lane.  Every
+// form of the FP64 tier takes its squared ratio zz / d2 from here (or from
+// the block form in select_update.cu), so all forms give the same bits.
+//
+// Above kSliceN coordinates the sums are cut into kFp64Slices slices of the
+// coordinates (slice s: those with (l / 32) % kFp64Slices == s), each summed
+// over the warp by itself and added in slice order: a block can then give
+// each of its warps one slice.  A warp's FP64 instruction occupies its
+// sub-partition's pipe for about 64 cycles, so one warp alone needs n/32
+// (k + 1) of those per pair (107 us at n = 4096, k = 24).
+constexpr int kSliceN = 256;
+constexpr int kFp64Slices = 8;
+
+template <typename TX, bool RO>
+__device__ __forceinline__ double ld_fp64(const TX *p)
+{
+    if constexpr (RO) return (double)__ldg(p);
+    return (double)*p;
+}
+
+// One slice's warp totals: lane L returns the total of entry rs_index<S>(L)
+// (S = 8, 16 or 32 >= K + 1), K < 32; entries 0..K-1 are U^T D, entry K is |D|^2.
+template <typename TX, int K, bool RO>
+__device__ __forceinline__ double fp64_slice(const TX *xi, const TX *xj, const double *U64, int n, int k, int slice,
+                                             int lane, double &extra)
+{
+    double v[K + 1];
+#pragma unroll
+    for (int q = 0; q <= K; ++q) v[q] = 0.0;
+#pragma unroll 2
+    for (int l = slice * 32 + lane; l < n; l += 32 * kFp64Slices) {
+        const double D = ld_fp64<TX, RO>(xi + l) - ld_fp64<TX, RO>(xj + l);
+        v[K] = fma(D, D, v[K]);
+#pragma unroll
+        for (int c = 0; c < K; ++c)
+            if (c < k) v[c] = fma(ld_fp64<double, RO>(U64 + (size_t)c * n + l), D, v[c]);
+    }
+    constexpr int M = K + 1;
+    constexpr int S = M <= 8 ? 8 : M <= 16 ? 16 : 32;
+    double r[S];
+#pragma unroll
+    for (int q = 0; q < S; ++q) r[q] = q < M ? v[q < M ? q : 0] : 0.0;
+    extra = 0.0;
+    if constexpr (M > 32) {  // K = 32: |D|^2 is the 33rd sum
+        extra = v[K];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) extra += __shfl_xor_sync(0xffffffffu, extra, o);
+    }
+    return warp_reduce_scatter<S>(r, lane);
+}
+
+template <typename TX, int K, bool RO>
+__device__ __forceinline__ void fp64_pair_parts(const TX *X, const double *U64, int n, int k, int2 ij, int lane,
+                                                double &zz, double &d2)
+{
+    const TX *xi = X + (size_t)ij.x * n, *xj = X + (size_t)ij.y * n;
+    if (n <= kSliceN) {
+        double v[K + 1];
+#pragma unroll
+        for (int q = 0; q <= K; ++q) v[q] = 0.0;
+#pragma unroll 4
+        for (int l = lane; l < n; l += 32) {
+            const double D = ld_fp64<TX, RO>(xi + l) - ld_fp64<TX, RO>(xj + l);
+            v[K] = fma(D, D, v[K]);
+#pragma unroll
+            for (int c = 0; c < K; ++c)
+                if (c < k) v[c] = fma(ld_fp64<double, RO>(U64 + (size_t)c * n + l), D, v[c]);
+        }
+        warp_ratio_parts<K>(v, lane, zz, d2);
+        return;
+    }
+    constexpr int M = K + 1, S = M <= 8 ? 8 : M <= 16 ? 16 : 32, dup = 32 / S;
+    double t = 0.0, ex = 0.0;
+#pragma unroll 1
+    for (int s = 0; s < kFp64Slices; ++s) {
+        double e;
+        t += fp64_slice<TX, K, RO>(xi, xj, U64, n, k, s, lane, e);
+        ex += e;
+    }
+    zz = 0.0;
+#pragma unroll
+    for (int c = 0; c < K; ++c) {
+        const double z = __shfl_sync(0xffffffffu, t, c * dup);
+        zz = fma(z, z, zz);
+    }
+    if constexpr (M > 32) d2 = ex;
+    else d2 = __shfl_sync(0xffffffffu, t, K * dup);
+}
+
 // (q, i, j) ordering for q >= 0 (no NaN): the bit patterns of non-negative
 // doubles order like their values, so the compare stays off the FP64 pipe.
 __device__ __forceinline__ bool better_q(double q, int i, int j, double qb, int ib, int jb)
@@ -589,9 +679,9 @@ struct SelectUpdateArgs {
     //  fused == 3: the same pairs from explicit differences in extended
     //    precision (cert2), each survivor evaluated in FP64 at once by the
     //    same warp (k <= 8; the grid is the tier's);
-    //  fused == 4: the list (count in st->cnt2) holds the extended-precision
-    //    tier's packed (i, j, ratio) entries; those within the final bound
-    //    (cert2) are evaluated in FP64
+    //  fused == 4: the list (count in st->cnt2) holds a second tier's packed
+    //    (i, j, ratio) entries; those within the final bound (cert2) are
+    //    evaluated in FP64
     int fused;
     const int2 *near;
     int n_near;

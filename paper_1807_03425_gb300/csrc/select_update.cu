@@ -45,8 +45,7 @@ namespace {
 
 constexpr int SB = 256;          // threads per block
 constexpr int NW = SB / 32;
-constexpr size_t kDynSmem = 40 * 1024;  // dynamic part of phase 2 (static part < 8 KB: total within 48 KB)
-constexpr int kSeedRegs = 4;     // watch-pair coordinates prefetched per lane (n <= 128)
+constexpr size_t kDynSmem = 36 * 1024;  // dynamic part of phase 2 (static part < 12 KB at K <= 8: total within 48 KB)
 constexpr int kQW = 4;           // warps of the small-basis update (one row per thread, n <= 128)
 
 // Named barriers of phase 2: warps 0..kQW-1 (the small-basis update) and
@@ -89,7 +88,7 @@ __device__ __forceinline__ void block_sum_multi(V (&v)[M], V *scratch /* NW*M */
 template <typename TX>
 __host__ __device__ inline size_t su_dyn_bytes(int n, int K)
 {
-    return (size_t)n * K * 8 + ((size_t)n * sizeof(TX) + 7) / 8 * 8 + (size_t)n * K * 4;
+    return (size_t)n * K * 8 + (size_t)n * sizeof(TX);
 }
 
 template <typename WT, int K>
@@ -120,6 +119,7 @@ struct Shared {
     float R2f[KS][KS], Sqf[KS][KS];  // second-order terms of the series (K <= 8)
     int degen;                     // the rotated direction vanished (small-basis update)
     int scan[33];
+    int2 queue[SB];                // pairs waiting for the block's FP64 evaluation (n > kSliceN)
 };
 
 // FP64 evaluation of one pair by a warp: D = x_i - x_j, d^2 = |D|^2 and
@@ -131,23 +131,51 @@ template <typename TX, int K>
 __device__ __forceinline__ void fp64_eval(const SelectUpdateArgs &a, int2 ij, int lane, Partial &best)
 {
     if (!SAP_PAIR_OK(a.st, ij, a.N)) return;
-    const int n = a.n, kk = a.k;
-    double v[K + 1];
-#pragma unroll
-    for (int q = 0; q <= K; ++q) v[q] = 0.0;
-#pragma unroll 4
-    for (int l = lane; l < n; l += 32) {
-        const double D = (double)ld_x<TX>(a.X, (size_t)ij.x * n + l) - (double)ld_x<TX>(a.X, (size_t)ij.y * n + l);
-        v[K] = fma(D, D, v[K]);
-#pragma unroll
-        for (int c = 0; c < K; ++c)
-            if (c < kk) v[c] = fma(a.U64[(size_t)c * n + l], D, v[c]);
-    }
     double zz, d2;
-    warp_ratio_parts<K>(v, lane, zz, d2);
+    fp64_pair_parts<TX, K, false>(static_cast<const TX *>(a.X), a.U64, a.n, a.k, ij, lane, zz, d2);
     if (d2 == 0.0 || d2 < a.eps2) return;
     const double q = zz / d2;  // squared ratio
     if (better_q(q, ij.x, ij.y, best.r, best.i, best.j)) best = Partial{q, ij.x, ij.y};
+}
+
+// The same by a whole block, warp w summing slice w of the coordinates (n >
+// kSliceN); warp 0 keeps the best.
+template <typename TX, int K>
+__device__ __forceinline__ void fp64_eval_block(const SelectUpdateArgs &a, Shared<TX, K> &sh, int2 ij, int w, int lane,
+                                                Partial &best)
+{
+    static_assert(NW == kFp64Slices, "a slice per warp");
+    if (!SAP_PAIR_OK(a.st, ij, a.N)) return;
+    constexpr int M = K + 1, S = M <= 8 ? 8 : M <= 16 ? 16 : 32, dup = 32 / S;
+    const TX *X = static_cast<const TX *>(a.X);
+    double ex;
+    const double t = fp64_slice<TX, K, false>(X + (size_t)ij.x * a.n, X + (size_t)ij.y * a.n, a.U64, a.n, a.k, w, lane, ex);
+    const int idx = rs_index<S>(lane);
+    if (lane % dup == 0 && idx < M) sh.red_d[w * M + idx] = t;
+    if (M > 32 && lane == 0) sh.red_d[w * M + K] = ex;
+    __syncthreads();
+    if (w == 0) {
+        // the slices in order, then the squares in order (as fp64_pair_parts)
+        double z = 0.0, d2 = 0.0;
+        if (lane < M)
+            for (int s = 0; s < NW; ++s) z += sh.red_d[s * M + lane];
+        if constexpr (M > 32) {
+            for (int s = 0; s < NW; ++s) d2 += sh.red_d[s * M + K];
+        } else {
+            d2 = __shfl_sync(0xffffffffu, z, K);
+        }
+        double zz = 0.0;
+#pragma unroll
+        for (int c = 0; c < K; ++c) {
+            const double zc = __shfl_sync(0xffffffffu, z, c);
+            zz = fma(zc, zc, zz);
+        }
+        if (!(d2 == 0.0 || d2 < a.eps2)) {
+            const double q = zz / d2;
+            if (better_q(q, ij.x, ij.y, best.r, best.i, best.j)) best = Partial{q, ij.x, ij.y};
+        }
+    }
+    __syncthreads();
 }
 
 // The same evaluation from coordinates prefetched in registers (rows
@@ -576,29 +604,50 @@ __global__ void __launch_bounds__(SB) select_update_kernel(SelectUpdateArgs a)
                     fp64_eval<TX, K>(a, ij, lane, best);
                 }
             }
-        } else if (sizeof(TX) == 4 && a.fused == 4) {
-            // the extended-precision tier's list with its ratios: every pair
-            // that can still be the argmin under the final running bound is
-            // evaluated in FP64 (the tier emitted against earlier, looser
-            // values of the bound)
-            unsigned int cnt = *(volatile const unsigned int *)&st->cnt2;
-            if (cnt > a.cap) cnt = a.cap;
-            const float U = fminf(load_pos_float(&st->seed_ub), load_pos_float(&st->run_ub2));
-            const float th = cert_emit_threshold(U, a.cert2);
-            const unsigned long long *lst = reinterpret_cast<const unsigned long long *>(a.list);
-            for (unsigned int e = blockIdx.x + gridDim.x * w; e < cnt; e += gridDim.x * NW) {
-                const unsigned long long v = __ldcg(lst + e);
-                if (packed_ratio(v) <= th) fp64_eval<TX, K>(a, packed_pair(v), lane, best);  // uniform
-            }
         } else {
-            unsigned int cnt = a.which == 1 ? (unsigned int)st->cnt1 : (unsigned int)st->cnt2;
+            const bool packed = sizeof(TX) == 4 && a.fused == 4;
+            unsigned int cnt = !packed && a.which == 1 ? (unsigned int)st->cnt1 : (unsigned int)st->cnt2;
             if (cnt > a.cap) cnt = a.cap;
-            // the pair is read (within the list's storage) before the count
-            // is needed, so the two loads overlap
-            for (unsigned int e = blockIdx.x + gridDim.x * w; e < a.cap; e += gridDim.x * NW) {
-                const int2 ij = a.list[e];
-                if (e >= cnt) break;  // uniform over the warp
-                fp64_eval<TX, K>(a, ij, lane, best);
+            const unsigned long long *lst = reinterpret_cast<const unsigned long long *>(a.list);
+            // a packed list carries ratios (or lower bounds of them): every
+            // pair that can still be the argmin under the final running bound
+            // is evaluated (the tier emitted against earlier, looser values)
+            float th = INFINITY;
+            if (packed) th = cert_emit_threshold(fminf(load_pos_float(&st->seed_ub), load_pos_float(&st->run_ub2)), a.cert2);
+            if (n > kSliceN) {
+                // a block per pair, a slice of the coordinates per warp: the
+                // entries blockIdx.x + gridDim.x * t are read by thread t,
+                // the survivors queue in shared memory
+                for (long long base = 0; base < cnt; base += (long long)gridDim.x * SB) {
+                    const long long e = base + blockIdx.x + (long long)gridDim.x * tid;
+                    int2 ij = make_int2(0, 0);
+                    bool keep = e < cnt;
+                    if (keep && packed) {
+                        const unsigned long long v = __ldcg(lst + e);
+                        ij = packed_pair(v);
+                        keep = packed_ratio(v) <= th;
+                    } else if (keep) {
+                        ij = __ldcg(a.list + e);
+                    }
+                    int total;
+                    const int off = block_exclusive_scan(keep ? 1 : 0, sh.scan, &total);
+                    if (keep) sh.queue[off] = ij;
+                    __syncthreads();
+                    for (int p = 0; p < total; ++p) fp64_eval_block<TX, K>(a, sh, sh.queue[p], w, lane, best);
+                }
+            } else if (packed) {
+                for (unsigned int e = blockIdx.x + gridDim.x * w; e < cnt; e += gridDim.x * NW) {
+                    const unsigned long long v = __ldcg(lst + e);
+                    if (packed_ratio(v) <= th) fp64_eval<TX, K>(a, packed_pair(v), lane, best);  // uniform
+                }
+            } else {
+                // the pair is read (within the list's storage) before the count
+                // is needed, so the two loads overlap
+                for (unsigned int e = blockIdx.x + gridDim.x * w; e < a.cap; e += gridDim.x * NW) {
+                    const int2 ij = a.list[e];
+                    if (e >= cnt) break;  // uniform over the warp
+                    fp64_eval<TX, K>(a, ij, lane, best);
+                }
             }
         }
     }
@@ -1279,7 +1328,7 @@ cudaError_t launch_su(const SelectUpdateArgs &a, cudaStream_t s)
         // the small-basis update keeps its rows in registers; the new basis's
         // FP32 hi and lo parts go to shared memory for the seeds
         shm = sizeof(TX) == 4 ? (size_t)a.n * K * 8 : 0;
-    } else {
+    } else if (sizeof(TX) == 8) {
         const size_t need = su_dyn_bytes<TX>(a.n, K);
         shm = (K <= 8 && need <= kDynSmem) ? need : 0;
     }
