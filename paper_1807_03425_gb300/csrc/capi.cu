@@ -9,6 +9,7 @@
 // Nothing returns to the host inside the loop; sap_run replays captured
 // graphs of `chunk` iterations.
 #include "sap_internal.cuh"
+#include "basis_forms.cuh"
 #include "restructured.cuh"
 #include "softmin.cuh"
 #include "sweep.cuh"
@@ -79,6 +80,9 @@ struct sap_ctx {
     int2 *cand1 = nullptr, *cand2 = nullptr;
     long long cap = 0;
     Partial *partials = nullptr;
+    long long *pack = nullptr;   // results gathered for one copy to the host
+    size_t pack_cap = 0;
+    RunView *views = nullptr;    // batch: the datasets' result buffers
     double *work = nullptr;
     size_t work_elems = 0;
     ProbState *st = nullptr;
@@ -215,6 +219,16 @@ Cert cert_plain_f64()
     return c;
 }
 
+// The error a (non-zero) device status word stands for.
+sap_status status_error(sap_handle h, int status)
+{
+    if (status & ST_BOUNDS) return fail(h, SAP_E_BOUNDS, "a device index was out of range (debug build)");
+    if (status & ST_NO_SECANT) return fail(h, SAP_E_NO_SECANT, "every pair is excluded");
+    if (status & ST_TIMEOUT) return fail(h, SAP_E_TIMEOUT, "a device-side wait gave up");
+    if (status & ST_OVERFLOW) return fail(h, SAP_E_UNSUPPORTED, "candidate list overflow (too many near-ties)");
+    return SAP_OK;
+}
+
 sap_status sync_and_status(sap_handle h)
 {
     CK(cudaStreamSynchronize(h->stream));
@@ -222,12 +236,20 @@ sap_status sync_and_status(sap_handle h)
     CK(cudaMemcpy(&status, &h->st->status, sizeof(int), cudaMemcpyDeviceToHost));
     if (status) {
         CK(cudaMemset(&h->st->status, 0, sizeof(int)));
-        if (status & ST_BOUNDS) return fail(h, SAP_E_BOUNDS, "a device index was out of range (debug build)");
-        if (status & ST_NO_SECANT) return fail(h, SAP_E_NO_SECANT, "every pair is excluded");
-        if (status & ST_TIMEOUT) return fail(h, SAP_E_TIMEOUT, "a device-side wait gave up");
-        if (status & ST_OVERFLOW)
-            return fail(h, SAP_E_UNSUPPORTED, "candidate list overflow (too many near-ties)");
+        return status_error(h, status);
     }
+    return SAP_OK;
+}
+
+// Grows a device buffer of 64-bit words (contents are not kept).
+sap_status ensure_words(sap_handle h, long long **p, size_t *cap, size_t need)
+{
+    if (*cap >= need) return SAP_OK;
+    CK(cudaStreamSynchronize(h->stream));
+    dfree(*p);
+    *cap = 0;
+    CK(dalloc(p, need));
+    *cap = need;
     return SAP_OK;
 }
 
@@ -324,6 +346,17 @@ sap_status enqueue_iteration(sap_handle h, double alpha, int eval_only, Partial 
         CK(launch_select_update(u, s));
     }
     return SAP_OK;
+}
+
+// The basis `src` (device, n x k column-major FP64; the handle's own FP64
+// buffer or another) in every form the kernels read, on the handle's stream.
+cudaError_t basis_forms(sap_handle h, const double *src, bool reset)
+{
+    BasisFormsArgs f;
+    f.b[0] = BasisForms{h->U64, h->U32, h->U32lo, h->rs.Uhi, h->rs.Ulo, reset ? h->st : nullptr, h->k, h->KP, h->rs.NP};
+    f.bf16 = h->split == SAP_SPLIT_BF16;
+    f.hist_cap = h->hist_cap;
+    return launch_basis_forms(src, h->n, f, 1, h->stream);
 }
 
 sap_status reset_state(sap_handle h)
@@ -465,19 +498,7 @@ void handle_drop_graphs(sap_handle h) { drop_graphs(h); }
 bool handle_path_restructured(sap_handle h) { return h->path == SAP_RESTRUCTURED && h->dt != SAP_F64; }
 int handle_mode(sap_handle h) { return (int)h->mode; }
 Cert handle_seed_cert(int n, int k) { return cert_plain_f32(n, k); }
-sap_status handle_check_status(sap_handle h, ProbState *st)
-{
-    int status = 0;
-    CK(cudaMemcpy(&status, &st->status, sizeof(int), cudaMemcpyDeviceToHost));
-    if (status) {
-        CK(cudaMemset(&st->status, 0, sizeof(int)));
-        if (status & ST_BOUNDS) return fail(h, SAP_E_BOUNDS, "a device index was out of range (debug build)");
-        if (status & ST_NO_SECANT) return fail(h, SAP_E_NO_SECANT, "every pair is excluded");
-        if (status & ST_TIMEOUT) return fail(h, SAP_E_TIMEOUT, "a device-side wait gave up");
-        if (status & ST_OVERFLOW) return fail(h, SAP_E_UNSUPPORTED, "candidate list overflow (too many near-ties)");
-    }
-    return SAP_OK;
-}
+sap_status handle_status_error(sap_handle h, int status) { return status_error(h, status); }
 void handle_add_launches(sap_handle h, long long delta) { h->launches += delta; }
 } // namespace sap
 
@@ -572,7 +593,7 @@ sap_status sap_destroy(sap_handle h)
     softmin_free(h);
     sweep_free(h->sw);
     dfree(h->X32); dfree(h->X64); dfree(h->U64); dfree(h->U32); dfree(h->U32lo);
-    dfree(h->shard_rec); dfree(h->recs);
+    dfree(h->shard_rec); dfree(h->recs); dfree(h->pack); dfree(h->views);
     dfree(h->tiles); dfree(h->cand1); dfree(h->cand2); dfree(h->partials);
     dfree(h->work); dfree(h->st); dfree(h->hist); dfree(h->am);
     if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
@@ -772,9 +793,8 @@ sap_status sap_set_split(sap_handle h, sap_split s)
     sap_status st = restructured_prepare(h);
     if (st != SAP_OK || h->k == 0) return st;
     // re-split the current basis for the new operand type
-    std::vector<double> Uh((size_t)h->n * h->k);
-    CK(cudaMemcpy(Uh.data(), h->U64, Uh.size() * sizeof(double), cudaMemcpyDeviceToHost));
-    st = restructured_upload_basis(h, Uh.data());
+    CK(basis_forms(h, h->U64, false));
+    st = restructured_basis_changed(h);
     if (st != SAP_OK) return st;
     return tune_lookup(h);
 }
@@ -999,14 +1019,8 @@ sap_status sap_set_basis(sap_handle h, const double *U, int32_t k, int u_is_devi
     } else {
         std::memcpy(Uh.data(), U, Uh.size() * sizeof(double));
     }
-    double dev = 0.0;
-    for (int a = 0; a < k; ++a)
-        for (int b = 0; b < k; ++b) {
-            double s = 0.0;
-            for (int l = 0; l < n; ++l) s += Uh[(size_t)a * n + l] * Uh[(size_t)b * n + l];
-            dev = std::max(dev, std::fabs(s - (a == b ? 1.0 : 0.0)));
-        }
-    if (!(dev <= 1e-10)) return fail(h, SAP_E_NOT_ORTHONORMAL, "max |U^T U - I| > 1e-10");
+    if (!(orthonormality_error(Uh.data(), n, k) <= 1e-10))
+        return fail(h, SAP_E_NOT_ORTHONORMAL, "max |U^T U - I| > 1e-10");
     CK(cudaStreamSynchronize(h->stream));
     if (k != h->k) {
         drop_graphs(h);
@@ -1016,6 +1030,8 @@ sap_status sap_set_basis(sap_handle h, const double *U, int32_t k, int u_is_devi
         CK(dalloc(&h->U64, (size_t)n * k));
         CK(dalloc(&h->U32, (size_t)n * h->KP));
         CK(dalloc(&h->U32lo, (size_t)n * h->KP));
+        CK(cudaMemsetAsync(h->U32, 0, (size_t)n * h->KP * sizeof(float), h->stream));
+        CK(cudaMemsetAsync(h->U32lo, 0, (size_t)n * h->KP * sizeof(float), h->stream));
         h->work_elems = (size_t)(kMaxK + 1) * n;
         CK(dalloc(&h->work, h->work_elems));
         if (h->dt != SAP_F64) {
@@ -1023,25 +1039,16 @@ sap_status sap_set_basis(sap_handle h, const double *U, int32_t k, int u_is_devi
             if (s != SAP_OK) return s;
         }
     }
-    CK(cudaMemcpy(h->U64, Uh.data(), Uh.size() * sizeof(double), cudaMemcpyHostToDevice));
-    std::vector<float> u32((size_t)n * h->KP, 0.f), u32lo((size_t)n * h->KP, 0.f);
-    for (int l = 0; l < n; ++l)
-        for (int c = 0; c < k; ++c) {
-            const double v = Uh[(size_t)c * n + l];
-            const float f = (float)v;
-            u32[(size_t)l * h->KP + c] = f;
-            u32lo[(size_t)l * h->KP + c] = (float)(v - (double)f);
-        }
-    CK(cudaMemcpy(h->U32, u32.data(), u32.size() * sizeof(float), cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(h->U32lo, u32lo.data(), u32lo.size() * sizeof(float), cudaMemcpyHostToDevice));
+    // one copy (staged by the runtime before it returns), then every other
+    // form and the reset state by one kernel
+    CK(cudaMemcpyAsync(h->U64, Uh.data(), Uh.size() * sizeof(double), cudaMemcpyHostToDevice, h->stream));
+    CK(basis_forms(h, h->U64, true));
     if (h->dt != SAP_F64) {
-        sap_status s = restructured_upload_basis(h, Uh.data());
+        sap_status s = restructured_basis_changed(h);
         if (s != SAP_OK) return s;
     }
-    sap_status s = tune_lookup(h);
-    if (s != SAP_OK) return s;
     h->shard_steps = 0;
-    return reset_state(h);
+    return tune_lookup(h);
 }
 
 sap_status sap_get_basis(sap_handle h, double *U_out, int out_is_device)
@@ -1058,10 +1065,13 @@ sap_status sap_get_basis(sap_handle h, double *U_out, int out_is_device)
 
 static sap_status read_last(sap_handle h, int64_t *i, int64_t *j, double *ratio)
 {
-    sap_status s = sync_and_status(h);
-    if (s != SAP_OK) return s;
     ProbState p;
-    CK(cudaMemcpy(&p, h->st, sizeof(p), cudaMemcpyDeviceToHost));
+    CK(cudaMemcpyAsync(&p, h->st, sizeof(p), cudaMemcpyDeviceToHost, h->stream));
+    CK(cudaStreamSynchronize(h->stream));
+    if (p.status) {
+        CK(cudaMemsetAsync(&h->st->status, 0, sizeof(int), h->stream));
+        return status_error(h, p.status);
+    }
     if (i) *i = p.last_i;
     if (j) *j = p.last_j;
     if (ratio) *ratio = p.last_r;
@@ -1267,17 +1277,16 @@ sap_status sap_get_history(sap_handle h, double *hist, int64_t *argmins, int32_t
     if (h->last_iters < 0) return fail(h, SAP_E_STATE, "no sap_run yet");
     const int cnt = std::min(capacity, h->last_iters + 1);
     if (cnt < 0) return fail(h, SAP_E_ARG, "negative capacity");
-    sap_status s = sync_and_status(h);
+    const size_t words = gather_words(1, cnt, argmins != nullptr);
+    sap_status s = ensure_words(h, &h->pack, &h->pack_cap, words);
     if (s != SAP_OK) return s;
-    if (hist) CK(cudaMemcpy(hist, h->hist, (size_t)cnt * sizeof(double), cudaMemcpyDeviceToHost));
-    if (argmins) {
-        std::vector<int2> tmp(cnt);
-        CK(cudaMemcpy(tmp.data(), h->am, (size_t)cnt * sizeof(int2), cudaMemcpyDeviceToHost));
-        for (int q = 0; q < cnt; ++q) {
-            argmins[2 * q] = tmp[q].x;
-            argmins[2 * q + 1] = tmp[q].y;
-        }
-    }
+    CK(launch_gather(nullptr, RunView{h->hist, h->am, h->st}, 1, cnt, argmins != nullptr, h->pack, h->stream));
+    std::vector<long long> w(words);
+    CK(cudaMemcpyAsync(w.data(), h->pack, words * sizeof(long long), cudaMemcpyDeviceToHost, h->stream));
+    CK(cudaStreamSynchronize(h->stream));
+    if (w[0]) return status_error(h, (int)w[0]);
+    if (hist) std::memcpy(hist, w.data() + 1, (size_t)cnt * sizeof(double));
+    if (argmins) std::memcpy(argmins, w.data() + 1 + cnt, 2 * (size_t)cnt * sizeof(int64_t));
     return SAP_OK;
 }
 
@@ -1619,8 +1628,10 @@ sap_status sap_run_batch(sap_handle h, double alpha, int32_t iters, double *hist
         if (kid->k == 0) return fail(h, SAP_E_STATE, "dataset " + std::to_string(b) + " has no basis");
         sap_status st = ensure_hist(kid, iters + 1);
         if (st != SAP_OK) return kid_result(h, (int32_t)b, kid, st);
+        // the batch's graph runs after whatever the dataset's stream holds
         if (cudaMemsetAsync(&kid->st->iter, 0, sizeof(int), kid->stream) != cudaSuccess ||
-            cudaStreamSynchronize(kid->stream) != cudaSuccess)
+            cudaEventRecord(h->kid_done[b], kid->stream) != cudaSuccess ||
+            cudaStreamWaitEvent(h->stream, h->kid_done[b], 0) != cudaSuccess)
             return fail(h, SAP_E_CUDA, "dataset stream");
     }
     // the batch's graphs replay the datasets' buffers: rebuild them once any
@@ -1661,14 +1672,28 @@ sap_status sap_run_batch(sap_handle h, double alpha, int32_t iters, double *hist
     }
     if (st == SAP_OK) st = run(1, 1, 1);
     if (st != SAP_OK) return st;
-    CK(cudaStreamSynchronize(h->stream));
-    for (size_t b = 0; b < h->kids.size(); ++b) {
+    // every dataset's status, ratios and pairs in one copy
+    const int B = (int)h->kids.size(), cnt = iters + 1;
+    std::vector<RunView> views(B);
+    for (int b = 0; b < B; ++b) {
         sap_handle kid = h->kids[b];
         kid->last_iters = iters;
-        const size_t off = b * (size_t)(iters + 1);
-        st = sap_get_history(kid, hist ? hist + off : nullptr, argmins ? argmins + 2 * off : nullptr, iters + 1);
-        if (st != SAP_OK) return kid_result(h, (int32_t)b, kid, st);
+        views[b] = RunView{kid->hist, kid->am, kid->st};
     }
+    if (!h->views) CK(dalloc(&h->views, B));
+    const bool pairs = argmins != nullptr;
+    const size_t words = gather_words(B, cnt, pairs);
+    st = ensure_words(h, &h->pack, &h->pack_cap, words);
+    if (st != SAP_OK) return st;
+    CK(cudaMemcpyAsync(h->views, views.data(), (size_t)B * sizeof(RunView), cudaMemcpyHostToDevice, h->stream));
+    CK(launch_gather(h->views, views[0], B, cnt, pairs, h->pack, h->stream));
+    std::vector<long long> w(words);
+    CK(cudaMemcpyAsync(w.data(), h->pack, words * sizeof(long long), cudaMemcpyDeviceToHost, h->stream));
+    CK(cudaStreamSynchronize(h->stream));
+    for (int b = 0; b < B; ++b)
+        if (w[b]) return kid_result(h, b, h->kids[b], status_error(h->kids[b], (int)w[b]));
+    if (hist) std::memcpy(hist, w.data() + B, (size_t)B * cnt * sizeof(double));
+    if (pairs) std::memcpy(argmins, w.data() + B + (size_t)B * cnt, 2 * (size_t)B * cnt * sizeof(int64_t));
     return SAP_OK;
 }
 

@@ -1807,6 +1807,7 @@ sap_status restructured_basis_alloc(sap_handle h)
     RestrState &r = restr_state(h);
     const int k = handle_k(h);
     const bool bf16 = handle_split_bf16(h) != 0;
+    cudaStream_t s = handle_stream(h);
     dfree(r.Uhi);
     dfree(r.Ulo);
     dfree(r.Y);
@@ -1816,16 +1817,18 @@ sap_status restructured_basis_alloc(sap_handle h)
     r.KY = padded_stride(k);   // <= KPG; columns >= k are zero
     RCK(cudaMalloc(&r.Uhi, (size_t)r.KPG * r.NP * 2));
     RCK(cudaMalloc(&r.Ulo, (size_t)r.KPG * r.NP * 2));
+    RCK(cudaMemsetAsync(r.Uhi, 0, (size_t)r.KPG * r.NP * 2, s));  // pad rows and columns stay zero
+    RCK(cudaMemsetAsync(r.Ulo, 0, (size_t)r.KPG * r.NP * 2, s));
     RCK(cudaMalloc(&r.Y, (size_t)r.Npad * r.KY * sizeof(float)));
-    RCK(cudaMemset(r.Y, 0, (size_t)r.Npad * r.KY * sizeof(float)));
+    RCK(cudaMemsetAsync(r.Y, 0, (size_t)r.Npad * r.KY * sizeof(float), s));
     RCK(cudaMalloc(&r.Yd, (size_t)r.Npad * r.KY * 2 * sizeof(float)));
-    RCK(cudaMemset(r.Yd, 0, (size_t)r.Npad * r.KY * 2 * sizeof(float)));
+    RCK(cudaMemsetAsync(r.Yd, 0, (size_t)r.Npad * r.KY * 2 * sizeof(float), s));
     dfree(r.Ydh);
     dfree(r.Ydl);
     RCK(cudaMalloc(&r.Ydh, (size_t)r.Npad * r.KY * sizeof(float)));
     RCK(cudaMalloc(&r.Ydl, (size_t)r.Npad * r.KY * sizeof(float)));
-    RCK(cudaMemset(r.Ydh, 0, (size_t)r.Npad * r.KY * sizeof(float)));
-    RCK(cudaMemset(r.Ydl, 0, (size_t)r.Npad * r.KY * sizeof(float)));
+    RCK(cudaMemsetAsync(r.Ydh, 0, (size_t)r.Npad * r.KY * sizeof(float), s));
+    RCK(cudaMemsetAsync(r.Ydl, 0, (size_t)r.Npad * r.KY * sizeof(float), s));
     dfree(r.Ypart);
     if (r.ksplit > 1) RCK(cudaMalloc(&r.Ypart, (size_t)r.ksplit * r.Npad * r.KY * sizeof(float)));
     if (!make_map(&r.gemm.tb_hi, r.Uhi, bf16, r.NP, r.KPG, r.KPG) ||
@@ -1835,15 +1838,11 @@ sap_status restructured_basis_alloc(sap_handle h)
     return SAP_OK;
 }
 
-sap_status restructured_upload_basis(sap_handle h, const double *U)
+// The basis's operands were rewritten: the near list must fit its width.
+sap_status restructured_basis_changed(sap_handle h)
 {
-    RestrState &r = restr_state(h);
     const int k = handle_k(h);
-    std::vector<uint16_t> hi((size_t)r.KPG * r.NP, 0), lo((size_t)r.KPG * r.NP, 0);
-    restructured_split_host(h, U, k, hi.data(), lo.data());
-    RCK(cudaMemcpy(r.Uhi, hi.data(), hi.size() * 2, cudaMemcpyHostToDevice));
-    RCK(cudaMemcpy(r.Ulo, lo.data(), lo.size() * 2, cudaMemcpyHostToDevice));
-    if (r.k_cls != k) return classify(h, k);
+    if (restr_state(h).k_cls != k) return classify(h, k);
     return SAP_OK;
 }
 
@@ -2058,30 +2057,6 @@ bool restructured_u_maps(sap_handle h, void *Uhi, void *Ulo, int KPG, CUtensorMa
     RestrState &r = restr_state(h);
     const bool bf16 = handle_split_bf16(h) != 0;
     return make_map(mhi, Uhi, bf16, r.NP, KPG, KPG) && make_map(mlo, Ulo, bf16, r.NP, KPG, KPG);
-}
-
-void restructured_split_host(sap_handle h, const double *U, int k, uint16_t *hi, uint16_t *lo)
-{
-    RestrState &r = restr_state(h);
-    const int n = handle_n_dim(h);
-    const bool bf16 = handle_split_bf16(h) != 0;
-    const double lo_mul = bf16 ? 256.0 : 2048.0;
-    for (int c = 0; c < k; ++c)
-        for (int l = 0; l < n; ++l) {
-            const double v = U[(size_t)c * n + l];
-            const size_t idx = (size_t)c * r.NP + l;
-            if (bf16) {
-                const __nv_bfloat16 hv = __double2bfloat16(v);
-                const __nv_bfloat16 lv = __double2bfloat16((v - (double)__bfloat162float(hv)) * lo_mul);
-                std::memcpy(&hi[idx], &hv, 2);
-                std::memcpy(&lo[idx], &lv, 2);
-            } else {
-                const __half hv = __double2half(v);
-                const __half lv = __double2half((v - (double)__half2float(hv)) * lo_mul);
-                std::memcpy(&hi[idx], &hv, 2);
-                std::memcpy(&lo[idx], &lv, 2);
-            }
-        }
 }
 
 sap_status restructured_classify(sap_handle h, int k)

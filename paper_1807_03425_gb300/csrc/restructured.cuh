@@ -101,11 +101,10 @@ sap_status restructured_enqueue_product(sap_handle h, const CUtensorMap *mhi, co
                                         bool seeds = false);
 sap_status restructured_enqueue_basis(sap_handle h, const BasisView &b, cudaStream_t s); // pass + explicit tier
 bool restructured_u_maps(sap_handle h, void *Uhi, void *Ulo, int KPG, CUtensorMap *mhi, CUtensorMap *mlo);
-void restructured_split_host(sap_handle h, const double *U, int k, uint16_t *hi, uint16_t *lo); // k rows of NP
 sap_status restructured_classify(sap_handle h, int k);  // near list for width k (valid for every k' <= k)
 sap_status restructured_prepare(sap_handle h);          // X split, norms, lengths, near list
 sap_status restructured_basis_alloc(sap_handle h);      // U operands and Y for k
-sap_status restructured_upload_basis(sap_handle h, const double *U); // n x k col-major
+sap_status restructured_basis_changed(sap_handle h);    // after the basis's operands were rewritten
 sap_status restructured_enqueue(sap_handle h, double alpha);
 int restructured_kernels_per_iteration(sap_handle h);
 // Second tier of the restructured form: 0 explicit differences (own

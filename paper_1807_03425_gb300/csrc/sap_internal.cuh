@@ -337,7 +337,7 @@ __device__ __forceinline__ void fp64_pair_parts(const TX *X, const double *U64, 
                                                 double &zz, double &d2)
 {
     const TX *xi = X + (size_t)ij.x * n, *xj = X + (size_t)ij.y * n;
-    if (n <= kSliceN) {
+    if (sizeof(TX) == 8 || n <= kSliceN) {  // FP64 data: one chain at any n (one form evaluates it)
         double v[K + 1];
 #pragma unroll
         for (int q = 0; q <= K; ++q) v[q] = 0.0;
@@ -352,6 +352,7 @@ __device__ __forceinline__ void fp64_pair_parts(const TX *X, const double *U64, 
         warp_ratio_parts<K>(v, lane, zz, d2);
         return;
     }
+    if constexpr (sizeof(TX) == 4) {
     constexpr int M = K + 1, S = M <= 8 ? 8 : M <= 16 ? 16 : 32, dup = 32 / S;
     double t = 0.0, ex = 0.0;
 #pragma unroll 1
@@ -368,6 +369,7 @@ __device__ __forceinline__ void fp64_pair_parts(const TX *X, const double *U64, 
     }
     if constexpr (M > 32) d2 = ex;
     else d2 = __shfl_sync(0xffffffffu, t, K * dup);
+    }
 }
 
 // (q, i, j) ordering for q >= 0 (no NaN): the bit patterns of non-negative

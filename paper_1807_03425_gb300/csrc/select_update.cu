@@ -119,7 +119,7 @@ struct Shared {
     float R2f[KS][KS], Sqf[KS][KS];  // second-order terms of the series (K <= 8)
     int degen;                     // the rotated direction vanished (small-basis update)
     int scan[33];
-    int2 queue[SB];                // pairs waiting for the block's FP64 evaluation (n > kSliceN)
+    int2 queue[sizeof(WT) == 4 ? SB : 1];  // pairs waiting for the block's FP64 evaluation (n > kSliceN)
 };
 
 // FP64 evaluation of one pair by a warp: D = x_i - x_j, d^2 = |D|^2 and
@@ -614,7 +614,10 @@ __global__ void __launch_bounds__(SB) select_update_kernel(SelectUpdateArgs a)
             // is evaluated (the tier emitted against earlier, looser values)
             float th = INFINITY;
             if (packed) th = cert_emit_threshold(fminf(load_pos_float(&st->seed_ub), load_pos_float(&st->run_ub2)), a.cert2);
-            if (n > kSliceN) {
+            bool by_block = false;
+            if constexpr (sizeof(TX) == 4) by_block = n > kSliceN;
+            if (by_block) {
+                if constexpr (sizeof(TX) == 4) {
                 // a block per pair, a slice of the coordinates per warp: the
                 // entries blockIdx.x + gridDim.x * t are read by thread t,
                 // the survivors queue in shared memory
@@ -634,6 +637,7 @@ __global__ void __launch_bounds__(SB) select_update_kernel(SelectUpdateArgs a)
                     if (keep) sh.queue[off] = ij;
                     __syncthreads();
                     for (int p = 0; p < total; ++p) fp64_eval_block<TX, K>(a, sh, sh.queue[p], w, lane, best);
+                }
                 }
             } else if (packed) {
                 for (unsigned int e = blockIdx.x + gridDim.x * w; e < cnt; e += gridDim.x * NW) {

@@ -12,6 +12,7 @@
 // the bases' chains overlap on the GPU.
 #include "sweep.cuh"
 #include "restructured.cuh"
+#include "basis_forms.cuh"
 
 #include <algorithm>
 #include <cmath>
@@ -79,11 +80,16 @@ sap_status alloc_impl(sap_handle h, SweepState *&swp, int kmax, int hist_need)
     sw.ksplit = r.ksplit;
     WCK(cudaMalloc(&sw.Uhi, (size_t)sw.KPG * r.NP * 2));
     WCK(cudaMalloc(&sw.Ulo, (size_t)sw.KPG * r.NP * 2));
+    cudaStream_t s0 = handle_stream(h);
+    WCK(cudaMemsetAsync(sw.Uhi, 0, (size_t)sw.KPG * r.NP * 2, s0));  // pad rows and columns stay zero
+    WCK(cudaMemsetAsync(sw.Ulo, 0, (size_t)sw.KPG * r.NP * 2, s0));
     WCK(cudaMalloc(&sw.Y, (size_t)sw.KY * r.Npad * sizeof(float)));
     WCK(cudaMalloc(&sw.Yd, (size_t)sw.KY * r.Npad * 2 * sizeof(float)));
     if (sw.ksplit > 1) WCK(cudaMalloc(&sw.Ypart, (size_t)sw.ksplit * sw.KY * r.Npad * sizeof(float)));
     WCK(cudaMalloc(&sw.gst, sizeof(ProbState)));
-    WCK(cudaMemset(sw.gst, 0, sizeof(ProbState)));
+    WCK(cudaMemsetAsync(sw.gst, 0, sizeof(ProbState), s0));
+    WCK(cudaMalloc(&sw.views, (size_t)(kmax + 1) * sizeof(RunView)));
+    WCK(cudaMalloc(&sw.pack, gather_words(kmax + 1, 1, false) * sizeof(long long)));
     WCK(cudaEventCreateWithFlags(&sw.fork, cudaEventDisableTiming));
     if (!restructured_u_maps(h, sw.Uhi, sw.Ulo, sw.KPG, &sw.mhi, &sw.mlo))
         return handle_fail(h, SAP_E_CUDA, "cuTensorMapEncodeTiled failed for the sweep's bases");
@@ -105,10 +111,12 @@ sap_status alloc_impl(sap_handle h, SweepState *&swp, int kmax, int hist_need)
         WCK(cudaMalloc(&b.U64, (size_t)n * b.k * sizeof(double)));
         WCK(cudaMalloc(&b.Ydh, (size_t)b.KY * r.Npad * sizeof(float)));
         WCK(cudaMalloc(&b.Ydl, (size_t)b.KY * r.Npad * sizeof(float)));
-        WCK(cudaMemset(b.Ydh, 0, (size_t)b.KY * r.Npad * sizeof(float)));
-        WCK(cudaMemset(b.Ydl, 0, (size_t)b.KY * r.Npad * sizeof(float)));
+        WCK(cudaMemsetAsync(b.Ydh, 0, (size_t)b.KY * r.Npad * sizeof(float), s0));
+        WCK(cudaMemsetAsync(b.Ydl, 0, (size_t)b.KY * r.Npad * sizeof(float), s0));
         WCK(cudaMalloc(&b.U32, (size_t)n * b.KP * sizeof(float)));
         WCK(cudaMalloc(&b.U32lo, (size_t)n * b.KP * sizeof(float)));
+        WCK(cudaMemsetAsync(b.U32, 0, (size_t)n * b.KP * sizeof(float), s0));
+        WCK(cudaMemsetAsync(b.U32lo, 0, (size_t)n * b.KP * sizeof(float), s0));
         WCK(cudaMalloc(&b.work, (size_t)(kMaxK + 1) * n * sizeof(double)));
         WCK(cudaMalloc(&b.st, sizeof(ProbState)));
         WCK(cudaMalloc(&b.cand1, (size_t)sw.cap * sizeof(int2)));
@@ -123,35 +131,26 @@ sap_status alloc_impl(sap_handle h, SweepState *&swp, int kmax, int hist_need)
     return SAP_OK;
 }
 
-// Initial bases: basis k is the first k columns of U0 (n x kmax).
+// Initial bases: basis k is the first k columns of U0 (n x kmax), uploaded
+// once into the widest basis's FP64 buffer; every form of every basis and the
+// fresh states by one kernel.
 sap_status upload(sap_handle h, SweepState &sw, const double *U0)
 {
     RestrState &r = restr_state(h);
     const int n = handle_n_dim(h);
-    std::vector<uint16_t> hi((size_t)sw.KPG * r.NP, 0), lo((size_t)sw.KPG * r.NP, 0);
-    for (SweepBasis &b : sw.b) {
-        WCK(cudaMemcpy(b.U64, U0, (size_t)n * b.k * sizeof(double), cudaMemcpyHostToDevice));
-        std::vector<float> u32((size_t)n * b.KP, 0.f), u32lo((size_t)n * b.KP, 0.f);
-        for (int l = 0; l < n; ++l)
-            for (int c = 0; c < b.k; ++c) {
-                const double v = U0[(size_t)c * n + l];
-                const float f = (float)v;
-                u32[(size_t)l * b.KP + c] = f;
-                u32lo[(size_t)l * b.KP + c] = (float)(v - (double)f);
-            }
-        WCK(cudaMemcpy(b.U32, u32.data(), u32.size() * sizeof(float), cudaMemcpyHostToDevice));
-        WCK(cudaMemcpy(b.U32lo, u32lo.data(), u32lo.size() * sizeof(float), cudaMemcpyHostToDevice));
-        restructured_split_host(h, U0, b.k, hi.data() + (size_t)b.off * r.NP, lo.data() + (size_t)b.off * r.NP);
-        ProbState p;
-        std::memset(&p, 0, sizeof(p));
-        p.seed_ub = p.run_ub1 = p.run_ub2 = 0x7f800000u;
-        p.hist_cap = sw.hist_cap;
-        p.last_r = INFINITY;
-        p.last_i = p.last_j = -1;
-        WCK(cudaMemcpy(b.st, &p, sizeof(p), cudaMemcpyHostToDevice));
+    cudaStream_t s0 = handle_stream(h);
+    double *src = sw.b.back().U64;
+    WCK(cudaMemcpyAsync(src, U0, (size_t)n * sw.kmax * sizeof(double), cudaMemcpyHostToDevice, s0));
+    static_assert(kMaxForms >= 20, "one upload for all bases");
+    BasisFormsArgs f;
+    for (int q = 0; q < sw.kmax; ++q) {
+        SweepBasis &b = sw.b[q];
+        f.b[q] = BasisForms{b.U64, b.U32, b.U32lo, static_cast<uint16_t *>(sw.Uhi) + (size_t)b.off * r.NP,
+                            static_cast<uint16_t *>(sw.Ulo) + (size_t)b.off * r.NP, b.st, b.k, b.KP, r.NP};
     }
-    WCK(cudaMemcpy(sw.Uhi, hi.data(), hi.size() * 2, cudaMemcpyHostToDevice));
-    WCK(cudaMemcpy(sw.Ulo, lo.data(), lo.size() * 2, cudaMemcpyHostToDevice));
+    f.bf16 = handle_split_bf16(h);
+    f.hist_cap = sw.hist_cap;
+    WCK(launch_basis_forms(src, n, f, sw.kmax, s0));
     return SAP_OK;
 }
 
@@ -314,14 +313,8 @@ sap_status sweep_run(sap_handle h, const double *U0, int kmax, int iters, double
     if (!handle_x32(h)) return handle_fail(h, SAP_E_UNSUPPORTED, "the sweep needs FP32 or BF16 data");
     if (total_width(kmax) > kSweepMaxKY) return handle_fail(h, SAP_E_UNSUPPORTED, "the sweep supports k_max <= 20");
     // U0 must have orthonormal columns (then every prefix does)
-    double dev = 0.0;
-    for (int a = 0; a < kmax; ++a)
-        for (int c = 0; c <= a; ++c) {
-            double s = 0.0;
-            for (int l = 0; l < n; ++l) s += U0[(size_t)a * n + l] * U0[(size_t)c * n + l];
-            dev = std::max(dev, std::fabs(s - (a == c ? 1.0 : 0.0)));
-        }
-    if (!(dev <= 1e-10)) return handle_fail(h, SAP_E_NOT_ORTHONORMAL, "max |U0^T U0 - I| > 1e-10");
+    if (!(orthonormality_error(U0, n, kmax) <= 1e-10))
+        return handle_fail(h, SAP_E_NOT_ORTHONORMAL, "max |U0^T U0 - I| > 1e-10");
     cudaStream_t s0 = handle_stream(h);
     WCK(cudaStreamSynchronize(s0));
     SweepState *&swp = sweep_state(h);
@@ -335,18 +328,25 @@ sap_status sweep_run(sap_handle h, const double *U0, int kmax, int iters, double
     st = run_graph(h, sw, alpha, 0, iters);
     if (st == SAP_OK) st = run_graph(h, sw, 0.0, 1, 1);
     if (st != SAP_OK) return st;
+    // every basis's status and final ratio (and the product's status) in one
+    // copy
+    std::vector<RunView> views(kmax + 1);
+    views[0] = RunView{sw.b[0].hist + iters, sw.b[0].am + iters, sw.gst};
+    for (int q = 0; q < kmax; ++q) views[q + 1] = RunView{sw.b[q].hist + iters, sw.b[q].am + iters, sw.b[q].st};
+    WCK(cudaMemcpyAsync(sw.views, views.data(), views.size() * sizeof(RunView), cudaMemcpyHostToDevice, s0));
+    WCK(launch_gather(sw.views, views[0], kmax + 1, 1, false, sw.pack, s0));
+    std::vector<long long> w(gather_words(kmax + 1, 1, false));
+    WCK(cudaMemcpyAsync(w.data(), sw.pack, w.size() * sizeof(long long), cudaMemcpyDeviceToHost, s0));
     WCK(cudaStreamSynchronize(s0));
-    st = handle_check_status(h, sw.gst);
-    for (SweepBasis &b : sw.b)
-        if (st == SAP_OK) st = handle_check_status(h, b.st);
-    if (st != SAP_OK) return st;
+    for (int q = 0; q <= kmax; ++q)
+        if (w[q]) return handle_status_error(h, (int)w[q]);
     sw.last_iters = iters;
     int kk = -1;
-    for (SweepBasis &b : sw.b) {
+    for (int q = 0; q < kmax; ++q) {
         double r = 0.0;
-        WCK(cudaMemcpy(&r, b.hist + iters, sizeof(double), cudaMemcpyDeviceToHost));
-        if (ratios_out) ratios_out[b.k - 1] = r;
-        if (kk < 0 && r > threshold) kk = b.k;
+        std::memcpy(&r, &w[kmax + 1 + q + 1], sizeof(double));
+        if (ratios_out) ratios_out[q] = r;
+        if (kk < 0 && r > threshold) kk = q + 1;
     }
     if (k_out) *k_out = kk;
     // the handle's own basis goes back to its own near classification
@@ -396,6 +396,7 @@ void sweep_free(SweepState *&s)
         if (b.done) cudaEventDestroy(b.done);
     }
     wfree(s->Uhi); wfree(s->Ulo); wfree(s->Y); wfree(s->Yd); wfree(s->Ypart); wfree(s->gst);
+    wfree(s->views); wfree(s->pack);
     if (s->fork) cudaEventDestroy(s->fork);
     delete s;
     s = nullptr;

@@ -6,6 +6,7 @@
 #include <vector>
 
 #include "sap_internal.cuh"
+#include "basis_forms.cuh"
 #include "../../include/sap.h"
 
 namespace sap {
@@ -40,6 +41,8 @@ struct SweepState {
     float *Ypart = nullptr;
     int ksplit = 1;
     ProbState *gst = nullptr;             // status word of the product
+    RunView *views = nullptr;             // kmax + 1 result buffers (the product's status first)
+    long long *pack = nullptr;            // their status words and final ratios
     cudaEvent_t fork = nullptr;
     // captured chunks, reused while the handle's buffers and settings stay
     struct Graph {
@@ -62,6 +65,6 @@ SweepState *&sweep_state(sap_handle h);
 long long handle_graph_gen(sap_handle h);
 int handle_mode(sap_handle h);
 Cert handle_seed_cert(int n, int k);
-sap_status handle_check_status(sap_handle h, ProbState *st);
+sap_status handle_status_error(sap_handle h, int status);
 
 } // namespace sap
