@@ -26,6 +26,7 @@
 // off-diagonal Frobenius norm is below 4 n 2^-53 of the whole (quadratic
 // convergence: typically 6 to 10 sweeps), or after 40.
 #include "sap_internal.cuh"
+#include "colmean.cuh"
 #include "../../include/sap.h"
 
 #include <algorithm>
@@ -156,16 +157,6 @@ __global__ void __launch_bounds__(256) lap_rows_kernel(const TX *X, int N, int n
     }
 }
 
-template <typename TX>
-__global__ void colmean64_kernel(const TX *X, int N, int n, double *mean)
-{
-    const int l = blockIdx.x * blockDim.x + threadIdx.x;
-    if (l >= n) return;
-    double s = 0.0;
-    for (int i = 0; i < N; ++i) s += ldx(X, (size_t)i * n + l);
-    mean[l] = s / N;
-}
-
 // C[a][b] = sum_i (x_ia - mean_a) R_ib over a 16 x 16 block of (a, b).
 template <typename TX>
 __global__ void __launch_bounds__(256) gram_kernel(const TX *X, const double *mean, const double *R, int N, int n,
@@ -294,14 +285,14 @@ __global__ void jacobi_norms_kernel(const double *A, int n, double *out)
 
 struct Scratch {
     double *w = nullptr, *R = nullptr, *mean = nullptr, *C = nullptr, *C2 = nullptr, *V = nullptr, *V2 = nullptr,
-           *norms = nullptr;
+           *norms = nullptr, *part = nullptr;
     double2 *fg = nullptr;
     int2 *tiles = nullptr;
     int *partner = nullptr;
     ~Scratch()
     {
         for (void *p : {(void *)w, (void *)R, (void *)mean, (void *)C, (void *)C2, (void *)V, (void *)V2,
-                        (void *)norms, (void *)fg, (void *)tiles, (void *)partner})
+                        (void *)norms, (void *)part, (void *)fg, (void *)tiles, (void *)partner})
             if (p) cudaFree(p);
     }
 };
@@ -334,6 +325,7 @@ sap_status secant_pca(sap_handle h, int k, double *U_out, double *sigma_out)
     PCK(cudaMalloc(&sc.w, (size_t)ntiles * PT * PT * sizeof(double)));
     PCK(cudaMalloc(&sc.R, (size_t)N * n * sizeof(double)));
     PCK(cudaMalloc(&sc.mean, (size_t)n * sizeof(double)));
+    PCK(cudaMalloc(&sc.part, colmean_scratch(N, n) * sizeof(double)));
     PCK(cudaMalloc(&sc.C, (size_t)n * n * sizeof(double)));
     PCK(cudaMalloc(&sc.C2, (size_t)n * n * sizeof(double)));
     PCK(cudaMalloc(&sc.V, (size_t)n * n * sizeof(double)));
@@ -346,12 +338,12 @@ sap_status secant_pca(sap_handle h, int k, double *U_out, double *sigma_out)
     if (X64) {
         w64_kernel<double><<<(unsigned)ntiles, 256, 0, s>>>(X64, N, n, sc.tiles, eps2, sc.w);
         lap_rows_kernel<double><<<lgrid, 256, 0, s>>>(X64, N, n, sc.w, nb, sc.R);
-        colmean64_kernel<double><<<(n + 127) / 128, 128, 0, s>>>(X64, N, n, sc.mean);
+        PCK(launch_colmean(X64, N, n, sc.part, sc.mean, s));
         gram_kernel<double><<<ggrid, 256, 0, s>>>(X64, sc.mean, sc.R, N, n, sc.C);
     } else {
         w64_kernel<float><<<(unsigned)ntiles, 256, 0, s>>>(X32, N, n, sc.tiles, eps2, sc.w);
         lap_rows_kernel<float><<<lgrid, 256, 0, s>>>(X32, N, n, sc.w, nb, sc.R);
-        colmean64_kernel<float><<<(n + 127) / 128, 128, 0, s>>>(X32, N, n, sc.mean);
+        PCK(launch_colmean(X32, N, n, sc.part, sc.mean, s));
         gram_kernel<float><<<ggrid, 256, 0, s>>>(X32, sc.mean, sc.R, N, n, sc.C);
     }
     PCK(cudaGetLastError());

@@ -22,6 +22,7 @@
 // w + t*128*128; entries with i >= j, with an index beyond N, excluded pairs
 // and near pairs hold NaN.
 #include "restructured.cuh"
+#include "colmean.cuh"
 #include "tc_ptx.cuh"
 #include "update_cluster.cuh"
 
@@ -41,15 +42,6 @@ constexpr int T = kTile;       // 128
 constexpr int WLC = 16;        // coordinates per chunk in the length prep
 
 // ------------------------------------------------------------------ prep ---
-
-__global__ void colmean_kernel(const float *X, int N, int n, float *center)
-{
-    const int l = blockIdx.x * blockDim.x + threadIdx.x;
-    if (l >= n) return;
-    double acc = 0.0;
-    for (int i = 0; i < N; ++i) acc += (double)X[(size_t)i * n + l];
-    center[l] = (float)(acc / N);
-}
 
 __global__ void absmax_kernel(const float *X, size_t count, int n, const float *center,
                               unsigned int *out)
@@ -152,45 +144,84 @@ __device__ bool excluded_fp64(const float *X, int n, int i, int j, double eps2)
 }
 
 // One 128 x 128 tile of lengths per block: 256 threads, 8 x 8 pairs each.
-__global__ void __launch_bounds__(256) wprep_kernel(WPrepArgs a)
+// Bound by FP32 issue (2 n operations per pair; the 6 bytes per pair it
+// writes take a tenth of that at n = 90), so the differences and squares are
+// packed FP32 pairs (half the instructions, the same roundings in the same
+// order) and the next chunk's points are copied asynchronously while a chunk
+// is evaluated.  Chunk coordinate l of point r is staged at [l][r ^ 4 (l %
+// 8)], and a warp copies 8 coordinates (one 32-byte sector) of 4 points: no
+// bank conflicts on either side, and the readers' 16-byte groups stay whole.
+__global__ void __launch_bounds__(256, 2) wprep_kernel(WPrepArgs a)
 {
-    __shared__ __align__(16) float xsI[WLC][T + 4];
-    __shared__ __align__(16) float xsJ[WLC][T + 4];
+    __shared__ __align__(16) float xsI[2][WLC][T];
+    __shared__ __align__(16) float xsJ[2][WLC][T];
     __shared__ int scan[33];
     __shared__ int base_sh;
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const int2 IJ = a.wtiles[blockIdx.x];
     const int i0 = IJ.x * T, j0 = IJ.y * T;
+    uint64_t acc[8][4];  // row p, columns 2 c and 2 c + 1
+#pragma unroll
+    for (int p = 0; p < 8; ++p)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[p][c] = 0ull;
+    // thread: chunk coordinate sl of the points sr, sr + 16, ...
+    const int sl = ((tid >> 2) & 7) + 8 * ((tid >> 5) & 1), sr = (tid & 3) + 4 * (tid >> 6);
+    auto copy = [&](int l0, int st) {
+        const int gl = l0 + sl;
+        const bool inl = gl < a.n;
+#pragma unroll
+        for (int q = 0; q < T / 16; ++q) {
+            const int r = sr + 16 * q, col = r ^ ((sl & 7) << 2);
+            const bool ini = inl && i0 + r < a.N, inj = inl && j0 + r < a.N;
+            tc::cp_async4(&xsI[st][sl][col], ini ? a.X + (size_t)(i0 + r) * a.n + gl : a.X, ini);
+            tc::cp_async4(&xsJ[st][sl][col], inj ? a.X + (size_t)(j0 + r) * a.n + gl : a.X, inj);
+        }
+        tc::cp_async_commit();
+    };
+    copy(0, 0);
+    for (int l0 = 0, st = 0; l0 < a.n; l0 += WLC, st ^= 1) {
+        if (l0 + WLC < a.n) {
+            copy(l0 + WLC, st ^ 1);
+            tc::cp_async_wait<1>();
+        } else {
+            tc::cp_async_wait<0>();
+        }
+        __syncthreads();
+        // coordinates past n are zero on both sides: they add nothing
+#pragma unroll 4
+        for (int l = 0; l < WLC; ++l) {
+            const int sw = (l & 7) << 2;
+            const float4 ia = *reinterpret_cast<const float4 *>(&xsI[st][l][(ty * 8) ^ sw]);
+            const float4 ib = *reinterpret_cast<const float4 *>(&xsI[st][l][(ty * 8 + 4) ^ sw]);
+            const ulonglong2 ja = *reinterpret_cast<const ulonglong2 *>(&xsJ[st][l][(tx * 8) ^ sw]);
+            const ulonglong2 jb = *reinterpret_cast<const ulonglong2 *>(&xsJ[st][l][(tx * 8 + 4) ^ sw]);
+            const float xi[8] = {ia.x, ia.y, ia.z, ia.w, ib.x, ib.y, ib.z, ib.w};
+            const uint64_t xj[4] = {ja.x, ja.y, jb.x, jb.y};
+#pragma unroll
+            for (int p = 0; p < 8; ++p) {
+                const uint64_t xx = tc::pk2(xi[p], xi[p]);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const uint64_t D = tc::sub2(xx, xj[c]);
+                    acc[p][c] = tc::fma2(D, D, acc[p][c]);
+                }
+            }
+        }
+        __syncthreads();
+    }
     float d2[8][8];
 #pragma unroll
     for (int p = 0; p < 8; ++p)
 #pragma unroll
-        for (int q = 0; q < 8; ++q) d2[p][q] = 0.f;
-    for (int l0 = 0; l0 < a.n; l0 += WLC) {
-        __syncthreads();
-        for (int idx = tid; idx < T * WLC; idx += 256) {
-            const int r = idx / WLC, l = idx % WLC, gl = l0 + l;
-            xsI[l][r] = (i0 + r < a.N && gl < a.n) ? a.X[(size_t)(i0 + r) * a.n + gl] : 0.f;
-            xsJ[l][r] = (j0 + r < a.N && gl < a.n) ? a.X[(size_t)(j0 + r) * a.n + gl] : 0.f;
+        for (int c = 0; c < 4; ++c) {
+            const float2 t = tc::upk2(acc[p][c]);
+            d2[p][2 * c] = t.x;
+            d2[p][2 * c + 1] = t.y;
         }
-        __syncthreads();
-        const int lc = min(WLC, a.n - l0);
-        for (int l = 0; l < lc; ++l) {
-            const float4 i4a = *reinterpret_cast<const float4 *>(&xsI[l][ty * 8]);
-            const float4 i4b = *reinterpret_cast<const float4 *>(&xsI[l][ty * 8 + 4]);
-            const float4 j4a = *reinterpret_cast<const float4 *>(&xsJ[l][tx * 8]);
-            const float4 j4b = *reinterpret_cast<const float4 *>(&xsJ[l][tx * 8 + 4]);
-            const float xi[8] = {i4a.x, i4a.y, i4a.z, i4a.w, i4b.x, i4b.y, i4b.z, i4b.w};
-            const float xj[8] = {j4a.x, j4a.y, j4a.z, j4a.w, j4b.x, j4b.y, j4b.z, j4b.w};
+    float nuj[8];
 #pragma unroll
-            for (int p = 0; p < 8; ++p)
-#pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    const float D = xi[p] - xj[q];
-                    d2[p][q] = fmaf(D, D, d2[p][q]);
-                }
-        }
-    }
+    for (int q = 0; q < 8; ++q) nuj[q] = __ldg(a.nu + j0 + tx * 8 + q);  // Npad entries
     const bool epson = a.eps2_hi > 0.f;
     int nnear = 0, nexcl = 0;
     unsigned long long near_bits = 0ull;  // bit p*8+q marks a near pair
@@ -199,6 +230,7 @@ __global__ void __launch_bounds__(256) wprep_kernel(WPrepArgs a)
 #pragma unroll
     for (int p = 0; p < 8; ++p) {
         const int i = i0 + ty * 8 + p;
+        const float nui = __ldg(a.nu + i);
         float out[8];
         __nv_bfloat16 hout[8];
 #pragma unroll
@@ -213,9 +245,10 @@ __global__ void __launch_bounds__(256) wprep_kernel(WPrepArgs a)
                 else if ((epson && dd < a.eps2_hi) || dd < 1e-30f)
                     cls = excluded_fp64(a.X, a.n, i, j, a.eps2) ? 0 : 1;
                 else {
-                    const float inv = 1.0f / dd;
-                    const float id = 1.0f / sqrtf(dd);
-                    const float beta = a.beta_coef * (a.nu[i] + a.nu[j]) * id;
+                    const float inv = __frcp_rn(dd);
+                    // the hardware estimate is within 2^-22 of 1/d: far
+                    // inside the margin between the cap and the pass's bound
+                    const float beta = a.beta_coef * (nui + nuj[q]) * rsqrtf(dd);
                     // near: the bound exceeds the cap
                     if (beta > a.b_cap) cls = 1;
                     else { cls = 2; wv = inv; hv = __float2bfloat16_rn(inv); }
@@ -1730,6 +1763,7 @@ sap_status restructured_prepare(sap_handle h)
         r.Npad = (N + T - 1) / T * T;
         r.NP = (n + 63) / 64 * 64;
         RCK(cudaMalloc(&r.center, n * sizeof(float)));
+        RCK(cudaMalloc(&r.colpart, colmean_scratch(N, n) * sizeof(double)));
         RCK(cudaMalloc(&r.nu, r.Npad * sizeof(float)));
         RCK(cudaMalloc(&r.Xhi, (size_t)r.Npad * r.NP * 2));
         RCK(cudaMalloc(&r.Xlo, (size_t)r.Npad * r.NP * 2));
@@ -1758,8 +1792,7 @@ sap_status restructured_prepare(sap_handle h)
         RCK(configure_pass_kernels());
     }
     const int sms = handle_sms(h);
-    colmean_kernel<<<(n + 127) / 128, 128, 0, s>>>(X, N, n, r.center);
-    RCK(cudaGetLastError());
+    RCK(launch_colmean(X, N, n, r.colpart, r.center, s));
     RCK(cudaMemsetAsync(r.counters, 0, 8 * sizeof(unsigned int), s));
     absmax_kernel<<<4 * sms, 256, 0, s>>>(X, (size_t)N * n, n, r.center, r.counters);
     RCK(cudaGetLastError());
@@ -2210,7 +2243,7 @@ int restructured_kernels_per_iteration(sap_handle h)
 void restructured_free(sap_handle h)
 {
     RestrState &r = restr_state(h);
-    dfree(r.Xhi); dfree(r.Xlo); dfree(r.center); dfree(r.nu); dfree(r.w); dfree(r.wtiles);
+    dfree(r.Xhi); dfree(r.Xlo); dfree(r.center); dfree(r.colpart); dfree(r.nu); dfree(r.w); dfree(r.wtiles);
     dfree(r.near); dfree(r.counters); dfree(r.Uhi); dfree(r.Ulo); dfree(r.Y); dfree(r.Yd); dfree(r.Ypart);
     dfree(r.near_w); dfree(r.xn); dfree(r.Ydh); dfree(r.Ydl); dfree(r.wb);
 }

@@ -16,6 +16,7 @@ struct RestrState {
     int NP = 0;           // n rounded up to the GEMM k-block (64)
     float xscale = 1.f;   // power of two applied to (x - mean) before splitting
     float *center = nullptr;  // column means (n), FP32
+    double *colpart = nullptr; // partial column sums of the means
     float *nu = nullptr;  // ||fl(x_i - mean)||, rounded up (Npad)
     // inverse squared lengths, tile-major upper triangle (kTile x kTile tiles);
     // NaN marks a pair the pass skips (invalid, excluded, or near)
