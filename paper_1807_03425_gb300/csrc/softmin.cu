@@ -31,6 +31,7 @@
 #include "restructured.cuh"
 #include "tc_ptx.cuh"
 
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -38,6 +39,8 @@
 #include <cmath>
 #include <cstring>
 #include <vector>
+
+namespace cg = cooperative_groups;
 
 namespace sap {
 namespace {
@@ -829,126 +832,208 @@ struct SoftStepArgs {
     SoftDev *dev;
 };
 
-// One block: G_R = G - U (U^T G) (projection onto the tangent space of the
-// Grassmannian at U), V = U + eta G_R / ||G_R||_F, U <- Q factor of V (two
-// Cholesky-QR passes in FP64; positive diagonal of R, as a Householder QR
-// with signs fixed), and the FP32 / 16-bit copies the other kernels read.
-template <int K>
-__global__ void __launch_bounds__(256) soft_step_kernel(SoftStepArgs a)
+// G_R = G - U (U^T G) (projection onto the tangent space of the Grassmannian
+// at U), V = U + eta G_R / ||G_R||_F, U <- Q factor of V (Cholesky QR in FP64
+// with a second pass; positive diagonal of R, as a Householder QR with signs
+// fixed), and the FP32 / 16-bit copies the other kernels read.
+//
+// Bound by FP64 latency and rate (1/64 of FP32): in one block, with the
+// factorisation in one thread, it took 112 us at n = 150, k = 8.  A cluster
+// shares the rows; every sum over rows (U^T G, ||G_R||^2, V^T V) is formed
+// per block, exchanged through distributed shared memory and added in block
+// order everywhere, so all blocks go on with the same bits.  The
+// factorisation is warp-wide, the triangular solve one row per thread.  The
+// second pass finds |V^T V - I| at rounding level, where (I + R)^-1 = I -
+// triu(E) with halved diagonal: an FP32 correction, unless the first pass
+// left more than 1e-9 (then the factorisation is repeated).
+constexpr int kStepThreads = 256;
+constexpr int kStepClusterMax = 8;
+
+__host__ inline int step_blocks(int n)
 {
+    int c = 1;
+    while (c < kStepClusterMax && c * 64 < n) c <<= 1;
+    return c;
+}
+__host__ __device__ inline int step_rows(int n, int blocks) { return (n + blocks - 1) / blocks; }
+__host__ inline size_t step_smem(int K, int n) { return (size_t)2 * step_rows(n, step_blocks(n)) * (K + 1) * 8; }
+
+template <int K>
+__global__ void __launch_bounds__(kStepThreads) soft_step_kernel(SoftStepArgs a)
+{
+    constexpr int KS = K + 1, E = K * (K + 1) / 2;
     extern __shared__ double sd[];
-    double *sU = sd, *sV = sd + (size_t)K * a.n;
-    __shared__ double sA[K][K], sR[K][K], sRi[K][K];
-    __shared__ double red[8];
+    __shared__ double pA[K * K], pN, pG[2][E];            // this block's sums, read by the cluster
+    __shared__ double sA[K * K], sH[K][K], sRinv[K], slice[kStepThreads], red[kStepThreads / 32];
+    __shared__ float sS[K][K];
+    cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank(), C = (int)cluster.num_blocks();
     const int n = a.n, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    for (int idx = tid; idx < K * n; idx += blockDim.x) {
-        sU[idx] = a.U64[idx];
-        sV[idx] = a.G[idx];
+    const int R = step_rows(n, C), l0 = rank * R, nr = max(0, min(R, n - l0));
+    double *sU = sd, *sV = sd + (size_t)R * KS;           // rows x KS
+    for (int idx = tid; idx < K * nr; idx += kStepThreads) {
+        const int m = idx / nr, r = idx % nr;
+        sU[r * KS + m] = a.U64[(size_t)m * n + l0 + r];
+        sV[r * KS + m] = a.G[(size_t)m * n + l0 + r];
     }
     __syncthreads();
-    // A = U^T G (A[c][m] = <u_c, g_m>)
-    for (int d = warp; d < K * K; d += 8) {
-        const int c = d / K, m = d % K;
+    // sums over this block's rows of x[r][p] y[r][q] for M entries, the rows
+    // dealt to slices of the threads
+    auto row_sums = [&](const double *x, const double *y, int M, auto pq, double *out) {
+        const int sl = min(16, kStepThreads / M), s = tid / M, e = tid % M;
+        double acc = 0.0;
+        if (s < sl) {
+            const int2 v = pq(e);
+            for (int r = s; r < nr; r += sl) acc = fma(x[r * KS + v.x], y[r * KS + v.y], acc);
+        }
+        slice[tid] = acc;
+        __syncthreads();
+        if (tid < M) {
+            for (int q = 1; q < sl; ++q) acc += slice[q * M + tid];
+            out[tid] = acc;
+        }
+    };
+    // A = U^T G (A[c K + m] = <u_c, g_m>)
+    row_sums(sU, sV, K * K, [](int e) { return make_int2(e / K, e % K); }, pA);
+    cluster.sync();
+    if (tid < K * K) {
         double s = 0.0;
-        for (int l = lane; l < n; l += 32) s = fma(sU[c * n + l], sV[m * n + l], s);
-        s = warp_sum(s);
-        if (lane == 0) sA[c][m] = s;
+        for (int q = 0; q < C; ++q) s += *cluster.map_shared_rank(pA + tid, q);
+        sA[tid] = s;
     }
     __syncthreads();
     double nr2 = 0.0;
-    for (int idx = tid; idx < K * n; idx += blockDim.x) {
-        const int m = idx / n, l = idx % n;
-        double g = sV[idx];
+    for (int idx = tid; idx < K * nr; idx += kStepThreads) {
+        const int m = idx % K, r = idx / K;
+        double g = sV[r * KS + m];
 #pragma unroll
-        for (int c = 0; c < K; ++c) g = fma(-sU[c * n + l], sA[c][m], g);
-        sV[idx] = g;
+        for (int c = 0; c < K; ++c) g = fma(-sU[r * KS + c], sA[c * K + m], g);
+        sV[r * KS + m] = g;
         nr2 = fma(g, g, nr2);
     }
     nr2 = warp_sum(nr2);
     if (lane == 0) red[warp] = nr2;
     __syncthreads();
-    nr2 = 0.0;
-    for (int w = 0; w < 8; ++w) nr2 += red[w];
-    const double gn = sqrt(nr2);
     if (tid == 0) {
+        double s = 0.0;
+        for (int q = 0; q < kStepThreads / 32; ++q) s += red[q];
+        pN = s;
+    }
+    cluster.sync();
+    nr2 = 0.0;
+    for (int q = 0; q < C; ++q) nr2 += *cluster.map_shared_rank(&pN, q);
+    const double gn = sqrt(nr2);
+    if (tid == 0 && rank == 0) {
         a.dev->gnorm = gn;
         a.dev->step += 1;
     }
-    if (!(gn > 0.0)) return;  // stationary: U unchanged
+    if (!(gn > 0.0)) {  // stationary: U unchanged
+        cluster.sync();
+        return;
+    }
     const double f = a.eta / gn;
-    for (int idx = tid; idx < K * n; idx += blockDim.x) sV[idx] = fma(f, sV[idx], sU[idx]);
+    for (int idx = tid; idx < K * nr; idx += kStepThreads) {
+        const int m = idx % K, r = idx / K;
+        sV[r * KS + m] = fma(f, sV[r * KS + m], sU[r * KS + m]);
+    }
     __syncthreads();
     for (int pass = 0; pass < 2; ++pass) {
-        for (int d = warp; d < K * K; d += 8) {
-            const int c = d / K, m = d % K;
-            if (m < c) continue;
+        // H = V^T V (upper triangle)
+        auto pq = [](int e) {
+            int p = 0;
+            while (e >= K - p) { e -= K - p; ++p; }
+            return make_int2(p, p + e);
+        };
+        row_sums(sV, sV, E, pq, pG[pass]);
+        cluster.sync();
+        if (tid < E) {
             double s = 0.0;
-            for (int l = lane; l < n; l += 32) s = fma(sV[c * n + l], sV[m * n + l], s);
-            s = warp_sum(s);
-            if (lane == 0) sA[c][m] = s;
+            for (int q = 0; q < C; ++q) s += *cluster.map_shared_rank(pG[pass] + tid, q);
+            const int2 v = pq(tid);
+            sH[v.x][v.y] = s;
         }
         __syncthreads();
-        if (tid == 0) {
-            // H = R^T R, R upper triangular with positive diagonal
-            for (int c = 0; c < K; ++c) {
-                double dgn = sA[c][c];
-                for (int q = 0; q < c; ++q) dgn -= sR[q][c] * sR[q][c];
-                const double rc = sqrt(dgn > 0.0 ? dgn : 0.0);
-                sR[c][c] = rc;
-                for (int m = c + 1; m < K; ++m) {
-                    double v = sA[c][m];
-                    for (int q = 0; q < c; ++q) v -= sR[q][c] * sR[q][m];
-                    sR[c][m] = rc > 0.0 ? v / rc : 0.0;
-                }
-                for (int m = 0; m < c; ++m) sR[c][m] = 0.0;
+        if (pass == 1) {
+            bool tiny = true;
+            if (tid < E) {
+                const int2 v = pq(tid);
+                const double e = sH[v.x][v.y] - (v.x == v.y ? 1.0 : 0.0);
+                tiny = fabs(e) <= 1e-9;
+                sS[v.x][v.y] = (float)(v.x == v.y ? -0.5 * e : -e);
             }
-            // Ri = R^-1 (upper), column by column
-            for (int m = 0; m < K; ++m) {
-                for (int c = K - 1; c >= 0; --c) {
-                    double v = (c == m) ? 1.0 : 0.0;
-                    for (int q = c + 1; q < K; ++q) v -= sR[c][q] * sRi[q][m];
-                    sRi[c][m] = (c <= m && sR[c][c] > 0.0) ? v / sR[c][c] : 0.0;
+            if (__syncthreads_and(tiny ? 1 : 0)) {
+                for (int r = tid; r < nr; r += kStepThreads) {
+                    float x[K];
+#pragma unroll
+                    for (int c = 0; c < K; ++c) x[c] = (float)sV[r * KS + c];
+#pragma unroll
+                    for (int m = 0; m < K; ++m) {
+                        float s = 0.f;
+#pragma unroll
+                        for (int c = 0; c < K; ++c)
+                            if (c <= m) s = fmaf(x[c], sS[c][m], s);
+                        sV[r * KS + m] += (double)s;
+                    }
                 }
+                __syncthreads();
+                break;
+            }
+        }
+        if (warp == 0) {
+            // H = R^T R, R upper triangular with positive diagonal, row by
+            // row; lanes over the entries still to be reduced
+            for (int j = 0; j < K; ++j) {
+                const double h = sH[j][j];
+                const double ri = h > 0.0 ? rsqrt(h) : 0.0;
+                __syncwarp();
+                if (lane == 0) sRinv[j] = ri;
+                if (lane >= j && lane < K) sH[j][lane] *= ri;
+                __syncwarp();
+                for (int e = lane; e < K * K; e += 32) {
+                    const int p = e / K, q = e % K;
+                    if (p > j && q >= p) sH[p][q] = fma(-sH[j][p], sH[j][q], sH[p][q]);
+                }
+                __syncwarp();
             }
         }
         __syncthreads();
-        for (int l = tid; l < n; l += blockDim.x) {
-            double row[K];
-#pragma unroll
-            for (int c = 0; c < K; ++c) row[c] = sV[c * n + l];
+        for (int r = tid; r < nr; r += kStepThreads) {  // row <- row R^-1
+            double x[K];
 #pragma unroll
             for (int m = 0; m < K; ++m) {
-                double s = 0.0;
+                double s = sV[r * KS + m];
 #pragma unroll
                 for (int c = 0; c < K; ++c)
-                    if (c <= m) s = fma(row[c], sRi[c][m], s);
-                sV[m * n + l] = s;
+                    if (c < m) s = fma(-x[c], sH[c][m], s);
+                x[m] = s * sRinv[m];
             }
+#pragma unroll
+            for (int m = 0; m < K; ++m) sV[r * KS + m] = x[m];
         }
         __syncthreads();
     }
-    for (int l = tid; l < n; l += blockDim.x)
-#pragma unroll
-        for (int m = 0; m < K; ++m) {
-            const double s = sV[m * n + l];
-            a.U64[(size_t)m * n + l] = s;
-            const float sf = (float)s;
-            a.U32[(size_t)l * a.KP + m] = sf;
-            a.U32lo[(size_t)l * a.KP + m] = (float)(s - (double)sf);
-            if (a.Uhi) {
-                const size_t idx = (size_t)m * a.NP + l;
-                if (a.split_bf16) {
-                    const __nv_bfloat16 h = __float2bfloat16_rn(sf);
-                    static_cast<__nv_bfloat16 *>(a.Uhi)[idx] = h;
-                    static_cast<__nv_bfloat16 *>(a.Ulo)[idx] =
-                        __float2bfloat16_rn((sf - __bfloat162float(h)) * a.split_scale);
-                } else {
-                    const __half h = __float2half_rn(sf);
-                    static_cast<__half *>(a.Uhi)[idx] = h;
-                    static_cast<__half *>(a.Ulo)[idx] = __float2half_rn((sf - __half2float(h)) * a.split_scale);
-                }
+    for (int idx = tid; idx < K * nr; idx += kStepThreads) {
+        const int m = idx / nr, r = idx % nr, l = l0 + r;
+        const double s = sV[r * KS + m];
+        a.U64[(size_t)m * n + l] = s;
+        const float sf = (float)s;
+        a.U32[(size_t)l * a.KP + m] = sf;
+        a.U32lo[(size_t)l * a.KP + m] = (float)(s - (double)sf);
+        if (a.Uhi) {
+            const size_t o = (size_t)m * a.NP + l;
+            if (a.split_bf16) {
+                const __nv_bfloat16 h = __float2bfloat16_rn(sf);
+                static_cast<__nv_bfloat16 *>(a.Uhi)[o] = h;
+                static_cast<__nv_bfloat16 *>(a.Ulo)[o] =
+                    __float2bfloat16_rn((sf - __bfloat162float(h)) * a.split_scale);
+            } else {
+                const __half h = __float2half_rn(sf);
+                static_cast<__half *>(a.Uhi)[o] = h;
+                static_cast<__half *>(a.Ulo)[o] = __float2half_rn((sf - __half2float(h)) * a.split_scale);
             }
         }
+    }
+    cluster.sync();  // no block leaves while another reads its sums
 }
 
 // ------------------------------------------------------------ host side ---
@@ -1000,9 +1085,6 @@ struct SoftKernels {
             e = cudaFuncSetAttribute(soft_near_kernel<K, 16, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      kNearWarps * kSoftMaxN * K * 4);
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(soft_step_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     2 * K * kSoftMaxN * 8);
-        if (e == cudaSuccess)
             e = cudaFuncSetAttribute(ydf_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      2 * K * kSoftMaxN * 4);
         if (e == cudaSuccess)
@@ -1048,8 +1130,20 @@ struct SoftKernels {
     }
     static cudaError_t step(const SoftStepArgs &a, cudaStream_t s)
     {
-        soft_step_kernel<K><<<1, 256, 2 * K * a.n * 8, s>>>(a);
-        return cudaGetLastError();
+        const int C = step_blocks(a.n);
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(C);
+        cfg.blockDim = dim3(kStepThreads);
+        cfg.dynamicSmemBytes = step_smem(K, a.n);
+        cfg.stream = s;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = C;
+        at[0].val.clusterDim.y = 1;
+        at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        return cudaLaunchKernelEx(&cfg, soft_step_kernel<K>, a);
     }
 };
 
