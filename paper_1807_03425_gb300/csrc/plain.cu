@@ -6,7 +6,13 @@
 // j in block J, I <= J; diagonal blocks keep i < j).  X rows of both blocks
 // are staged in shared memory in chunks of 32 coordinates, transposed so a
 // thread reads its 4 i's and 4 j's with one 16-byte load each; U's chunk is
-// broadcast from shared memory.  Each thread accumulates, for its 4 x 4 pairs,
+// broadcast from shared memory as {u, u} pairs.  The next chunk is copied
+// asynchronously while one is evaluated; chunk coordinate l of point r sits at
+// [l][r ^ 4 (l % 8)] and a warp copies 8 coordinates (a 32-byte sector) of 4
+// points, so neither side meets bank conflicts.  Bound by FP32 issue ((k + 2)
+// n operations per pair): the arithmetic is packed FP32 pairs (two columns
+// j), half the instructions with the same roundings in the same order.
+// Each thread accumulates, for its 4 x 4 pairs,
 //     d^2 = sum_l (x_il - x_jl)^2  and  z_c = sum_l u_lc (x_il - x_jl)
 // with explicit FP32 differences and FMA chains, then r~ = sqrt(|z|^2 / d^2).
 // Error model (u = 2^-24, gamma_m = m u/(1 - m u)):
@@ -17,76 +23,108 @@
 // (d == 0, or d < eps of Sec. VII) is too close to call in FP32 are emitted
 // for the FP64 tier to decide.
 #include "sap_internal.cuh"
+#include "tc_ptx.cuh"
 
 namespace sap {
 namespace {
 
 constexpr int PB = 64;   // points per block edge
 constexpr int LC = 32;   // coordinates per shared-memory chunk
-constexpr int PAD = 4;
 
 template <int K>
 __global__ void __launch_bounds__(256) plain_f32_kernel(PlainArgsF32 a)
 {
-    __shared__ __align__(16) float xsI[LC][PB + PAD];
-    __shared__ __align__(16) float xsJ[LC][PB + PAD];
-    __shared__ float us[LC][K];
+    __shared__ __align__(16) float xsI[2][LC][PB];
+    __shared__ __align__(16) float xsJ[2][LC][PB];
+    __shared__ __align__(16) float us[2][LC][2 * K];
     __shared__ float red[32];
     __shared__ int scan[33];
     __shared__ int base_sh;
 
     const int tid = threadIdx.x;
     const int tx = tid & 15, ty = tid >> 4;
+    // copies: chunk coordinate sl of the points sr, sr + 8, ...
+    const int sl = ((tid >> 2) & 7) + 8 * ((tid >> 5) & 3), sr = (tid & 3) + 4 * (tid >> 7);
 
     for (int t = blockIdx.x; t < a.ntiles; t += gridDim.x) {
         const int2 IJ = a.tiles[t];
         const int i0 = IJ.x * PB, j0 = IJ.y * PB;
-        float d2[4][4];
-        float z[4][4][K];
+        uint64_t d2p[4][2];     // row p, columns 2 c and 2 c + 1
+        uint64_t zp[4][2][K];
 #pragma unroll
         for (int p = 0; p < 4; ++p)
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                d2[p][q] = 0.f;
+            for (int c = 0; c < 2; ++c) {
+                d2p[p][c] = 0ull;
 #pragma unroll
-                for (int c = 0; c < K; ++c) z[p][q][c] = 0.f;
+                for (int m = 0; m < K; ++m) zp[p][c][m] = 0ull;
             }
-
-        for (int l0 = 0; l0 < a.n; l0 += LC) {
-            __syncthreads();
-            for (int idx = tid; idx < PB * LC; idx += 256) {
-                const int r = idx / LC, l = idx % LC;
-                const int gl = l0 + l;
-                const int gi = i0 + r, gj = j0 + r;
-                xsI[l][r] = (gi < a.N && gl < a.n) ? a.X[(size_t)gi * a.n + gl] : 0.f;
-                xsJ[l][r] = (gj < a.N && gl < a.n) ? a.X[(size_t)gj * a.n + gl] : 0.f;
+        auto copy = [&](int l0, int st) {
+            const int gl = l0 + sl;
+            const bool inl = gl < a.n;
+#pragma unroll
+            for (int q = 0; q < PB / 8; ++q) {
+                const int r = sr + 8 * q, col = r ^ ((sl & 7) << 2);
+                const bool ini = inl && i0 + r < a.N, inj = inl && j0 + r < a.N;
+                tc::cp_async4(&xsI[st][sl][col], ini ? a.X + (size_t)(i0 + r) * a.n + gl : a.X, ini);
+                tc::cp_async4(&xsJ[st][sl][col], inj ? a.X + (size_t)(j0 + r) * a.n + gl : a.X, inj);
             }
-            for (int idx = tid; idx < LC * K; idx += 256) {
-                const int l = idx / K, c = idx % K;
-                const int gl = l0 + l;
-                us[l][c] = (gl < a.n) ? a.U32[(size_t)gl * a.KP + c] : 0.f;
+            for (int idx = tid; idx < LC * K * 2; idx += 256) {
+                const int l = idx / (2 * K), c = (idx % (2 * K)) >> 1;
+                const bool in = l0 + l < a.n;
+                tc::cp_async4(&us[st][l][idx % (2 * K)], in ? a.U32 + (size_t)(l0 + l) * a.KP + c : a.U32, in);
+            }
+            tc::cp_async_commit();
+        };
+        __syncthreads();  // the previous tile's last chunk has been read
+        copy(0, 0);
+        for (int l0 = 0, st = 0; l0 < a.n; l0 += LC, st ^= 1) {
+            if (l0 + LC < a.n) {
+                copy(l0 + LC, st ^ 1);
+                tc::cp_async_wait<1>();
+            } else {
+                tc::cp_async_wait<0>();
             }
             __syncthreads();
             const int lc = min(LC, a.n - l0);
+#pragma unroll 4
             for (int l = 0; l < lc; ++l) {
-                const float4 xi = *reinterpret_cast<const float4 *>(&xsI[l][ty * 4]);
-                const float4 xj = *reinterpret_cast<const float4 *>(&xsJ[l][tx * 4]);
+                const int sw = (l & 7) << 2;
+                const float4 xi = *reinterpret_cast<const float4 *>(&xsI[st][l][(ty * 4) ^ sw]);
+                const ulonglong2 xj = *reinterpret_cast<const ulonglong2 *>(&xsJ[st][l][(tx * 4) ^ sw]);
                 const float ai[4] = {xi.x, xi.y, xi.z, xi.w};
-                const float bj[4] = {xj.x, xj.y, xj.z, xj.w};
-                float u[K];
+                uint64_t uu[K];
 #pragma unroll
-                for (int c = 0; c < K; ++c) u[c] = us[l][c];
+                for (int m = 0; m < K; ++m) uu[m] = *reinterpret_cast<const uint64_t *>(&us[st][l][2 * m]);
 #pragma unroll
-                for (int p = 0; p < 4; ++p)
+                for (int p = 0; p < 4; ++p) {
+                    const uint64_t xx = tc::pk2(ai[p], ai[p]);
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const float D = ai[p] - bj[q];
-                        d2[p][q] = fmaf(D, D, d2[p][q]);
+                    for (int c = 0; c < 2; ++c) {
+                        const uint64_t D = tc::sub2(xx, c ? xj.y : xj.x);
+                        d2p[p][c] = tc::fma2(D, D, d2p[p][c]);
 #pragma unroll
-                        for (int c = 0; c < K; ++c) z[p][q][c] = fmaf(u[c], D, z[p][q][c]);
+                        for (int m = 0; m < K; ++m) zp[p][c][m] = tc::fma2(uu[m], D, zp[p][c][m]);
                     }
+                }
             }
+            __syncthreads();
         }
+        float d2[4][4], z[4][4][K];
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                const float2 v = tc::upk2(d2p[p][c]);
+                d2[p][2 * c] = v.x;
+                d2[p][2 * c + 1] = v.y;
+#pragma unroll
+                for (int m = 0; m < K; ++m) {
+                    const float2 y = tc::upk2(zp[p][c][m]);
+                    z[p][2 * c][m] = y.x;
+                    z[p][2 * c + 1][m] = y.y;
+                }
+            }
 
         // classify and evaluate the 16 pairs: 0 excluded, 1 normal, 2 decide in FP64
         float rt[4][4];

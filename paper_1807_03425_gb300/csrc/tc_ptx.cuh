@@ -80,6 +80,21 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t by
                  : "memory");
 }
 
+// Asynchronous 4-byte copy global -> shared by the calling thread (zero when
+// `in` is false: nothing is read), its groups and the wait for all but the
+// latest N of them.
+__device__ __forceinline__ void cp_async4(float *dst, const float *src, bool in)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(in ? 4 : 0)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait()
+{
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
 // Packed FP32 pairs (two IEEE round-to-nearest operations per instruction).
 __device__ __forceinline__ uint64_t pk2(float x, float y)
 {
