@@ -21,6 +21,8 @@
 #include "tc_ptx.cuh"
 #include "gemm_tc.cuh"
 
+#include <cuda_fp16.h>
+
 #include <algorithm>
 
 namespace sap {
@@ -101,6 +103,46 @@ __device__ float product_seeds(const GemmArgs &a, int q0, int step, int lane)
         if (dd > 1e-30f) best = fminf(best, cert_upper(sqrtf(zz / dd), cert));
     }
     return best;
+}
+
+// Four components of one row as operands of the all-pairs filter (OpGroup);
+// s accumulates the row's |y|^2 over the basis's groups.
+__device__ __forceinline__ void op_group(unsigned char *images, const OpGroup &og, int r, const float (&y)[4],
+                                         float scale, float &s)
+{
+    if (og.g < 0) return;
+    if (og.g == 0) s = 0.f;
+    unsigned char *base = images + og.off + (r >> 3) * 128 + (r & 7) * 16;
+    auto put = [&](uint32_t img, int half, __half2 x, __half2 z) {
+        uint2 v;
+        v.x = *reinterpret_cast<uint32_t *>(&x);
+        v.y = *reinterpret_cast<uint32_t *>(&z);
+        *reinterpret_cast<uint2 *>(base + img + (half >> 1) * 2048 + (half & 1) * 8) = v;
+    };
+    float h[4], l[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const float v = y[q] * scale;
+        h[q] = __half2float(__float2half_rn(v));
+        l[q] = v - h[q];
+        s = fmaf(v, v, s);
+    }
+    const __half2 h0 = __floats2half2_rn(h[0], h[1]), h1 = __floats2half2_rn(h[2], h[3]);
+    const __half2 l0 = __floats2half2_rn(l[0], l[1]), l1 = __floats2half2_rn(l[2], l[3]);
+    const __half2 m2 = __floats2half2_rn(-2.f, -2.f);
+    put(0, 3 * og.g, h0, h1);
+    put(0, 3 * og.g + 1, h0, h1);
+    put(0, 3 * og.g + 2, l0, l1);
+    put(og.img, 3 * og.g, __hmul2(h0, m2), __hmul2(h1, m2));
+    put(og.img, 3 * og.g + 1, __hmul2(l0, m2), __hmul2(l1, m2));
+    put(og.img, 3 * og.g + 2, __hmul2(h0, m2), __hmul2(h1, m2));
+    if (og.last) {
+        const float sp = s * og.keep - og.kabs2;
+        const float sh = __half2float(__float2half_rn(sp));
+        const __half2 sv = __floats2half2_rn(sh, sp - sh), one = __floats2half2_rn(1.f, 1.f);
+        put(0, 3 * (og.g + 1), sv, one);
+        put(og.img, 3 * (og.g + 1), one, sv);
+    }
 }
 
 // 128 threads (TMA producer, MMA issuer, four epilogue warps over the TMEM
@@ -215,6 +257,7 @@ __global__ void __launch_bounds__(192, 1) gemm_y_kernel(const __grid_constant__ 
     if (good && warp < 4) {
         const int row = m0 + warp * 32 + lane;
         const uint32_t lane_base = tbase + ((uint32_t)(warp * 32) << 16);
+        float s = 0.f;
         for (int c0 = 0; c0 < a.KY; c0 += 8) {
             float d1[8], d2[8];
             tc::tmem_ld8(lane_base + c0, d1);
@@ -224,15 +267,19 @@ __global__ void __launch_bounds__(192, 1) gemm_y_kernel(const __grid_constant__ 
                 if (a.ksplit == 1) {
                     // block-major: the KY components of each 128-row block are contiguous
                     float *yb = a.Y + (size_t)(row >> 7) * ((size_t)a.KY * 128) + (row & 127);
-                    float *yd = a.Yd ? a.Yd + (size_t)(row >> 7) * ((size_t)a.KY * 256) + yd_offset(row & 127)
-                                     : nullptr;
 #pragma unroll
-                    for (int q = 0; q < 8; ++q)
-                        if (c0 + q < a.KY) {
-                            const float y = fmaf(d2[q], a.lo_scale, d1[q]) * a.out_scale;
-                            yb[(size_t)(c0 + q) * 128] = y;
-                            if (yd) *reinterpret_cast<float2 *>(yd + (size_t)(c0 + q) * 256) = make_float2(y, y);
+                    for (int g = 0; g < 2; ++g) {
+                        if (c0 + 4 * g >= a.KY) break;
+                        float y[4];
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            y[q] = fmaf(d2[4 * g + q], a.lo_scale, d1[4 * g + q]) * a.out_scale;
+                            yb[(size_t)(c0 + 4 * g + q) * 128] = y[q];
                         }
+                        if (a.ops)
+                            op_group(a.ops + (size_t)(row >> 7) * a.ops_stride, a.groups[(c0 >> 2) + g], row & 127, y,
+                                     a.ops_scale, s);
+                    }
                 } else {
                     float *dst = a.Ypart + (size_t)blockIdx.y * a.KY * a.Npad;
 #pragma unroll
@@ -249,21 +296,30 @@ __global__ void __launch_bounds__(192, 1) gemm_y_kernel(const __grid_constant__ 
     if (warp == 0) tc::tmem_dealloc(tbase, ncols);
 }
 
-// Y = (sum of the K slices, in slice order) * out_scale; the slices are
-// component-major (c * Npad + row), Y (and Yd) block-major like the
-// product's output.
-__global__ void ksum_kernel(const float *Ypart, int ksplit, int KY, int Npad, float out_scale, float *Y, float *Yd)
+// Y = (sum of the K slices, in slice order) * out_scale, block-major like the
+// product's output, and the filter's operands; the slices are
+// component-major (c * Npad + row).  One block per 128 rows and basis.
+__global__ void __launch_bounds__(128) ksum_kernel(const __grid_constant__ GemmArgs a)
 {
-    const size_t count = (size_t)KY * Npad;
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < count; e += (size_t)gridDim.x * blockDim.x) {
-        float s = Ypart[e];
-        for (int q = 1; q < ksplit; ++q) s += Ypart[(size_t)q * count + e];
-        const size_t c = e / Npad, row = e % Npad;
-        const float y = s * out_scale;
-        Y[(row >> 7) * ((size_t)KY * 128) + c * 128 + (row & 127)] = y;
-        if (Yd)
-            *reinterpret_cast<float2 *>(Yd + (row >> 7) * ((size_t)KY * 256) + c * 256 + yd_offset((int)(row & 127))) =
-                make_float2(y, y);
+    const int row = blockIdx.x * 128 + threadIdx.x;
+    const size_t count = (size_t)a.KY * a.Npad;
+    float *yb = a.Y + (size_t)blockIdx.x * ((size_t)a.KY * 128) + threadIdx.x;
+    const int g0 = a.nbases > 0 ? a.base_group[blockIdx.y] : 0;
+    const int g1 = a.nbases > 0 ? a.base_group[blockIdx.y + 1] : a.KY / 4;
+    float s = 0.f;
+    for (int g = g0; g < g1; ++g) {
+        float y[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float *src = a.Ypart + (size_t)(4 * g + q) * a.Npad + row;
+            float v = src[0];
+#pragma unroll 4
+            for (int p = 1; p < a.ksplit; ++p) v += src[(size_t)p * count];
+            y[q] = v * a.out_scale;
+            yb[(size_t)(4 * g + q) * 128] = y[q];
+        }
+        if (a.ops)
+            op_group(a.ops + (size_t)blockIdx.x * a.ops_stride, a.groups[g], threadIdx.x, y, a.ops_scale, s);
     }
 }
 
@@ -297,9 +353,7 @@ cudaError_t launch_gemm_y(const GemmArgs &a, cudaStream_t s)
     cudaError_t e = launch_pdl(a.pdl != 0, gemm_y_kernel, dim3(a.Npad / GM, ksplit), dim3(a.seed_st ? 192 : 128), shm,
                                s, b);
     if (e != cudaSuccess || ksplit == 1) return e;
-    const size_t count = (size_t)a.KY * a.Npad;
-    ksum_kernel<<<(unsigned)std::min<size_t>((count + 255) / 256, 2048), 256, 0, s>>>(a.Ypart, ksplit, a.KY, a.Npad,
-                                                                                    a.out_scale, a.Y, a.Yd);
+    ksum_kernel<<<dim3(a.Npad / GM, std::max(1, a.nbases)), 128, 0, s>>>(b);
     return cudaGetLastError();
 }
 

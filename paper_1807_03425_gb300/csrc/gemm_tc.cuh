@@ -6,14 +6,41 @@
 
 namespace sap {
 
+// Operands of the all-pairs filter.  For a pair, |y_i - y_j|^2 = s_i + s_j -
+// 2 <y_i, y_j> is one contraction of K-axis vectors
+//     A_i = [h_i, h_i, l_i | s_i', 1],   B_j = -2 [h_j, l_j, h_j | ...] resp. [.. | 1, s_j'],
+// with y (scaled by a power of two to |y| <= 64) = h + l in two FP16 terms and
+// s' = (1 - kappa) |y|^2 - kabs / 2 in two FP16 terms: kappa and kabs bound
+// every error of the contraction, so the result is a certified lower bound of
+// |y_i - y_j|^2 (op_bounds).  Four components take three 4-element halves
+// (8 bytes) of the K axis, the norms one.  An image holds 128 rows in the
+// unswizzled K-major core-matrix order of the MMA: [K / 8][row / 8][row % 8][8
+// elements]; a block's A image is followed by its B image.
+struct OpGroup {
+    uint32_t off;      // the basis's A image within a block's images
+    uint32_t img;      // bytes of one image
+    int g;             // group of 4 components within the basis; -1: padding
+    int last;          // the basis's last group: writes the norms
+    float keep, kabs2; // 1 - kappa, kabs / 2
+};
+constexpr int kMaxOpGroups = 64;   // 256 components
+constexpr int kMaxOpBases = 20;
+__host__ __device__ inline int op_ksteps(int k) { return ((3 * ((k + 3) / 4) + 1) * 4 + 15) / 16; }  // K / 16
+__host__ __device__ inline uint32_t op_image_bytes(int k) { return (uint32_t)op_ksteps(k) * 4096u; }
+
 struct GemmArgs {
     CUtensorMap ta_hi, ta_lo;   // X split parts: Npad x NP, 16-bit, box 64 x 128
     CUtensorMap tb_hi, tb_lo;   // U split parts: KPG x NP, 16-bit, box 64 x KPG
     float *Y;                   // FP32, block-major: [Npad/128][KY][128]
-    // optional second copy for the row side of the all-pairs pass: per
-    // block and component 256 floats, row a = 16 r + g at g * 16 + (r / 2) * 4
-    // + (r % 2) * 2, written twice ({y, y} pairs)
-    float *Yd;
+    // optional: the rows of Y as operands of the all-pairs pass's tensor-core
+    // filter (see OpGroup), for `nbases` bases whose components follow one
+    // another in Y; block b's images start at ops + b * ops_stride
+    unsigned char *ops = nullptr;
+    uint32_t ops_stride = 0;
+    int nbases = 0;
+    int base_group[kMaxOpBases + 1];    // first group of 4 components of each basis, and the end
+    OpGroup groups[kMaxOpGroups];
+    float ops_scale = 1.f;              // power of two: |y| * ops_scale <= 64
     int KY;                     // components written (multiple of 4, <= KPG)
     int Npad;                   // rows (multiple of 128)
     int nkb;                    // K blocks of 64

@@ -121,7 +121,8 @@ struct WPrepArgs {
     const float *nu;
     const int2 *wtiles;
     float *w;
-    __nv_bfloat16 *wb;       // BF16 1/d^2 of the stored pairs (NaN elsewhere)
+    __nv_bfloat16 *wb;       // BF16 1/d^2 of the stored pairs over yscale^2 (NaN elsewhere)
+    float wb_scale;          // 1 / yscale^2 (a power of two)
     float eps2_lo, eps2_hi;  // FP32 window around eps^2 (0,0: no threshold)
     double eps2;
     float beta_coef;         // sqrt(k) * eps_Y, rounded up
@@ -251,7 +252,7 @@ __global__ void __launch_bounds__(256, 2) wprep_kernel(WPrepArgs a)
                     const float beta = a.beta_coef * (nui + nuj[q]) * rsqrtf(dd);
                     // near: the bound exceeds the cap
                     if (beta > a.b_cap) cls = 1;
-                    else { cls = 2; wv = inv; hv = __float2bfloat16_rn(inv); }
+                    else { cls = 2; wv = inv; hv = __float2bfloat16_rn(inv * a.wb_scale); }
                 }
                 if (cls == 0) ++nexcl;
                 if (cls == 1) { ++nnear; near_bits |= 1ull << (p * 8 + q); }
@@ -267,7 +268,7 @@ __global__ void __launch_bounds__(256, 2) wprep_kernel(WPrepArgs a)
         hp.y = (unsigned)__bfloat16_as_ushort(hout[2]) | ((unsigned)__bfloat16_as_ushort(hout[3]) << 16);
         hp.z = (unsigned)__bfloat16_as_ushort(hout[4]) | ((unsigned)__bfloat16_as_ushort(hout[5]) << 16);
         hp.w = (unsigned)__bfloat16_as_ushort(hout[6]) | ((unsigned)__bfloat16_as_ushort(hout[7]) << 16);
-        *reinterpret_cast<uint4 *>(ht + (size_t)(ty * 8 + p) * T + tx * 8) = hp;
+        *reinterpret_cast<uint4 *>(ht + ((size_t)tx * T + ty * 8 + p) * 8) = hp;  // column group tx, this row
     }
     int total;
     const int off = block_exclusive_scan(nnear, scan, &total);
@@ -300,12 +301,16 @@ __global__ void __launch_bounds__(256, 2) wprep_kernel(WPrepArgs a)
 constexpr int kPassStagesMax = 5;
 
 struct PassArgs {
-    const uint16_t *wb;  // BF16 1/d^2 tiles (tile-major upper triangle; NaN: skipped)
+    const uint16_t *wb;  // BF16 1/d^2 tiles over yscale^2 (tile-major upper triangle; NaN: skipped)
     const int2 *wtiles;
     int ntiles;
+    const unsigned char *ops;  // this basis's A image in block 0 (gemm_tc.cuh: OpGroup)
+    uint32_t ops_stride;       // bytes between blocks
+    uint32_t img;              // bytes of one image
+    int ksteps;                // MMA steps of 16
+    int stage_y;               // 1: the FP32 Y of both sides is staged beside the tile
+    float w_scale;             // yscale^2: a stored w times this is 1/d^2
     const float *Y;   // this basis's first component in block 0 of the block-major Y
-    const float *Yd;  // the same in the doubled row-side copy (block stride Ykt * 256 floats)
-    int KY;           // components of this basis
     int Ykt;          // components per block of the Y buffer (block stride / 128)
     int Npad;
     const float *nu;  // ||fl(x_i - mean)||, rounded up (Npad)
@@ -316,9 +321,10 @@ struct PassArgs {
     int2 *cand;
     long long cap;
     int pdl;
+    int k = 0;
     // second and third tiers inside the pass (non-null X; k <= 16): the
-    // near pairs (before the tiles) and every emitted pair are evaluated at
-    // once by the warp that holds them, from explicit FP32 differences (the
+    // near pairs that Y cannot rule out and every emitted pair are evaluated
+    // by the warp that holds them, from explicit FP32 differences (the
     // explicit tier's arithmetic and error model, cert32), which tightens
     // the bounds; the survivors wait in the warp's list and, once its tiles
     // are done, those that can still be the argmin under the bound as it is
@@ -331,63 +337,67 @@ struct PassArgs {
     const float *U32 = nullptr;  // n x KP FP32 basis (pad columns zero)
     int KP = 0;
     const double *U64 = nullptr;  // n x k FP64 basis, column-major
-    int k = 0;
     double eps2 = 0.0;            // squared minimum secant length
     const int2 *near = nullptr;
+    const float *near_w = nullptr;  // their 1/d^2 (+inf: too short for FP32)
     int n_near = 0;
     Partial *partials = nullptr;
     Cert cert32;
 };
 
-// One ring stage: the BF16 1/d^2 tile (32 KB), then the row side's point
-// block -- for k <= 8 the k used components of the doubled copy ({y, y}
-// pairs, 1 KB each), else the KY components of Y -- and the column side's
-// (k, else KY, components of Y; one copy each, block-major), then the 128
-// point norms nu of each side.
-// kd: the compute width of a pass class with four columns per thread
-// (k <= 16), which stages kd components per side (the row side from the
-// doubled copy); 0: the other classes, which stage all KY components.
-__host__ __device__ inline uint32_t pass_row_bytes(int kd, int KY) { return kd ? (uint32_t)kd * T * 8 : (uint32_t)T * KY * 4; }
-__host__ __device__ inline uint32_t pass_col_bytes(int kd, int KY) { return kd ? (uint32_t)kd * T * 4 : (uint32_t)T * KY * 4; }
-__host__ __device__ inline uint32_t pass_stage_bytes(int kd, int KY)
+// One ring stage: the BF16 1/d^2 tile (32 KB), the row block's A image and
+// the column block's B image, the k components of both blocks' Y (when
+// staged), then the 128 point norms nu of each side.
+inline uint32_t pass_stage_bytes(int k, bool stage_y)
 {
-    return (uint32_t)T * T * 2 + pass_row_bytes(kd, KY) + pass_col_bytes(kd, KY) + 2u * T * 4;
+    return (uint32_t)T * T * 2 + 2u * op_image_bytes(k) + (stage_y ? 2u * k * T * 4 : 0u) + 2u * T * 4;
 }
-inline int pass_kd(int k) { return k <= 8 ? k : k <= 10 ? 10 : k <= 12 ? 12 : k <= 16 ? 16 : 0; }
 
 // Certified error of one stored pair's ratio from the tensor-core Y:
 // |r~ - r| <= beta (nu_i + nu_j) / d_ij + rho r.  1/d_ij is taken as the
 // square root of the stored BF16 w = 1/d^2 (relative error of w <= 2^-8, so
 // of its root <= 2^-9 + 2^-23 with the FP32 root: inflated by 3 10^-3).  The
 // same product the length preparation compares with b_cap.
+__device__ __forceinline__ float sqrt_up(float x)  // the hardware square root (relative error 2^-22)
+{
+    float y;
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
 __device__ __forceinline__ float pair_bound(float beta, float nui, float nuj, float w)
 {
-    return beta * (nui + nuj) * sqrtf(w) * 1.003f;
+    return beta * (nui + nuj) * sqrt_up(w) * 1.003f;
 }
-
-// Two BF16 values packed in a 32-bit word, widened exactly to FP32 (a BF16
-// value is the upper half of the FP32 value): integer-pipe operations only.
-__device__ __forceinline__ float bf16_lo(uint32_t x) { return __uint_as_float(x << 16); }
-__device__ __forceinline__ float bf16_hi(uint32_t x) { return __uint_as_float(x & 0xffff0000u); }
-__device__ __forceinline__ float bf16_at(const uint16_t *p) { return __uint_as_float((uint32_t)*p << 16); }
 
 // Persistent, warp-specialised pass: one block per SM.  Each block's first
 // `stages` tiles are blockIdx.x + it * gridDim.x (their constant parts are
 // fetched before the previous kernel has finished); the remaining tiles
-// are handed out from a counter, so a block that starts late (its SM still
-// busy with the previous kernels) takes fewer.  A producer warp keeps a ring of
-// `stages` shared-memory buffers filled by 1-D TMA bulk copies (the 32 KB
-// BF16 w tile, for each side the basis's components of the point block and
-// the point norms); 16
-// consumer warps evaluate the tiles.  Full/empty mbarriers hand the buffers
-// over, so the loop has no block-wide barrier.  Each consumer thread owns CPT
-// adjacent columns (j) of rows spaced 16/(4/CPT) apart (32 pairs per tile);
-// K = compute width (k, or k rounded up for large k: Y's pad components are
-// zero).  q = ||y_i - y_j||^2 w is formed with packed FP32 pairs; w is
-// widened from BF16 by integer operations, off the FP32 pipe.  Every warp
-// bounds the minimum from its own pairs (a valid upper bound like any other),
-// tightens the global running bound with a fire-and-forget atomic, and
-// emits its candidates with one atomic per warp when it has any.
+// follow the same stride, or with programmatic launch are handed out from a
+// counter, so a block that starts late (its SM still busy with the previous
+// kernels) takes fewer.  A producer warp keeps a ring of `stages`
+// shared-memory buffers filled by 1-D TMA bulk copies, an MMA warp forms each
+// tile's 128 x 128 products on the tensor cores (accumulator in tensor
+// memory, two buffers), and 16 consumer warps read them back.  mbarriers hand
+// the buffers over, so the loop has no block-wide barrier.
+//
+// Filter.  The contraction of the operand images (gemm_tc.cuh) is a certified
+// lower bound of |y_i - y_j|^2 (in units of yscale), so its product with the
+// stored w bounds r~^2 from below: a pair whose product exceeds the squared
+// threshold cannot be the argmin, and a tile with no pair below it is done
+// after one multiplication and one minimum per pair.  (A stored w is read as
+// the upper half of a 32-bit word whose lower half is its neighbour: exact
+// after a shift for the even columns, at most 2^-7 too large for the odd
+// ones; kFilter widens the threshold by that.)  The rare tile that has one is
+// re-evaluated where it matters from the FP32 rows of Y: r~^2 = |y_i - y_j|^2
+// w, the value every bound below is certified for.
+//
+// What bounds it.  The differences and squares (2 k packed operations per
+// pair of pairs) kept the FP32 pipe busy for 42 us per pass at N = 8192, k = 5
+// and 184 us at N = 19939, k = 10; on the tensor cores they take 150-200
+// cycles per tile, and what is left on the consumers (3 operations per pair)
+// is below the stream of the stored lengths, about 1400 cycles per 32 KB tile
+// and SM (6 TB/s).  Both passes now take 22 us and 82 us: the stream (12 and
+// 70 us), 3 us until the first tile, 2-3 us for the survivors at the end.
 //
 // Bounds.  Every stored pair's error is at most b_p = beta (nu_i + nu_j) /
 // d_ij <= A (= b_cap; pairs above it are on the near list).  The fast path
@@ -396,18 +406,15 @@ __device__ __forceinline__ float bf16_at(const uint16_t *p) { return __uint_as_f
 // pair that passes the uniform test is emitted only if it passes its own:
 // r~_p <= U (1 + rho) + b_p.  Both refinements touch only the rare slow path.
 constexpr int kConsumerWarps = 16;
-constexpr int kPassThreads = (kConsumerWarps + 1) * 32;
+constexpr int kPassThreads = (kConsumerWarps + 2) * 32;
+constexpr int kTmemCols = 256;          // two 128-column accumulators
+constexpr float kFilter = 1.0081f;      // (1 + 2^-7) (1 + 2.8e-4): odd columns' w, FP32 roundings
 
-// A second-tier survivor of the pass waiting for the FP64 tier (r: its FP32
-// explicit ratio, -1 when too short for FP32).
-struct DeferredPair {
-    int i, j;
-    float r;
-};
-constexpr int kDefer = 32;     // deferred survivors per consumer warp
-constexpr int kDrainTile = 6;  // tiles before the first check of the deferred survivors
+// A warp's pending pairs, packed with a lower bound of their ratio (pack_cand).
+constexpr int kPending = 64;
+constexpr int kQueue = 8;      // survivors the whole block evaluates together
 // dynamic shared memory of the pass: the 227 KB a block may hold, less the
-// static part (barriers, tile coordinates, the deferred survivors)
+// static part (barriers, tile coordinates, the pending pairs)
 constexpr int kPassDynSmem = 216 * 1024;
 
 // Explicit FP32 differences of E pairs by one warp (lanes over the
@@ -483,42 +490,57 @@ __device__ __forceinline__ void expl32_eval(const float *X, int n, const float *
     expl32_finish<K, E>(acc, valid, lane, rr, code);
 }
 
-template <int K, int CPT, bool EXPL>
-__global__ void __launch_bounds__(kPassThreads, 1) restr_pass_kernel(PassArgs a)
+// K: compute width of the second tier inside the pass (EXPL); the filter and
+// the FP32 re-evaluation take k at run time.
+template <int K, bool EXPL>
+__global__ void __launch_bounds__(kPassThreads, 1) restr_pass_kernel(const __grid_constant__ PassArgs a)
 {
-    constexpr int SR = 4 / CPT;                  // warps sharing one row
-    constexpr int RSTEP = kConsumerWarps / SR;   // row step of one warp
-    constexpr int RPW = T / RSTEP;               // rows per warp
-    constexpr int NPR = CPT / 2;                 // column pairs per thread
-    static_assert(RPW * CPT == 32, "one bit per pair of a thread in the emission mask");
     // indexed directly (no integer round trip) so reads stay shared-memory loads
     extern __shared__ __align__(128) unsigned char sm[];
-    __shared__ __align__(8) uint64_t full[kPassStagesMax], empty[kPassStagesMax];
+    __shared__ __align__(8) uint64_t full[kPassStagesMax], empty[kPassStagesMax], tfull[2], tempty[2];
     __shared__ int2 sIJ[kPassStagesMax];
+    __shared__ uint32_t tslot;
+    __shared__ unsigned int sub;               // float bits: the block's best upper bound of the minimum
     __shared__ Partial pbest[kConsumerWarps];  // tiers inside: the warps' best pairs
-    __shared__ unsigned int pdone;             // consumer warps finished
-    __shared__ DeferredPair defer[EXPL ? kConsumerWarps : 1][EXPL ? kDefer : 1];
+    __shared__ unsigned long long pending[EXPL ? kConsumerWarps : 1][EXPL ? kPending : 1];
+    __shared__ unsigned long long queue[EXPL ? kQueue : 1];  // the block's survivors
+    __shared__ double entries[EXPL ? kQueue : 1][EXPL ? K + 1 : 1];
+    __shared__ int nqueue;
 
     const int tid = threadIdx.x;
     const int warp = tid >> 5, lane = tid & 31;
-    const int KY = a.KY, S = a.stages;
-    constexpr bool DBL = CPT == 4;  // row side from the doubled copy (K <= 16)
-    const uint32_t wbytes = T * T * 2, ibytes = pass_row_bytes(DBL ? K : 0, KY),
-                   jbytes = pass_col_bytes(DBL ? K : 0, KY), sbytes = wbytes + ibytes + jbytes + 2 * T * 4;
-    // tiles below gridDim.x * S are static (it < S); the rest are dynamic
+    const int S = a.stages, k = a.k;
+    const uint32_t wbytes = T * T * 2, img = a.img, ybytes = a.stage_y ? (uint32_t)k * T * 4 : 0u;
+    const uint32_t o_a = wbytes, o_b = o_a + img, o_yi = o_b + img, o_yj = o_yi + ybytes, o_nu = o_yj + ybytes;
+    const uint32_t sbytes = o_nu + 2 * T * 4;
+    // tiles below gridDim.x * S are static (it < S); the rest may be dynamic
     const int nall = blockIdx.x < (unsigned)a.ntiles ? (a.ntiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
     const int nstatic = nall < S ? nall : S;
     const long long budget = 4000000000ll;
 
     if (tid == 0) {
-        pdone = 0;
+        sub = 0x7f800000u;
+        nqueue = 0;
         for (int s = 0; s < S; ++s) {
             tc::mbar_init(&full[s], 1);
             tc::mbar_init(&empty[s], kConsumerWarps);
         }
+        for (int s = 0; s < 2; ++s) {
+            tc::mbar_init(&tfull[s], 1);
+            tc::mbar_init(&tempty[s], kConsumerWarps);
+        }
         tc::fence_mbar_init();
     }
     __syncthreads();
+    // tensor memory, while the producer issues its first copies
+    uint32_t tbase = 0;
+    if (warp != kConsumerWarps) {
+        if (warp == kConsumerWarps + 1) tc::tmem_alloc(&tslot, kTmemCols);
+        tc::tc_fence_before();
+        asm volatile("bar.sync 1, %0;" ::"n"(kPassThreads - 32) : "memory");
+        tc::tc_fence_after();
+        tbase = tslot;
+    }
 
     if (warp == kConsumerWarps) {
         // ---------------- producer warp ----------------
@@ -526,27 +548,37 @@ __global__ void __launch_bounds__(kPassThreads, 1) restr_pass_kernel(PassArgs a)
             // The stored lengths and point norms are constant: the first
             // stages' copies start before the product of this iteration has
             // finished (programmatic launch); Y follows after the wait.
+            auto constant_part = [&](int s, int t, int2 IJ) {
+                unsigned char *base = sm + (size_t)s * sbytes;
+                tc::mbar_expect_tx(&full[s], sbytes);
+                tc::bulk_g2s(base, a.wb + (size_t)t * T * T, wbytes, &full[s]);
+                tc::bulk_g2s(base + o_nu, a.nu + (size_t)IJ.x * T, T * 4, &full[s]);
+                tc::bulk_g2s(base + o_nu + T * 4, a.nu + (size_t)IJ.y * T, T * 4, &full[s]);
+            };
+            auto basis_part = [&](int s, int2 IJ) {
+                unsigned char *base = sm + (size_t)s * sbytes;
+                tc::bulk_g2s(base + o_a, a.ops + (size_t)IJ.x * a.ops_stride, img, &full[s]);
+                tc::bulk_g2s(base + o_b, a.ops + (size_t)IJ.y * a.ops_stride + img, img, &full[s]);
+                if (ybytes) {
+                    tc::bulk_g2s(base + o_yi, a.Y + (size_t)IJ.x * a.Ykt * T, ybytes, &full[s]);
+                    tc::bulk_g2s(base + o_yj, a.Y + (size_t)IJ.y * a.Ykt * T, ybytes, &full[s]);
+                }
+            };
+            auto tile_at = [&](int t) {
+                int2 IJ = a.wtiles[t];
+                if (!SAP_BOUNDS_OK(a.st, IJ.x >= 0 && IJ.x <= IJ.y && IJ.y < a.Npad / T)) IJ = make_int2(0, 0);
+                return IJ;
+            };
             const int pre = nstatic;
             for (int it = 0; it < pre; ++it) {
                 const int t = blockIdx.x + it * gridDim.x;
-                int2 IJ = a.wtiles[t];
-                if (!SAP_BOUNDS_OK(a.st, IJ.x >= 0 && IJ.x <= IJ.y && IJ.y < a.Npad / T)) IJ = make_int2(0, 0);
+                const int2 IJ = tile_at(t);
                 sIJ[it] = IJ;  // published by the mbarrier completion
-                unsigned char *base = sm + (size_t)it * sbytes;
-                tc::mbar_expect_tx(&full[it], sbytes);
-                tc::bulk_g2s(base, a.wb + (size_t)t * T * T, wbytes, &full[it]);
-                tc::bulk_g2s(base + wbytes + ibytes + jbytes, a.nu + (size_t)IJ.x * T, T * 4, &full[it]);
-                tc::bulk_g2s(base + wbytes + ibytes + jbytes + T * 4, a.nu + (size_t)IJ.y * T, T * 4, &full[it]);
+                constant_part(it, t, IJ);
             }
             grid_dep_wait();
             grid_dep_launch();
-            for (int it = 0; it < pre; ++it) {
-                const int2 IJ = sIJ[it];
-                unsigned char *base = sm + (size_t)it * sbytes;
-                if (DBL) tc::bulk_g2s(base + wbytes, a.Yd + (size_t)IJ.x * a.Ykt * 2 * T, ibytes, &full[it]);
-                else tc::bulk_g2s(base + wbytes, a.Y + (size_t)IJ.x * a.Ykt * T, ibytes, &full[it]);
-                tc::bulk_g2s(base + wbytes + ibytes, a.Y + (size_t)IJ.y * a.Ykt * T, jbytes, &full[it]);
-            }
+            for (int it = 0; it < pre; ++it) basis_part(it, sIJ[it]);
             int issued = pre;
             bool marked = false;
             // Tiles after the first `stages`: with programmatic launch they
@@ -559,41 +591,29 @@ __global__ void __launch_bounds__(kPassThreads, 1) restr_pass_kernel(PassArgs a)
                 return (int)blockIdx.x + it * (int)gridDim.x;
             };
             int tnext = next_tile(pre);
-            int2 IJnext = tnext < a.ntiles ? a.wtiles[tnext] : make_int2(-1, -1);
-            if (tnext < a.ntiles && !SAP_BOUNDS_OK(a.st, IJnext.x >= 0 && IJnext.x <= IJnext.y && IJnext.y < a.Npad / T))
-                IJnext = make_int2(0, 0);
+            int2 IJnext = tnext < a.ntiles ? tile_at(tnext) : make_int2(-1, -1);
             for (int it = pre;; ++it) {
                 const int s = it % S;
                 const int t = tnext;
                 const int2 IJ = IJnext;
                 if (t < a.ntiles) {
                     tnext = next_tile(it + 1);
-                    IJnext = tnext < a.ntiles ? a.wtiles[tnext] : make_int2(-1, -1);
-                    if (tnext < a.ntiles &&
-                        !SAP_BOUNDS_OK(a.st, IJnext.x >= 0 && IJnext.x <= IJnext.y && IJnext.y < a.Npad / T))
-                        IJnext = make_int2(0, 0);
+                    IJnext = tnext < a.ntiles ? tile_at(tnext) : make_int2(-1, -1);
                 }
                 if (it >= S && !tc::mbar_wait_bounded(&empty[s], ((it / S) - 1) & 1, budget)) {
                     atomicOr(&a.st->status, ST_TIMEOUT);
                     break;
                 }
                 if (t >= a.ntiles) {
-                    // no tile left: an arrival without bytes tells the consumers
+                    // no tile left: an arrival without bytes tells the others
                     sIJ[s] = make_int2(-1, -1);
                     tc::mbar_arrive(&full[s]);
                     marked = true;
                     break;
                 }
                 sIJ[s] = IJ;  // published by the mbarrier completion below
-                unsigned char *base = sm + (size_t)s * sbytes;
-                tc::mbar_expect_tx(&full[s], sbytes);
-                tc::bulk_g2s(base, a.wb + (size_t)t * T * T, wbytes, &full[s]);
-                // one copy per side: the basis's components of the point block
-                if (DBL) tc::bulk_g2s(base + wbytes, a.Yd + (size_t)IJ.x * a.Ykt * 2 * T, ibytes, &full[s]);
-                else tc::bulk_g2s(base + wbytes, a.Y + (size_t)IJ.x * a.Ykt * T, ibytes, &full[s]);
-                tc::bulk_g2s(base + wbytes + ibytes, a.Y + (size_t)IJ.y * a.Ykt * T, jbytes, &full[s]);
-                tc::bulk_g2s(base + wbytes + ibytes + jbytes, a.nu + (size_t)IJ.x * T, T * 4, &full[s]);
-                tc::bulk_g2s(base + wbytes + ibytes + jbytes + T * 4, a.nu + (size_t)IJ.y * T, T * 4, &full[s]);
+                constant_part(s, t, IJ);
+                basis_part(s, IJ);
                 ++issued;
             }
             // no copy of ours may still be in flight when the block exits
@@ -605,21 +625,75 @@ __global__ void __launch_bounds__(kPassThreads, 1) restr_pass_kernel(PassArgs a)
             grid_dep_wait();
             grid_dep_launch();
         }
-        return;
-    }
-
+        __syncwarp();
+    } else if (warp == kConsumerWarps + 1) {
+        // ---------------- MMA warp ----------------
+        grid_dep_wait();
+        grid_dep_launch();
+        if (lane == 0) {
+            const uint32_t idesc = tc::idesc_f16(T, T, 0);
+            int it = 0;
+            for (;; ++it) {
+                const int s = it % S, buf = it & 1;
+                if (!tc::mbar_wait_bounded(&full[s], (it / S) & 1, budget)) {
+                    atomicOr(&a.st->status, ST_TIMEOUT);
+                    break;
+                }
+                if (sIJ[s].x < 0) break;
+                if (it >= 2 && !tc::mbar_wait_bounded(&tempty[buf], ((it >> 1) - 1) & 1, budget)) {
+                    atomicOr(&a.st->status, ST_TIMEOUT);
+                    break;
+                }
+                tc::tc_fence_after();
+                const uint32_t sa = tc::smem_u32(sm + (size_t)s * sbytes + o_a);
+                const uint32_t sb = sa + img;
+                for (int q = 0; q < a.ksteps; ++q)
+                    tc::mma_f16(tbase + buf * T, tc::desc_k_plain(sa + q * 4096, 2048, 128),
+                                tc::desc_k_plain(sb + q * 4096, 2048, 128), idesc, q > 0 ? 1u : 0u);
+                tc::mma_commit(&tfull[buf]);
+            }
+            // the tensor memory is freed below: no MMA may be in flight
+            for (int j = it > 2 ? it - 2 : 0; j < it; ++j) tc::mbar_wait_bounded(&tfull[j & 1], (j >> 1) & 1, budget);
+        }
+        __syncwarp();
+    } else {
     // ---------------- consumer warps ----------------
+    // the lane's first near pair (constant over the run)
+    const int nearG = (int)gridDim.x * kConsumerWarps, near0 = (int)blockIdx.x * kConsumerWarps + warp;
+    int2 npr = make_int2(0, 0);
+    float nw = INFINITY;
+    if (EXPL && near0 + lane * nearG < a.n_near) {
+        npr = __ldcg(a.near + near0 + lane * nearG);
+        nw = __ldcg(a.near_w + near0 + lane * nearG);
+    }
     grid_dep_wait();  // Y, the bounds and the lists of this iteration
     grid_dep_launch();
-    const int seg = warp % SR, row0 = warp / SR;
-    const int col0 = seg * 32 * CPT + lane * CPT;
-    const float seed = load_pos_float(&a.st->seed_ub);
-    float uwarp = INFINITY;  // best upper bound this warp has produced
-    // second tier inside the pass: EX pairs per warp and round; the pairs
-    // that survive it are evaluated in FP64 later (this warp's best)
+    // this thread: row `row` of a tile, columns col0 .. col0 + 31
+    const int row = 32 * (warp & 3) + lane, col0 = 32 * (warp >> 2);
+    // Upper bounds of the minimum meet in shared memory; one warp per tile
+    // exchanges the block's with the grid's (thousands of warps polling and
+    // lowering one word cost 3 us at the start of a pass).
+    if (lane == 0) atomicMin(&sub, __float_as_uint(load_pos_float(&a.st->seed_ub)));
+    // r~ +- b_p to an upper and a lower bound (2 10^-6 for the roundings,
+    // the hardware square root's 2^-22 among them)
+    const float inv_up = 1.000002f / (1.0f - a.cert.rho), inv_dn = 0.999998f / (1.0f + a.cert.rho);
+    auto bound_now = [&]() { return __uint_as_float(*(volatile unsigned int *)&sub); };
+    auto lower_bound_to = [&](float ub) {
+        if (lane == 0) atomicMin(&sub, __float_as_uint(ub));
+    };
+    // Second and FP64 tiers inside the pass.  A pair that Y cannot rule out
+    // waits in the warp's pending list with a lower bound of its ratio; at the
+    // end of the tiles (or when the list is full) those the bound of that
+    // moment does not exclude are evaluated: two or fewer in FP64 at once,
+    // more first from explicit FP32 differences, EX per round, which raises
+    // their lower bounds and tightens the upper one.  Waiting matters: the
+    // bound is loose while the first tiles are read, and an evaluation (2-5
+    // us of latency) stalls the block's ring for pairs that are mostly
+    // excluded a few tiles later (a look at the list after 6 tiles left the
+    // slowest blocks 6 us behind at N = 8192 and 20 us at N = 12000).
     constexpr int EX = (K + 1) * 2 <= 32 ? 2 : 1;
     Partial best = {INFINITY, 0x7fffffff, 0x7fffffff};
-    int nd = 0;  // deferred survivors of this warp (warp-uniform)
+    int nd = 0;  // pending pairs of this warp (warp-uniform)
     auto fp64_pair = [&](int2 ij) {
         if constexpr (EXPL) {
             if (!SAP_PAIR_OK(a.st, ij, a.N)) return;
@@ -633,313 +707,393 @@ __global__ void __launch_bounds__(kPassThreads, 1) restr_pass_kernel(PassArgs a)
             if (better_q(q, ij.x, ij.y, best.r, best.i, best.j)) best = Partial{q, ij.x, ij.y};
         }
     };
-    // the bounds from a round's FP32 ratios (lane e < EX: pair e), then its
-    // survivors to the warp's deferred list
-    auto expl_after = [&](const int2 (&pr)[EX], float rr, int code) {
-        if constexpr (EXPL) {
-            const float wmin = warp_min(rr);
-            // any earlier value of the running bound is a valid (looser) bound
-            float U2 = fminf(fminf(seed, uwarp), load_pos_float(&a.st->run_ub2));
-            auto tighten = [&](float ub) {
-                if (lane == 0 && ub < U2) {
-                    atomic_min_pos_float(&a.st->run_ub2, ub);
-                    atomic_min_pos_float(&a.st->run_ub1, ub);  // bounds the pass's own emission too
-                }
-                U2 = fminf(U2, ub);
-                uwarp = fminf(uwarp, ub);
-            };
-            if (wmin < INFINITY) tighten(cert_upper(wmin, a.cert32));
-            unsigned int m = __ballot_sync(0xffffffffu, code == 2 || (code == 1 && rr <= cert_emit_threshold(U2, a.cert32)));
-            // survivors wait in the warp's list until its tiles are done (the
-            // bound is far tighter by then); a full list evaluates at once
-            while (m) {
-                const int e = __ffs(m) - 1;
-                m &= m - 1u;
-                const float re = __shfl_sync(0xffffffffu, code == 2 ? -1.f : rr, e);
-                if (nd < kDefer) {
-                    if (lane == 0) defer[warp][nd] = DeferredPair{pr[e].x, pr[e].y, re};
-                    ++nd;
-                } else {
-                    fp64_pair(pr[e]);
-                }
-            }
-        }
-    };
-    // the deferred survivors against the bound as it is now
-    auto drain = [&]() {
+    auto flush = [&]() {
         if constexpr (EXPL) {
             __syncwarp();
-            const float U2 = fminf(fminf(seed, uwarp), load_pos_float(&a.st->run_ub2));
-            const float th = cert_emit_threshold(U2, a.cert32);
-            for (int q = 0; q < nd; ++q) {
-                const DeferredPair d = defer[warp][q];
-                if (d.r <= th) fp64_pair(make_int2(d.i, d.j));  // r < 0: too short for FP32
+            unsigned long long *list = pending[warp];
+            // one bit per pending pair that can still be the argmin
+            auto alive = [&](unsigned int (&m)[2]) {
+                const float th = bound_now() * 1.000001f;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int q = 32 * h + lane;
+                    m[h] = __ballot_sync(0xffffffffu, q < nd && packed_ratio(list[q < nd ? q : 0]) <= th);
+                }
+            };
+            auto take = [](unsigned int (&m)[2]) {  // the lowest set bit, removed
+                const int h = m[0] ? 0 : 1, e = __ffs(m[h]) - 1;
+                m[h] &= m[h] - 1u;
+                return 32 * h + e;
+            };
+            unsigned int m[2];
+            alive(m);
+            if (__popc(m[0]) + __popc(m[1]) > 2) {
+                unsigned int rem[2] = {m[0], m[1]};
+                while (rem[0] | rem[1]) {
+                    int2 pr[EX];
+                    int at[EX];
+                    bool valid[EX];
+#pragma unroll
+                    for (int e = 0; e < EX; ++e) {
+                        valid[e] = (rem[0] | rem[1]) != 0u;
+                        at[e] = valid[e] ? take(rem) : 0;
+                        pr[e] = valid[e] ? packed_pair(list[at[e]]) : make_int2(0, 0);
+                    }
+                    float rr;
+                    int code;
+                    expl32_eval<K, EX>(a.X, a.n, a.U32, a.KP, pr, valid, lane, rr, code);
+                    const float wmin = warp_min(rr);
+                    if (wmin < INFINITY) {
+                        const float ub = cert_upper(wmin, a.cert32);
+                        if (ub < bound_now()) {
+                            lower_bound_to(ub);
+                            if (lane == 0) atomic_min_pos_float(&a.st->run_ub1, ub);
+                        }
+                    }
+                    __syncwarp();
+#pragma unroll
+                    for (int e = 0; e < EX; ++e)
+                        if (lane == e && valid[e])
+                            list[at[e]] = pack_cand(pr[e].x, pr[e].y,
+                                                    fmaxf((rr - a.cert32.A) / (1.0f + a.cert32.rho) * 0.999998f, 0.f),
+                                                    code == 2);
+                    __syncwarp();
+                }
+                alive(m);
             }
+            while (m[0] | m[1]) fp64_pair(packed_pair(list[take(m)]));
+            __syncwarp();
             nd = 0;
         }
     };
-    auto expl_round = [&](const int2 (&pr)[EX], const bool (&valid)[EX]) {
+    // the pairs of the lanes with keep set join the list
+    auto append = [&](int pi, int pj, float lo, bool keep) {
         if constexpr (EXPL) {
-            float rr;
-            int code;
-            expl32_eval<K, EX>(a.X, a.n, a.U32, a.KP, pr, valid, lane, rr, code);
-            expl_after(pr, rr, code);
+            const unsigned int m = __ballot_sync(0xffffffffu, keep);
+            const int c = __popc(m);
+            if (c == 0) return;
+            if (nd + c > kPending) flush();
+            if (keep) pending[warp][nd + __popc(m & ((1u << lane) - 1u))] = pack_cand(pi, pj, lo, false);
+            nd += c;
         }
     };
-    if constexpr (EXPL) {
-        // the near pairs first, while the first stages' copies land: their
-        // bounds tighten the pass's early (survivors wait, see above)
-        const long long G = (long long)gridDim.x * kConsumerWarps * EX;
-        for (long long base = ((long long)blockIdx.x * kConsumerWarps + warp) * EX; base < a.n_near; base += G) {
-            int2 pr[EX];
-            bool valid[EX];
+    // The near pairs, one per lane: their ratio from Y with their own (large)
+    // bound rules most of them out in O(k); it also bounds the minimum.
+    auto near_pairs = [&]() {
+        if constexpr (EXPL) {
+            for (long long base = 0; base < a.n_near; base += 32ll * nearG) {
+                const long long idx = base + near0 + (long long)lane * nearG;
+                int2 pr = npr;
+                float ub = INFINITY, lo = INFINITY;
+                if (idx < a.n_near) {
+                    if (base > 0) {
+                        pr = __ldcg(a.near + idx);
+                        nw = __ldcg(a.near_w + idx);
+                    }
+                    if (SAP_PAIR_OK(a.st, pr, a.N)) {
+                        const float *yi = a.Y + (size_t)(pr.x >> 7) * a.Ykt * T + (pr.x & (T - 1));
+                        const float *yj = a.Y + (size_t)(pr.y >> 7) * a.Ykt * T + (pr.y & (T - 1));
+                        float zz = 0.f;
 #pragma unroll
-            for (int e = 0; e < EX; ++e) {
-                valid[e] = base + e < a.n_near;
-                pr[e] = valid[e] ? __ldcg(a.near + base + e) : make_int2(0, 0);
-                if (valid[e] && !SAP_PAIR_OK(a.st, pr[e], a.N)) {
-                    valid[e] = false;
-                    pr[e] = make_int2(0, 0);
+                        for (int c = 0; c < K; ++c)
+                            if (c < k) {
+                                const float e = __ldcg(yi + c * T) - __ldcg(yj + c * T);
+                                zz = fmaf(e, e, zz);
+                            }
+                        if (nw < INFINITY) {
+                            const float r = sqrt_up(zz * nw);
+                            const float b = pair_bound(a.beta, __ldg(a.nu + pr.x), __ldg(a.nu + pr.y), nw);
+                            ub = (r + b) * inv_up;
+                            lo = fmaxf((r - b) * inv_dn, 0.f);
+                        } else {
+                            lo = 0.f;  // too short for FP32: a later tier decides
+                        }
+                    }
                 }
+                ub = warp_min(ub);
+                const float U = bound_now();
+                if (ub < U) lower_bound_to(ub);
+                append(pr.x, pr.y, lo, lo <= fminf(U, ub) * 1.000001f && lo < INFINITY);
             }
-            expl_round(pr, valid);
         }
-    }
-    // ring position and barrier phase, advanced without integer division
+    };
+    near_pairs();  // while the first stages' copies land
+    // ring position and barrier phases, advanced without integer division
     int s = 0;
     uint32_t phase = 0;
-    int tcount = 0;  // tiles this warp has consumed
-    for (;; s = (s + 1 == S) ? 0 : s + 1, phase ^= (s == 0) ? 1u : 0u) {
-        // a checkpoint part-way: the survivors so far against the bound as it
-        // is by then (tight once the minimum's tile has been seen), so their
-        // FP64 evaluations overlap the other warps' tiles instead of the tail
-        if constexpr (EXPL) {
-            if (tcount == kDrainTile && nd) drain();
-            ++tcount;
-        }
-        if (!tc::mbar_wait_bounded(&full[s], phase, budget)) {
+    const uint32_t taddr = tbase + ((uint32_t)(32 * (warp & 3)) << 16) + col0;
+    const float wsc = a.w_scale;
+    for (int it = 0;; ++it, s = (s + 1 == S) ? 0 : s + 1, phase ^= (s == 0) ? 1u : 0u) {
+        if (!__all_sync(0xffffffffu, tc::mbar_wait_bounded(&full[s], phase, budget))) {
             if (lane == 0) atomicOr(&a.st->status, ST_TIMEOUT);
             break;
         }
         const int2 IJ = sIJ[s];
         if (IJ.x < 0) break;  // the producer has no more tiles
-        const float gnow = load_pos_float(&a.st->run_ub1);  // consumed after the tile
-        const uint16_t *hs = reinterpret_cast<const uint16_t *>(sm + (size_t)s * sbytes);
-        // row side: yI[c * T + a], or (DBL) the doubled copy yI[c * 2T + yd_offset(a)]
-        const float *yI = reinterpret_cast<const float *>(sm + (size_t)s * sbytes + wbytes);
-        const float *yJ = reinterpret_cast<const float *>(sm + (size_t)s * sbytes + wbytes + ibytes);  // yJ[c * T + b]
-
-        float v[RPW][CPT];
-        float mymin = INFINITY;
-        if (NPR > 0) {
-            uint64_t yj2[NPR > 0 ? NPR : 1][K];
+        const bool exch = warp == (it & (kConsumerWarps - 1));
+        float gnow = INFINITY;
+        if (exch) gnow = load_pos_float(&a.st->run_ub1);  // consumed after the tile
+        const unsigned char *stage = sm + (size_t)s * sbytes;
+        const int buf = it & 1;
+        if (!__all_sync(0xffffffffu, tc::mbar_wait_bounded(&tfull[buf], (it >> 1) & 1, budget))) {
+            if (lane == 0) atomicOr(&a.st->status, ST_TIMEOUT);
+            break;
+        }
+        tc::tc_fence_after();
+        float v[32];  // lower bounds of |y_i - y_j|^2, then of r~^2
+        tc::tmem_ld32(taddr + buf * T, v);
+        tc::tc_fence_before();
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(&tempty[buf]);
+        float m0 = INFINITY, m1 = INFINITY;
+        {
+            const uint4 *wp = reinterpret_cast<const uint4 *>(stage) + (col0 >> 3) * T + row;
 #pragma unroll
-            for (int c = 0; c < K; ++c) {
-                if (CPT == 4) {
-                    const float4 t = *reinterpret_cast<const float4 *>(yJ + c * T + col0);
-                    yj2[0][c] = tc::pk2(t.x, t.y);
-                    yj2[NPR > 1 ? 1 : 0][c] = tc::pk2(t.z, t.w);
-                } else {
-                    const float2 t = *reinterpret_cast<const float2 *>(yJ + c * T + col0);
-                    yj2[0][c] = tc::pk2(t.x, t.y);
+            for (int c = 0; c < 4; ++c) {
+                const uint4 w4 = wp[c * T];
+                const uint32_t ww[4] = {w4.x, w4.y, w4.z, w4.w};
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int e = c * 8 + 2 * q;
+                    const uint64_t p = tc::mul2(tc::pk2(v[e], v[e + 1]),
+                                                tc::pk2(__uint_as_float(ww[q] << 16), __uint_as_float(ww[q])));
+                    const float2 t = tc::upk2(p);
+                    v[e] = t.x;
+                    v[e + 1] = t.y;
+                    m0 = fminf(m0, t.x);
+                    m1 = fminf(m1, t.y);
                 }
-            }
-#pragma unroll
-            for (int r0 = 0; r0 < RPW; r0 += 2) {
-                uint64_t s2[2][NPR > 0 ? NPR : 1];
-#pragma unroll
-                for (int h = 0; h < 2; ++h)
-#pragma unroll
-                    for (int p = 0; p < NPR; ++p) s2[h][p] = 0ull;
-#pragma unroll
-                for (int c = 0; c < K; ++c) {
-                    // rows row0 + r0 RSTEP and the next, each as a {y, y} pair (broadcast)
-                    uint64_t yya, yyb;
-                    if constexpr (DBL) {
-                        const ulonglong2 yy = *reinterpret_cast<const ulonglong2 *>(yI + c * 2 * T + row0 * 16 + (r0 >> 1) * 4);
-                        yya = yy.x;
-                        yyb = yy.y;
-                    } else {
-                        const float yca = yI[c * T + row0 + r0 * RSTEP];
-                        const float ycb = yI[c * T + row0 + (r0 + 1) * RSTEP];
-                        yya = tc::pk2(yca, yca);
-                        yyb = tc::pk2(ycb, ycb);
-                    }
-#pragma unroll
-                    for (int p = 0; p < NPR; ++p) {
-                        const uint64_t ea = tc::sub2(yya, yj2[p][c]);
-                        const uint64_t eb = tc::sub2(yyb, yj2[p][c]);
-                        s2[0][p] = tc::fma2(ea, ea, s2[0][p]);
-                        s2[1][p] = tc::fma2(eb, eb, s2[1][p]);
-                    }
-                }
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int r = r0 + h;
-                    const uint16_t *hr = hs + (row0 + r * RSTEP) * T + col0;
-                    float wv[CPT];  // 1/d^2 of the thread's columns
-                    if (CPT == 4) {
-                        const uint2 raw = *reinterpret_cast<const uint2 *>(hr);
-                        wv[0] = bf16_lo(raw.x); wv[1 % CPT] = bf16_hi(raw.x);
-                        wv[2 % CPT] = bf16_lo(raw.y); wv[3 % CPT] = bf16_hi(raw.y);
-                    } else {
-                        const uint32_t raw = *reinterpret_cast<const uint32_t *>(hr);
-                        wv[0] = bf16_lo(raw); wv[1 % CPT] = bf16_hi(raw);
-                    }
-#pragma unroll
-                    for (int p = 0; p < NPR; ++p) {
-                        const uint64_t ww = tc::pk2(wv[2 * p], wv[(2 * p + 1) % CPT]);
-                        const float2 q = tc::upk2(tc::mul2(s2[h][p], ww));
-                        v[r][(2 * p) % CPT] = q.x;
-                        v[r][(2 * p + 1) % CPT] = q.y;
-                        mymin = fminf(mymin, fminf(q.x, q.y));
-                    }
-                }
-            }
-        } else {
-            float yj[K];
-#pragma unroll
-            for (int c = 0; c < K; ++c) yj[c] = yJ[c * T + col0];
-#pragma unroll
-            for (int r = 0; r < RPW; ++r) {
-                const int row = row0 + r * RSTEP;
-                float sacc = 0.f;
-#pragma unroll
-                for (int c = 0; c < K; ++c) {
-                    const float e = yI[c * T + row] - yj[c];
-                    sacc = fmaf(e, e, sacc);
-                }
-                v[r][0] = sacc * bf16_at(hs + row * T + col0);
-                mymin = fminf(mymin, v[r][0]);
             }
         }
-        float U = fminf(fminf(seed, gnow), uwarp);
+        const float mymin = fminf(m0, m1);
+        if (exch) {
+            const float mine = bound_now();
+            if (gnow < mine) lower_bound_to(gnow);
+            else if (mine < gnow && lane == 0) atomic_min_pos_float(&a.st->run_ub1, mine);
+        }
+        float U = fminf(gnow, bound_now());
         float thc = cert_emit_threshold(U, a.cert);
         float thc2 = thc * thc * 1.000001f;
         // thc >= U, so a tile that could tighten the bound (minimum below
         // U^2) also fails this test: the fast path needs no warp minimum
-        if (!__any_sync(0xffffffffu, mymin <= thc2)) {
+        if (!__any_sync(0xffffffffu, mymin <= thc2 * kFilter)) {
             // fast path: nothing in this tile can bound or be the minimum
-            __syncwarp();
             if (lane == 0) tc::mbar_arrive(&empty[s]);
             continue;
         }
+        // ---- slow path: FP32 rows of Y
+        const float *sI = reinterpret_cast<const float *>(stage + o_yi), *sJ = reinterpret_cast<const float *>(stage + o_yj);
+        const float *gI = a.Y + (size_t)IJ.x * a.Ykt * T, *gJ = a.Y + (size_t)IJ.y * a.Ykt * T;
+        const uint16_t *hs = reinterpret_cast<const uint16_t *>(stage);
+        const float *nuI = reinterpret_cast<const float *>(stage + o_nu), *nuJ = nuI + T;
+        // r~^2 of pair (r, c), its w in w
+        auto pair_q = [&](int r, int c, float &w) {
+            w = __uint_as_float((uint32_t)hs[((c >> 3) * T + r) * 8 + (c & 7)] << 16) * wsc;
+            float q = 0.f;
+            if constexpr (EXPL && K <= 12) {  // staged (pass_stages_y)
+#pragma unroll
+                for (int m = 0; m < K; ++m)
+                    if (m < k) {
+                        const float e = sI[m * T + r] - sJ[m * T + c];
+                        q = fmaf(e, e, q);
+                    }
+            } else if (ybytes) {
+                for (int m = 0; m < k; ++m) {
+                    const float e = sI[m * T + r] - sJ[m * T + c];
+                    q = fmaf(e, e, q);
+                }
+            } else {
+#pragma unroll 4
+                for (int m = 0; m < k; ++m) {
+                    const float e = __ldcg(gI + m * T + r) - __ldcg(gJ + m * T + c);
+                    q = fmaf(e, e, q);
+                }
+            }
+            return q * w;
+        };
         const float wmin = warp_min(mymin);
-        const bool refine = wmin < INFINITY && sqrtf(wmin) < U;  // warp-uniform
-        const float *nuI = reinterpret_cast<const float *>(sm + (size_t)s * sbytes + wbytes + ibytes + jbytes);
-        const float *nuJ = nuI + T;
-        if (refine) {
-            // the bound of the tile's minimum from that pair's own error
+        if (wmin < INFINITY) {
+            // the bound of (about) the tile's minimum from that pair's own error
             const int src = __ffs(__ballot_sync(0xffffffffu, mymin == wmin)) - 1;
-            float ub = 0.f;
+            float ub = INFINITY;
             if (lane == src) {
-                int prow = row0, pcol = col0;
+                int pcol = col0;
 #pragma unroll
-                for (int r = 0; r < RPW; ++r)
-#pragma unroll
-                    for (int q = 0; q < CPT; ++q)
-                        if (v[r][q] == wmin) { prow = row0 + r * RSTEP; pcol = col0 + q; }
-                const float b = pair_bound(a.beta, nuI[prow], nuJ[pcol], bf16_at(hs + prow * T + pcol));
-                ub = (sqrtf(wmin) + b) / (1.0f - a.cert.rho) * 1.000001f;
+                for (int e = 0; e < 32; ++e)
+                    if (v[e] == wmin) pcol = col0 + e;
+                float w;
+                const float r = sqrt_up(pair_q(row, pcol, w));
+                if (r < U) ub = (r + pair_bound(a.beta, nuI[row], nuJ[pcol], w)) * inv_up;
             }
             ub = __shfl_sync(0xffffffffu, ub, src);
-            if (lane == 0 && ub < gnow) atomic_min_pos_float(&a.st->run_ub1, ub);
-            U = fminf(U, ub);
-            uwarp = fminf(uwarp, ub);
-            thc = cert_emit_threshold(U, a.cert);
-            thc2 = thc * thc * 1.000001f;
+            if (ub < U) {
+                lower_bound_to(ub);
+                U = ub;
+                thc = cert_emit_threshold(U, a.cert);
+                thc2 = thc * thc * 1.000001f;
+            }
         }
         // emission: the uniform test, then each survivor against its own bound
         const float ut = U * (1.0f + a.cert.rho);
-        uint32_t emit = 0u;
-        int cnt = 0;
-        if (mymin <= thc2)
+        uint32_t flag = 0u, emit = 0u;
+        if (mymin <= thc2 * kFilter)
 #pragma unroll
-            for (int r = 0; r < RPW; ++r)
-#pragma unroll
-                for (int q = 0; q < CPT; ++q)
-                    if (v[r][q] <= thc2) {
-                        const int prow = row0 + r * RSTEP, pcol = col0 + q;
-                        const float th = (ut + pair_bound(a.beta, nuI[prow], nuJ[pcol], bf16_at(hs + prow * T + pcol))) *
-                                         1.000001f;
-                        if (v[r][q] <= th * th * 1.000001f) {
-                            emit |= 1u << (r * CPT + q);
-                            ++cnt;
-                        }
-                    }
-        // the warp's reads of stage s are done
-        __syncwarp();
-        if (lane == 0) tc::mbar_arrive(&empty[s]);
+            for (int e = 0; e < 32; ++e)
+                if (v[e] <= thc2 * kFilter) flag |= 1u << e;
+        const int i0 = IJ.x * T, j0 = IJ.y * T;
         if constexpr (EXPL) {
+            int total = 0;
+            while (__any_sync(0xffffffffu, flag != 0u)) {  // one flagged pair per lane
+                bool keep = false;
+                float lo = 0.f;
+                const int e = flag ? __ffs(flag) - 1 : 0;
+                if (flag) {
+                    float w;
+                    const float q = pair_q(row, col0 + e, w);
+                    if (q <= thc2) {
+                        const float bp = pair_bound(a.beta, nuI[row], nuJ[col0 + e], w);
+                        const float th = (ut + bp) * 1.000001f;
+                        keep = q <= th * th * 1.000001f;
+                        lo = fmaxf((sqrt_up(q) - bp) * inv_dn, 0.f);
+                    }
+                    flag &= flag - 1u;
+                }
+                total += __popc(__ballot_sync(0xffffffffu, keep));
+                append(i0 + row, j0 + col0 + e, lo, keep);
+            }
+            // the warp's reads of stage s are done
+            __syncwarp();
+            if (lane == 0) {
+                tc::mbar_arrive(&empty[s]);
+                if (total) atomicAdd((unsigned int *)&a.st->cnt1, (unsigned int)total);
+            }
+        } else {
+            while (flag) {
+                const int e = __ffs(flag) - 1;
+                flag &= flag - 1u;
+                float w;
+                const float q = pair_q(row, col0 + e, w);
+                if (q <= thc2) {
+                    const float th = (ut + pair_bound(a.beta, nuI[row], nuJ[col0 + e], w)) * 1.000001f;
+                    if (q <= th * th * 1.000001f) emit |= 1u << e;
+                }
+            }
+            const int cnt = __popc(emit);
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&empty[s]);
             const int total = __reduce_add_sync(0xffffffffu, cnt);
             if (total == 0) continue;
-            if (lane == 0) atomicAdd((unsigned int *)&a.st->cnt1, (unsigned int)total);
-            // the emitted pairs, EX per round: each round takes the lowest
-            // pending pair of each of the first EX lanes that have one
-            const int i0 = IJ.x * T, j0 = IJ.y * T;
-            uint32_t rem = emit;
-            for (;;) {
-                unsigned int has = __ballot_sync(0xffffffffu, rem != 0u);
-                if (!has) break;
-                const int bit = rem ? __ffs(rem) - 1 : 0;
-                const int pi = i0 + row0 + (bit / CPT) * RSTEP, pj = j0 + col0 + bit % CPT;
-                int2 pr[EX];
-                bool valid[EX];
-#pragma unroll
-                for (int e = 0; e < EX; ++e) {
-                    const int src = has ? __ffs(has) - 1 : 0;
-                    valid[e] = has != 0u;
-                    pr[e].x = __shfl_sync(0xffffffffu, pi, src);
-                    pr[e].y = __shfl_sync(0xffffffffu, pj, src);
-                    if (!valid[e]) pr[e] = make_int2(0, 0);
-                    if (has && lane == src) rem &= rem - 1u;
-                    has &= has - 1u;
-                }
-                expl_round(pr, valid);
-            }
-            continue;
-        }
-        if (__any_sync(0xffffffffu, cnt > 0)) {
+            unsigned int cbase = 0;
+            if (lane == 0) cbase = atomicAdd((unsigned int *)&a.st->cnt1, (unsigned int)total);
             int incl = cnt;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
                 const int y = __shfl_up_sync(0xffffffffu, incl, o);
                 if (lane >= o) incl += y;
             }
-            const int total = __shfl_sync(0xffffffffu, incl, 31);
-            unsigned int base = 0;
-            if (lane == 31) base = atomicAdd((unsigned int *)&a.st->cnt1, (unsigned int)total);
-            base = __shfl_sync(0xffffffffu, base, 31);
-            if (cnt) {
-                long long pos = (long long)base + incl - cnt;
-                const int i0 = IJ.x * T, j0 = IJ.y * T;
-#pragma unroll
-                for (int r = 0; r < RPW; ++r)
-#pragma unroll
-                    for (int q = 0; q < CPT; ++q)
-                        if (emit >> (r * CPT + q) & 1u) {
-                            if (pos < a.cap) a.cand[pos] = make_int2(i0 + row0 + r * RSTEP, j0 + col0 + q);
-                            else atomicOr(&a.st->status, ST_OVERFLOW);
-                            ++pos;
-                        }
+            long long pos = (long long)__shfl_sync(0xffffffffu, cbase, 0) + incl - cnt;
+            while (emit) {
+                const int e = __ffs(emit) - 1;
+                emit &= emit - 1u;
+                if (pos < a.cap) a.cand[pos] = make_int2(i0 + row, j0 + col0 + e);
+                else atomicOr(&a.st->status, ST_OVERFLOW);
+                ++pos;
             }
         }
     }
     if constexpr (EXPL) {
-        drain();
-        // the block's best pair: the last consumer warp to finish merges
-        if (lane == 0) {
-            pbest[warp] = best;
-            __threadfence_block();
-            if (atomicAdd(&pdone, 1u) == kConsumerWarps - 1) {
-                __threadfence_block();
-                const volatile Partial *vb = pbest;
-                Partial b = {vb[0].r, vb[0].i, vb[0].j};
-                for (int w2 = 1; w2 < kConsumerWarps; ++w2)
-                    if (better_q(vb[w2].r, vb[w2].i, vb[w2].j, b.r, b.i, b.j)) b = Partial{vb[w2].r, vb[w2].i, vb[w2].j};
-                a.partials[blockIdx.x] = b;
+        // The pending pairs against the grid's bound.  Usually one or two
+        // pairs of the whole grid survive: the block evaluates its own
+        // together, one warp per entry of U^T D and |D|^2 (a warp alone
+        // needs 5-8 us for one pair, most of it FP64 issue).
+        auto meet = [&]() { asm volatile("bar.sync 2, %0;" ::"n"(kConsumerWarps * 32) : "memory"); };
+        // the usual sizes: warp c holds entry c's basis column in registers,
+        // loaded ahead of the barriers that follow
+        const bool direct = a.n <= kSliceN && k < kConsumerWarps;
+        double ur[kSliceN / 32];
+        if (direct && warp < k)
+#pragma unroll
+            for (int t = 0; t < kSliceN / 32; ++t)
+                ur[t] = lane + 32 * t < a.n ? __ldg(a.U64 + (size_t)warp * a.n + lane + 32 * t) : 0.0;
+        meet();
+        if (warp == 0 && lane == 0) {
+            const float g = load_pos_float(&a.st->run_ub1), mine = bound_now();
+            if (mine < g) atomic_min_pos_float(&a.st->run_ub1, mine);
+            else lower_bound_to(g);
+        }
+        meet();
+        {
+            const float th = bound_now() * 1.000001f;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int q = 32 * h + lane;
+                if (q < nd && packed_ratio(pending[warp][q]) <= th) {
+                    const int at = atomicAdd(&nqueue, 1);
+                    if (at < kQueue) queue[at] = pending[warp][q];
+                }
             }
         }
+        meet();
+        const int nq = nqueue;
+        if (nq > kQueue || (size_t)nq * a.n * sizeof(double) > (size_t)T * T * 2) {
+            flush();
+        } else if (nq > 0) {
+            // D of every survivor, in the first ring stage (its tiles are done)
+            double *Ds = reinterpret_cast<double *>(sm);
+            for (int t = tid; t < nq * a.n; t += kConsumerWarps * 32) {
+                const int q = t / a.n, l = t - q * a.n;
+                const int2 ij = packed_pair(queue[q]);
+                Ds[t] = SAP_PAIR_OK(a.st, ij, a.N) ? diff_fp64(__ldg(a.X + (size_t)ij.x * a.n + l), __ldg(a.X + (size_t)ij.y * a.n + l)) : 0.0;
+            }
+            meet();
+            if (direct) {
+                if (warp <= k)
+                    for (int q = 0; q < nq; ++q) {
+                        const double *D = Ds + (size_t)q * a.n;
+                        double v = 0.0;
+#pragma unroll
+                        for (int t = 0; t < kSliceN / 32; ++t)
+                            if (lane + 32 * t < a.n) {
+                                const double d = D[lane + 32 * t];
+                                v = fma(warp < k ? ur[t] : d, d, v);
+                            }
+                        v = warp_sum(v);
+                        if (lane == 0) entries[q][warp] = v;
+                    }
+            } else
+            for (int t = warp; t < nq * (k + 1); t += kConsumerWarps) {
+                const int q = t / (k + 1), c = t - q * (k + 1);
+                const double e = fp64_entry<true>(Ds + (size_t)q * a.n, a.U64, a.n, k, c, lane);
+                if (lane == 0) entries[q][c] = e;
+            }
+            meet();
+            if (warp < nq) {
+                const int2 ij = packed_pair(queue[warp]);
+                constexpr int KS = K <= 8 ? K : K <= 12 ? 12 : K <= 16 ? 16 : K <= 24 ? 24 : 32;
+                double zz, d2;
+                fp64_combine<KS>(entries[warp], a.n, k, lane, zz, d2);
+                if (!(d2 == 0.0 || d2 < a.eps2)) {
+                    const double q = zz / d2;
+                    if (better_q(q, ij.x, ij.y, best.r, best.i, best.j)) best = Partial{q, ij.x, ij.y};
+                }
+            }
+            if (tid == 0) atomicAdd((unsigned int *)&a.st->cnt2, (unsigned int)nq);
+        }
+        if (lane == 0) pbest[warp] = best;
+    }
+    __syncwarp();
+    }
+    tc::tc_fence_before();
+    __syncthreads();
+    if (warp == kConsumerWarps + 1) {
+        tc::tc_fence_after();
+        tc::tmem_dealloc(tbase, kTmemCols);
+    }
+    if (EXPL && tid == 0) {
+        Partial b = pbest[0];
+        for (int w2 = 1; w2 < kConsumerWarps; ++w2)
+            if (better_q(pbest[w2].r, pbest[w2].i, pbest[w2].j, b.r, b.i, b.j)) b = pbest[w2];
+        a.partials[blockIdx.x] = b;
     }
 }
 
@@ -1662,6 +1816,7 @@ sap_status classify(sap_handle h, int k)
     a.wtiles = r.wtiles;
     a.w = r.w;
     a.wb = reinterpret_cast<__nv_bfloat16 *>(r.wb);
+    a.wb_scale = 1.0f / (r.yscale * r.yscale);
     a.eps2_lo = handle_eps2_lo(h);
     a.eps2_hi = handle_eps2_hi(h);
     a.eps2 = handle_eps2(h);
@@ -1685,68 +1840,75 @@ sap_status classify(sap_handle h, int k)
     return SAP_OK;
 }
 
-size_t pass_smem_bytes(int kd, int KY, int stages) { return (size_t)stages * pass_stage_bytes(kd, KY); }
+// The FP32 rows of Y are staged with a tile where that leaves three stages
+// (the slow path then stays in shared memory); wider bases read them from L2.
+bool pass_stages_y(int k) { return 3 * pass_stage_bytes(k, true) <= (uint32_t)kPassDynSmem; }
 
-int pass_pick_stages(int k, int KY)
+int pass_pick_stages(int k)
 {
     int s = kPassStagesMax;
-    while (s > 2 && pass_smem_bytes(pass_kd(k), KY, s) > (size_t)kPassDynSmem) --s;
+    while (s > 2 && s * pass_stage_bytes(k, pass_stages_y(k)) > (uint32_t)kPassDynSmem) --s;
     return s;
 }
 
-// the form with the second tier inside exists for k <= 16
-template <int K, int CPT>
+template <int K, bool EXPL>
 cudaError_t launch_pass_k(const PassArgs &a, int grid, cudaStream_t s)
 {
-    const size_t shm = pass_smem_bytes(CPT == 4 ? K : 0, a.KY, a.stages);
-    if constexpr (K <= 16) {
-        if (a.X) return launch_pdl(a.pdl != 0, restr_pass_kernel<K, CPT, true>, dim3(grid), dim3(kPassThreads), shm, s, a);
-    } else {
-        if (a.X) return cudaErrorNotSupported;
-    }
-    return launch_pdl(a.pdl != 0, restr_pass_kernel<K, CPT, false>, dim3(grid), dim3(kPassThreads), shm, s, a);
+    const size_t shm = (size_t)a.stages * pass_stage_bytes(a.k, a.stage_y != 0);
+    return launch_pdl(a.pdl != 0, restr_pass_kernel<K, EXPL>, dim3(grid), dim3(kPassThreads), shm, s, a);
 }
 
-template <int K, int CPT>
+template <int K, bool EXPL>
 cudaError_t config_pass_k()
 {
-    cudaError_t e = cudaFuncSetAttribute(restr_pass_kernel<K, CPT, false>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kPassDynSmem);
-    if constexpr (K <= 16)
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(restr_pass_kernel<K, CPT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     kPassDynSmem);
-    return e;
+    return cudaFuncSetAttribute(restr_pass_kernel<K, EXPL>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPassDynSmem);
 }
 
 cudaError_t configure_pass_kernels()
 {
     cudaError_t e = cudaSuccess;
     auto f = [&](cudaError_t x) { if (x != cudaSuccess) e = x; };
-    f(config_pass_k<1, 4>()); f(config_pass_k<2, 4>()); f(config_pass_k<3, 4>()); f(config_pass_k<4, 4>());
-    f(config_pass_k<5, 4>()); f(config_pass_k<6, 4>()); f(config_pass_k<7, 4>()); f(config_pass_k<8, 4>());
-    f(config_pass_k<10, 4>()); f(config_pass_k<12, 4>()); f(config_pass_k<16, 4>()); f(config_pass_k<24, 1>()); f(config_pass_k<32, 1>());
+    f(config_pass_k<1, true>()); f(config_pass_k<2, true>()); f(config_pass_k<3, true>()); f(config_pass_k<4, true>());
+    f(config_pass_k<5, true>()); f(config_pass_k<6, true>()); f(config_pass_k<7, true>()); f(config_pass_k<8, true>());
+    f(config_pass_k<10, true>()); f(config_pass_k<12, true>()); f(config_pass_k<16, true>());
+    f(config_pass_k<1, false>());
     return e;
 }
 
-cudaError_t launch_pass(const PassArgs &a, int k, int grid, cudaStream_t s)
+// The form with the second tier inside exists for k <= 16.
+cudaError_t launch_pass(const PassArgs &a, int grid, cudaStream_t s)
 {
-    switch (k) {
-    case 1: return launch_pass_k<1, 4>(a, grid, s);
-    case 2: return launch_pass_k<2, 4>(a, grid, s);
-    case 3: return launch_pass_k<3, 4>(a, grid, s);
-    case 4: return launch_pass_k<4, 4>(a, grid, s);
-    case 5: return launch_pass_k<5, 4>(a, grid, s);
-    case 6: return launch_pass_k<6, 4>(a, grid, s);
-    case 7: return launch_pass_k<7, 4>(a, grid, s);
-    case 8: return launch_pass_k<8, 4>(a, grid, s);
+    if (!a.X) return launch_pass_k<1, false>(a, grid, s);
+    switch (a.k) {
+    case 1: return launch_pass_k<1, true>(a, grid, s);
+    case 2: return launch_pass_k<2, true>(a, grid, s);
+    case 3: return launch_pass_k<3, true>(a, grid, s);
+    case 4: return launch_pass_k<4, true>(a, grid, s);
+    case 5: return launch_pass_k<5, true>(a, grid, s);
+    case 6: return launch_pass_k<6, true>(a, grid, s);
+    case 7: return launch_pass_k<7, true>(a, grid, s);
+    case 8: return launch_pass_k<8, true>(a, grid, s);
     default: break;
     }
-    if (k <= 10) return launch_pass_k<10, 4>(a, grid, s);
-    if (k <= 12) return launch_pass_k<12, 4>(a, grid, s);
-    if (k <= 16) return launch_pass_k<16, 4>(a, grid, s);
-    if (k <= 24) return launch_pass_k<24, 1>(a, grid, s);
-    return launch_pass_k<32, 1>(a, grid, s);
+    if (a.k <= 10) return launch_pass_k<10, true>(a, grid, s);
+    if (a.k <= 12) return launch_pass_k<12, true>(a, grid, s);
+    if (a.k <= 16) return launch_pass_k<16, true>(a, grid, s);
+    return cudaErrorNotSupported;
+}
+
+// Errors of the filter's contraction per unit s_i + s_j (kappa) and absolute
+// (kabs), in units of yscale, |y| <= 64: the two-term FP16 splits (dropped low
+// product and residuals 3 2^-22, norms 2 2^-22, subnormal residuals 2^-25
+// sqrt(k) relative and 2^-24 (sqrt(k) + 1) absolute), the FP32 sum of the
+// norms, and per MMA step a truncation of 2^-23 of twice the running
+// magnitude, itself at most 2 (s_i + s_j), plus slack for the adder tree.
+void op_bounds(int k, float *kappa, float *kabs)
+{
+    const double u22 = std::ldexp(1.0, -22);
+    const double kap = 5.0 * u22 + (k + 2) * std::ldexp(1.0, -24) + (op_ksteps(k) + 4) * std::ldexp(1.0, -21) +
+                       std::sqrt((double)k) * std::ldexp(1.0, -25);
+    *kappa = (float)(kap * 1.1);
+    *kabs = (float)((std::sqrt((double)k) + 1.0) * std::ldexp(1.0, -24) * 1.1);
 }
 
 } // namespace
@@ -1804,6 +1966,8 @@ sap_status restructured_prepare(sap_handle h)
     int e = 0;
     if (mx > 0.f) e = (int)std::ceil(std::log2((double)mx));
     r.xscale = (float)std::ldexp(1.0, -e);
+    // |y| <= ||x - mean|| <= sqrt(n) 2^e (1 + eps_Y): scaled to at most 64
+    r.yscale = (float)std::ldexp(1.0, 6 - e - (int)std::ceil(0.5 * std::log2((double)n) + 0.01));
     const float lo_mul = bf16 ? 256.f : 2048.f;
     if (bf16)
         split_kernel<__nv_bfloat16><<<4 * sms, 256, 0, s>>>(X, N, n, r.center, r.xscale, lo_mul,
@@ -1844,7 +2008,7 @@ sap_status restructured_basis_alloc(sap_handle h)
     dfree(r.Uhi);
     dfree(r.Ulo);
     dfree(r.Y);
-    dfree(r.Yd);
+    dfree(r.ops);
     dfree(r.Ypart);
     r.KPG = (k + 15) / 16 * 16;
     r.KY = padded_stride(k);   // <= KPG; columns >= k are zero
@@ -1854,8 +2018,9 @@ sap_status restructured_basis_alloc(sap_handle h)
     RCK(cudaMemsetAsync(r.Ulo, 0, (size_t)r.KPG * r.NP * 2, s));
     RCK(cudaMalloc(&r.Y, (size_t)r.Npad * r.KY * sizeof(float)));
     RCK(cudaMemsetAsync(r.Y, 0, (size_t)r.Npad * r.KY * sizeof(float), s));
-    RCK(cudaMalloc(&r.Yd, (size_t)r.Npad * r.KY * 2 * sizeof(float)));
-    RCK(cudaMemsetAsync(r.Yd, 0, (size_t)r.Npad * r.KY * 2 * sizeof(float), s));
+    const size_t op_bytes = (size_t)(r.Npad / T) * 2 * op_image_bytes(k);
+    RCK(cudaMalloc(&r.ops, op_bytes));
+    RCK(cudaMemsetAsync(r.ops, 0, op_bytes, s));  // pad halves stay zero
     dfree(r.Ydh);
     dfree(r.Ydl);
     RCK(cudaMalloc(&r.Ydh, (size_t)r.Npad * r.KY * sizeof(float)));
@@ -1890,7 +2055,6 @@ sap_status restructured_set_bound(sap_handle h, double b_cap)
 GemmArgs product_args(sap_handle h, const RestrState &r)
 {
     GemmArgs g = r.gemm;
-    g.Yd = nullptr;
     g.seed_st = nullptr;
     g.Npad = r.Npad;
     g.nkb = r.NP / 64;
@@ -1902,12 +2066,33 @@ GemmArgs product_args(sap_handle h, const RestrState &r)
     return g;
 }
 
+uint32_t restructured_op_groups(GemmArgs &g, const int *k, int count)
+{
+    uint32_t off = 0;
+    int grp = 0;
+    g.nbases = count;
+    for (int q = 0; q < count; ++q) {
+        float kappa, kabs;
+        op_bounds(k[q], &kappa, &kabs);
+        const int used = (k[q] + 3) / 4, all = padded_stride(k[q]) / 4;
+        g.base_group[q] = grp;
+        for (int c = 0; c < all; ++c)
+            g.groups[grp++] = OpGroup{off, op_image_bytes(k[q]), c < used ? c : -1, c == used - 1, 1.0f - kappa, 0.5f * kabs};
+        off += 2 * op_image_bytes(k[q]);
+    }
+    g.base_group[count] = grp;
+    return off;
+}
+
 sap_status restructured_enqueue_product(sap_handle h, const CUtensorMap *mhi, const CUtensorMap *mlo, int KPG,
-                                        float *Y, float *Yd, int KY, float *Ypart, ProbState *st, cudaStream_t s,
-                                        bool seeds)
+                                        float *Y, const OpsView &ops, int KY, float *Ypart, ProbState *st,
+                                        cudaStream_t s, bool seeds)
 {
     RestrState &r = restr_state(h);
     GemmArgs g = product_args(h, r);
+    g.ops = ops.ops;
+    g.ops_stride = restructured_op_groups(g, ops.k, ops.count);
+    g.ops_scale = r.yscale;
     if (seeds) {
         g.seed_X = handle_x32(h);
         g.seed_U = handle_u32(h);
@@ -1921,7 +2106,6 @@ sap_status restructured_enqueue_product(sap_handle h, const CUtensorMap *mhi, co
     g.tb_hi = *mhi;
     g.tb_lo = *mlo;
     g.Y = Y;
-    g.Yd = Yd;
     g.KY = KY;
     g.KPG = KPG;
     g.stages = gemm_pick_stages(KPG, g.nkb);
@@ -1948,14 +2132,19 @@ sap_status restructured_enqueue_basis(sap_handle h, const BasisView &b, cudaStre
         p.wtiles = r.wtiles;
         p.ntiles = r.nwtiles;
         p.Y = b.Y;
-        p.Yd = b.Yd;
-        p.KY = b.KY;
+        p.ops = b.ops;
+        p.ops_stride = b.ops_stride;
+        p.img = op_image_bytes(b.k);
+        p.ksteps = op_ksteps(b.k);
+        p.stage_y = pass_stages_y(b.k);
+        p.w_scale = r.yscale * r.yscale;
         p.Ykt = b.Ykt;
         p.Npad = r.Npad;
         p.nu = r.nu;
         p.beta = (float)(std::sqrt((double)b.k) * r.y_eps * 1.02);
-        p.stages = pass_pick_stages(b.k, b.KY);
+        p.stages = pass_pick_stages(b.k);
         if (handle_tune(h).pass_stages >= 2) p.stages = std::min(p.stages, handle_tune(h).pass_stages);
+        p.k = b.k;
         p.cert = cert_pass(n, b.k, r.b_cap);
         p.st = b.st;
         p.cand = b.cand1;
@@ -1968,16 +2157,16 @@ sap_status restructured_enqueue_basis(sap_handle h, const BasisView &b, cudaStre
             p.U32 = b.U32;
             p.KP = b.KP;
             p.U64 = b.U64;
-            p.k = b.k;
             p.eps2 = handle_eps2(h);
             p.near = r.near;
+            p.near_w = r.near_w;
             p.n_near = r.n_near;
             p.partials = b.partials;
             p.cert32 = cert_explicit(n, b.k);
         }
         handle_count_launch(h, 1, &ea, &eb);
         if (ea) cudaEventRecord(ea, s);
-        RCK(launch_pass(p, b.k, restructured_pass_grid(h), s));
+        RCK(launch_pass(p, restructured_pass_grid(h), s));
         if (eb) cudaEventRecord(eb, s);
         handle_push_timing(h, 1, ea, eb);
     }
@@ -2062,8 +2251,9 @@ sap_status restructured_enqueue(sap_handle h, double alpha)
     (void)alpha;
     RestrState &r = restr_state(h);
     cudaStream_t s = handle_stream(h);
-    sap_status st = restructured_enqueue_product(h, &r.gemm.tb_hi, &r.gemm.tb_lo, r.KPG, r.Y, r.Yd, r.KY, r.Ypart,
-                                                 handle_state(h), s, true);
+    const int k = handle_k(h);
+    sap_status st = restructured_enqueue_product(h, &r.gemm.tb_hi, &r.gemm.tb_lo, r.KPG, r.Y, OpsView{r.ops, &k, 1}, r.KY,
+                                                 r.Ypart, handle_state(h), s, true);
     if (st != SAP_OK) return st;
     BasisView b;
     b.k = handle_k(h);
@@ -2072,8 +2262,9 @@ sap_status restructured_enqueue(sap_handle h, double alpha)
     b.U32 = handle_u32(h);
     b.U32lo = handle_u32lo(h);
     b.Y = r.Y;
-    b.Yd = r.Yd;
     b.Ykt = r.KY;
+    b.ops = r.ops;
+    b.ops_stride = 2 * op_image_bytes(b.k);
     b.Ydh = r.Ydh;
     b.Ydl = r.Ydl;
     b.st = handle_state(h);
@@ -2244,7 +2435,7 @@ void restructured_free(sap_handle h)
 {
     RestrState &r = restr_state(h);
     dfree(r.Xhi); dfree(r.Xlo); dfree(r.center); dfree(r.colpart); dfree(r.nu); dfree(r.w); dfree(r.wtiles);
-    dfree(r.near); dfree(r.counters); dfree(r.Uhi); dfree(r.Ulo); dfree(r.Y); dfree(r.Yd); dfree(r.Ypart);
+    dfree(r.near); dfree(r.counters); dfree(r.Uhi); dfree(r.Ulo); dfree(r.Y); dfree(r.ops); dfree(r.Ypart);
     dfree(r.near_w); dfree(r.xn); dfree(r.Ydh); dfree(r.Ydl); dfree(r.wb);
 }
 

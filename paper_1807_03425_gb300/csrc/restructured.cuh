@@ -22,7 +22,8 @@ struct RestrState {
     // NaN marks a pair the pass skips (invalid, excluded, or near)
     float *w = nullptr;
     // the same tiles as BF16 w_ij (raw bits), the form the pass streams
-    // (2 bytes per pair); NaN where w is NaN
+    // (2 bytes per pair), divided by yscale^2; NaN where w is NaN.  Within a
+    // tile, pair (a, b) sits at ((b / 8) * 128 + a) * 8 + b % 8
     uint16_t *wb = nullptr;
     int2 *wtiles = nullptr;   // (I, J) per tile, I <= J
     int nwtiles = 0;
@@ -41,7 +42,8 @@ struct RestrState {
     void *Uhi = nullptr, *Ulo = nullptr;  // KPG x NP 16-bit
     int KPG = 0;              // k rounded up to the MMA N granule (16)
     float *Y = nullptr;       // block-major [Npad/128][KY][128]
-    float *Yd = nullptr;      // doubled row-side copy of Y for the pass: [Npad/128][KY][256]
+    unsigned char *ops = nullptr;  // the pass's filter operands: per 128-point block, A and B images
+    float yscale = 1.f;       // power of two: |y| * yscale <= 64 for any orthonormal basis
     float *Ydh = nullptr, *Ydl = nullptr;  // double-float Y of the refine tier, KY x Npad each
     int KY = 0;               // k rounded up to 4
     int ksplit = 1;           // K slices of the product (shorter accumulation chains)
@@ -84,8 +86,9 @@ struct BasisView {
     int k, KP, KY;            // width, FP32 basis stride, Y stride (components)
     const float *U32, *U32lo; // n x KP FP32 basis and its low part
     float *Y;                 // this basis's first component in block 0 of a block-major Y
-    float *Yd;                // the same in the doubled row-side copy (block stride Ykt * 256)
     int Ykt;                  // components per 128-point block of that Y buffer
+    const unsigned char *ops; // this basis's A image in block 0 of the filter operands
+    uint32_t ops_stride;      // bytes between blocks
     float *Ydh, *Ydl;         // double-float Y (refine tier), KY x Npad each
     ProbState *st;
     int2 *cand1, *cand2;      // candidate lists of the pass and of the explicit tier
@@ -94,12 +97,23 @@ struct BasisView {
     Partial *partials;        // per-block best pairs (tiers inside the pass)
 };
 
+// Filter operands of a product: the buffer and the bases' widths.
+struct OpsView {
+    unsigned char *ops = nullptr;
+    const int *k = nullptr;
+    int count = 0;
+};
+
 // Restructured-form entry points (restructured.cu).
 // seeds: the product also evaluates the next pass's seed bound (one basis
 // per handle; the update then leaves the seeds to it)
 sap_status restructured_enqueue_product(sap_handle h, const CUtensorMap *mhi, const CUtensorMap *mlo, int KPG,
-                                        float *Y, float *Yd, int KY, float *Ypart, ProbState *st, cudaStream_t s,
-                                        bool seeds = false);
+                                        float *Y, const OpsView &ops, int KY, float *Ypart, ProbState *st,
+                                        cudaStream_t s, bool seeds = false);
+// Fills the filter-operand part of a product's arguments for `count` bases of
+// widths k[q] whose components start at multiples of 4, padded_stride(k[q])
+// each; returns the bytes of a block's images.
+uint32_t restructured_op_groups(GemmArgs &g, const int *k, int count);
 sap_status restructured_enqueue_basis(sap_handle h, const BasisView &b, cudaStream_t s); // pass + explicit tier
 bool restructured_u_maps(sap_handle h, void *Uhi, void *Ulo, int KPG, CUtensorMap *mhi, CUtensorMap *mlo);
 sap_status restructured_classify(sap_handle h, int k);  // near list for width k (valid for every k' <= k)

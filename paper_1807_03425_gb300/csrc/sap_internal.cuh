@@ -397,6 +397,68 @@ __device__ __forceinline__ double warp_sum(double v)
     return v;
 }
 
+// The FP64 value of an FP32 number by integer operations (a conversion
+// occupies the FP64 pipe like an FP64 addition).
+__device__ __forceinline__ double widen(float f)
+{
+    const unsigned int u = __float_as_uint(f);
+    if ((u & 0x7f800000u) == 0u || (u & 0x7f800000u) == 0x7f800000u) return (double)f;  // zero, subnormal, not finite
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
+}
+
+// x - y in FP64: the exact FP32 sum and remainder, then one FP64 addition
+// (the same rounding as the subtraction of the widened numbers).
+__device__ __forceinline__ double diff_fp64(float x, float y)
+{
+    const float s = __fsub_rn(x, y);
+    const float bb = __fsub_rn(s, x);
+    const float e = __fsub_rn(__fsub_rn(x, __fsub_rn(s, bb)), __fadd_rn(y, bb));
+    return widen(s) + widen(e);
+}
+
+// The same sums with one warp per entry (a block evaluates a few pairs
+// together): entry c < k of U^T D, or |D|^2 for c == k, with D = x_i - x_j in
+// shared memory; every lane returns the total.  The order of the additions is
+// fp64_pair_parts's.
+template <bool RO>
+__device__ __forceinline__ double fp64_entry(const double *D, const double *U64, int n, int k, int c, int lane)
+{
+    const double *u = U64 + (size_t)(c < k ? c : 0) * n;
+    const int slices = n <= kSliceN ? 1 : kFp64Slices;
+    double t = 0.0;
+    for (int s = 0; s < slices; ++s) {
+        double v = 0.0;
+#pragma unroll 4
+        for (int l = 32 * s + lane; l < n; l += 32 * slices) v = fma(c < k ? ld_fp64<double, RO>(u + l) : D[l], D[l], v);
+        v = warp_sum(v);
+        t = slices == 1 ? v : t + v;
+    }
+    return t;
+}
+
+// zz and d2 from the k + 1 totals e[0 .. k] in shared memory (|D|^2 last), by
+// a warp; K is the compute width of fp64_pair_parts for this k.
+template <int K>
+__device__ __forceinline__ void fp64_combine(const double *e, int n, int k, int lane, double &zz, double &d2)
+{
+    constexpr int M = K + 1, S = M <= 8 ? 8 : M <= 16 ? 16 : 32, dup = 32 / S;
+    static_assert(M <= 32, "one entry per lane");
+    d2 = e[k];
+    if (n <= kSliceN) {
+        const int idx = rs_index<S>(lane);
+        double sq = 0.0;
+        if (idx < k && lane % dup == 0) sq = e[idx] * e[idx];
+#pragma unroll
+        for (int o = 16; o >= dup; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+        zz = __shfl_sync(0xffffffffu, sq, 0);
+    } else {
+        zz = 0.0;
+#pragma unroll
+        for (int c = 0; c < K; ++c)
+            if (c < k) zz = fma(e[c], e[c], zz);
+    }
+}
+
 __device__ __forceinline__ float warp_sumf(float v)
 {
 #pragma unroll
@@ -595,16 +657,6 @@ __device__ __forceinline__ float packed_ratio(unsigned long long v)
 __device__ __forceinline__ int2 packed_pair(unsigned long long v)
 {
     return make_int2((int)(v >> 47), (int)((v >> 30) & 0x1ffffull));
-}
-
-// Offset of row a (0..127) of a block in the doubled row-side copy of Y
-// (per component 256 floats): the all-pairs pass's consumer warp g (0..15)
-// takes rows g, g + 16, ..., g + 112, two at a time, so row a = 16 r + g
-// sits at g * 16 + (r / 2) * 4 + (r % 2) * 2 as the pair {y_a, y_a}.
-__host__ __device__ __forceinline__ int yd_offset(int a)
-{
-    const int g = a & 15, r = a >> 4;
-    return g * 16 + (r >> 1) * 4 + (r & 1) * 2;
 }
 
 // ---------------------------------------------------------------------------

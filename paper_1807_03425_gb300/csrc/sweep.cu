@@ -84,7 +84,13 @@ sap_status alloc_impl(sap_handle h, SweepState *&swp, int kmax, int hist_need)
     WCK(cudaMemsetAsync(sw.Uhi, 0, (size_t)sw.KPG * r.NP * 2, s0));  // pad rows and columns stay zero
     WCK(cudaMemsetAsync(sw.Ulo, 0, (size_t)sw.KPG * r.NP * 2, s0));
     WCK(cudaMalloc(&sw.Y, (size_t)sw.KY * r.Npad * sizeof(float)));
-    WCK(cudaMalloc(&sw.Yd, (size_t)sw.KY * r.Npad * 2 * sizeof(float)));
+    std::vector<int> ks(kmax);
+    for (int q = 0; q < kmax; ++q) ks[q] = q + 1;
+    GemmArgs sized;
+    sw.ops_stride = restructured_op_groups(sized, ks.data(), kmax);
+    WCK(cudaMalloc(&sw.ops, (size_t)(r.Npad / kTile) * sw.ops_stride));
+    WCK(cudaMemsetAsync(sw.ops, 0, (size_t)(r.Npad / kTile) * sw.ops_stride, handle_stream(h)));
+    sw.ks = ks;
     if (sw.ksplit > 1) WCK(cudaMalloc(&sw.Ypart, (size_t)sw.ksplit * sw.KY * r.Npad * sizeof(float)));
     WCK(cudaMalloc(&sw.gst, sizeof(ProbState)));
     WCK(cudaMemsetAsync(sw.gst, 0, sizeof(ProbState), s0));
@@ -202,9 +208,11 @@ sap_status enqueue_iteration(sap_handle h, SweepState &sw, double alpha, int eva
 {
     RestrState &r = restr_state(h);
     cudaStream_t s0 = handle_stream(h);
-    sap_status st = restructured_enqueue_product(h, &sw.mhi, &sw.mlo, sw.KPG, sw.Y, sw.Yd, sw.KY, sw.Ypart, sw.gst, s0);
+    sap_status st = restructured_enqueue_product(h, &sw.mhi, &sw.mlo, sw.KPG, sw.Y,
+                                                 OpsView{sw.ops, sw.ks.data(), sw.kmax}, sw.KY, sw.Ypart, sw.gst, s0);
     if (st != SAP_OK) return st;
     WCK(cudaEventRecord(sw.fork, s0));
+    uint32_t op_off = 0;
     for (SweepBasis &b : sw.b) {
         WCK(cudaStreamWaitEvent(b.stream, sw.fork, 0));
         BasisView v;
@@ -214,8 +222,10 @@ sap_status enqueue_iteration(sap_handle h, SweepState &sw, double alpha, int eva
         v.U32 = b.U32;
         v.U32lo = b.U32lo;
         v.Y = sw.Y + (size_t)b.off * 128;  // block-major: the basis's components within each block
-        v.Yd = sw.Yd + (size_t)b.off * 256;
         v.Ykt = sw.KY;
+        v.ops = sw.ops + op_off;
+        v.ops_stride = sw.ops_stride;
+        op_off += 2 * op_image_bytes(b.k);
         v.Ydh = b.Ydh;
         v.Ydl = b.Ydl;
         v.st = b.st;
@@ -395,7 +405,7 @@ void sweep_free(SweepState *&s)
         if (b.stream) cudaStreamDestroy(b.stream);
         if (b.done) cudaEventDestroy(b.done);
     }
-    wfree(s->Uhi); wfree(s->Ulo); wfree(s->Y); wfree(s->Yd); wfree(s->Ypart); wfree(s->gst);
+    wfree(s->Uhi); wfree(s->Ulo); wfree(s->Y); wfree(s->ops); wfree(s->Ypart); wfree(s->gst);
     wfree(s->views); wfree(s->pack);
     if (s->fork) cudaEventDestroy(s->fork);
     delete s;

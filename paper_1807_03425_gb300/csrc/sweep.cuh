@@ -36,7 +36,9 @@ struct SweepState {
     int KPG = 0;
     CUtensorMap mhi, mlo;
     float *Y = nullptr;                   // KY x Npad, all bases' components
-    float *Yd = nullptr;                  // doubled row-side copy for the pass (2 KY x Npad)
+    unsigned char *ops = nullptr;         // the passes' filter operands, all bases per 128-point block
+    uint32_t ops_stride = 0;
+    std::vector<int> ks;                  // widths 1..kmax
     int KY = 0;
     float *Ypart = nullptr;
     int ksplit = 1;

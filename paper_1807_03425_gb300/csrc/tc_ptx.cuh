@@ -165,6 +165,19 @@ __device__ __forceinline__ uint64_t desc_k_sw128(uint32_t saddr)
     return d;
 }
 
+// Shared-memory matrix descriptor of an unswizzled K-major operand in
+// core-matrix order: 8-row x 16-byte core matrices, `ldo` bytes between
+// neighbours along K and `sdo` bytes between neighbours along M/N.
+__device__ __forceinline__ uint64_t desc_k_plain(uint32_t saddr, uint32_t ldo, uint32_t sdo)
+{
+    uint64_t d = 0;
+    d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
+    d |= (uint64_t)(ldo >> 4) << 16;
+    d |= (uint64_t)(sdo >> 4) << 32;
+    d |= (uint64_t)1u << 46;
+    return d;
+}
+
 // Instruction descriptor of kind::f16 with FP32 accumulation, both operands
 // K-major.  ab_bf16 selects BF16 (1) or FP16 (0) for A and B alike.
 __host__ __device__ constexpr uint32_t idesc_f16(int M, int N, int ab_bf16)
@@ -203,6 +216,18 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float *v)
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
     for (int q = 0; q < 8; ++q) v[q] = __uint_as_float(r[q]);
+}
+
+// Each thread of a warp reads 32 consecutive 32-bit columns of its TMEM lane.
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32])
+{
+    uint32_t r[32];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+                 : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int q = 0; q < 32; ++q) v[q] = __uint_as_float(r[q]);
 }
 
 } // namespace tc

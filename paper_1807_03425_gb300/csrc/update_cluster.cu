@@ -62,16 +62,6 @@ __host__ inline int cluster_blocks(int n)
 }
 __host__ __device__ inline int cluster_rows(int n, int blocks) { return (n + blocks - 1) / blocks; }
 
-// The FP64 value of an FP32 number by integer operations (off the FP64
-// pipe); subnormals become zero.
-__device__ __forceinline__ double widen(float f)
-{
-    const unsigned int u = __float_as_uint(f);
-    const bool nz = (u & 0x7f800000u) != 0u;
-    const unsigned int hi = (u & 0x80000000u) | (nz ? ((u & 0x7fffffffu) >> 3) + 0x38000000u : 0u);
-    return __hiloint2double((int)hi, nz ? (int)(u << 29) : 0);
-}
-
 // Shared memory of one block (dynamic).
 template <int K>
 struct UpdLayout {
