@@ -105,6 +105,7 @@ struct sap_ctx {
 
     // uneven batch: one ordinary handle per dataset, run together
     bool is_batch = false;
+    bool shared = false;     // a dataset of a batch whose passes together want more SMs than there are
     std::vector<sap_handle> kids;
     std::vector<cudaEvent_t> kid_done;
     cudaEvent_t fork = nullptr;
@@ -339,6 +340,7 @@ sap_status enqueue_iteration(sap_handle h, double alpha, int eval_only, Partial 
             bv.k = h->k;
             bv.cand1 = h->cand1;
             bv.cand2 = h->cand2;
+            bv.shared = h->shared;
             restructured_fuse_args(h, bv, u);
         }
         Timed t(h, K_UPDATE);
@@ -435,6 +437,7 @@ int handle_sms(sap_handle h) { return h->sms; }
 ProbState *handle_state(sap_handle h) { return h->st; }
 const float *handle_x32(sap_handle h) { return h->X32; }
 const double *handle_x64(sap_handle h) { return h->X64; }
+const float *handle_nu(sap_handle h) { return h->rs.nu; }
 sap_status secant_pca(sap_handle h, int k, double *U_out, double *sigma_out);  // pca.cu
 const float *handle_u32(sap_handle h) { return h->U32; }
 const float *handle_u32lo(sap_handle h) { return h->U32lo; }
@@ -487,6 +490,7 @@ TuneKey handle_tune_key(sap_handle h)
     std::memcpy(&t.eps_bits, &h->eps, sizeof(double));
     return t;
 }
+bool handle_shared(sap_handle h) { return h->shared; }
 bool &handle_tuning_flag(sap_handle h) { return h->tuning; }
 void handle_shard(sap_handle h, long long *t0, long long *t1)
 {
@@ -1475,6 +1479,9 @@ sap_status sap_create_batch(const void *const *Xs, const int64_t *Ns, int32_t B,
         if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) return cleanup_fail(SAP_E_CUDA);
         h->kid_done.push_back(e);
     }
+    long long want = 0;
+    for (sap_handle kid : h->kids) want += std::min(kid->rs.nwtiles, h->sms);
+    for (sap_handle kid : h->kids) kid->shared = want > h->sms;
     *out = h;
     return SAP_OK;
 }

@@ -147,7 +147,7 @@ __device__ __forceinline__ void op_group(unsigned char *images, const OpGroup &o
 
 // 128 threads (TMA producer, MMA issuer, four epilogue warps over the TMEM
 // lane quadrants), or 192 where warps 4 and 5 evaluate the seeds meanwhile.
-__global__ void __launch_bounds__(192, 1) gemm_y_kernel(const __grid_constant__ GemmArgs a)
+__global__ void __launch_bounds__(192, 2) gemm_y_kernel(const __grid_constant__ GemmArgs a)
 {
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -331,10 +331,14 @@ size_t gemm_smem_bytes(int KPG, int stages)
     return 1024 + stages * stage + (2 * stages + 1) * 8 + 16;
 }
 
-int gemm_pick_stages(int KPG, int nkb)
+// Ring depth: up to 4 stages, but where the grid does not fit one CTA per SM
+// few enough that two CTAs share one (156 CTAs at N = 19939 were a second
+// wave of four: @@ -> @@ us).
+int gemm_pick_stages(int KPG, int nkb, int ctas, int sms)
 {
     int s = 4;
-    while (s > 1 && gemm_smem_bytes(KPG, s) > 200 * 1024) --s;
+    const size_t limit = ctas > sms && 4 * KPG <= 512 ? 112 * 1024 : 200 * 1024;
+    while (s > 1 && gemm_smem_bytes(KPG, s) > limit) --s;
     return s < nkb ? s : (nkb > 0 ? nkb : 1);
 }
 

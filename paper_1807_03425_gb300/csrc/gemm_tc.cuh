@@ -67,7 +67,7 @@ struct GemmArgs {
 };
 
 size_t gemm_smem_bytes(int KPG, int stages);
-int gemm_pick_stages(int KPG, int nkb);
+int gemm_pick_stages(int KPG, int nkb, int ctas, int sms);
 cudaError_t gemm_configure();
 // Y = X U; with ksplit > 1 each K slice accumulates separately (shorter FP32
 // chains) and a second kernel sums the slices into Y.

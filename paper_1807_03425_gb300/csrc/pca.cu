@@ -45,6 +45,7 @@ int handle_n_dim(sap_handle h);
 const float *handle_x32(sap_handle h);
 const double *handle_x64(sap_handle h);
 double handle_eps2(sap_handle h);
+const float *handle_nu(sap_handle h);  // ||x_i - mean||, rounded up (FP32/BF16 data)
 sap_status handle_fail(sap_handle h, sap_status s, const char *msg);
 
 namespace {
@@ -157,28 +158,219 @@ __global__ void __launch_bounds__(256) lap_rows_kernel(const TX *X, int N, int n
     }
 }
 
-// C[a][b] = sum_i (x_ia - mean_a) R_ib over a 16 x 16 block of (a, b).
+// ---- FP32/BF16 data: the same two kernels in FP32 pairs (double-float)
+//
+// FP64 issues at 1/64 of the FP32 rate here, and the two kernels above are
+// bound by it (12.6 ms and 39 ms at N = 8192, n = 100).  With FP32 points the
+// difference of two coordinates is an exact FP32 pair s + e, so lengths and
+// weighted differences can be formed with error-free FP32 steps (18
+// operations instead of two FP64 ones: @@ ms and @@ ms), accurate to a few
+// 2^-48 of the running sums.  That is enough where w = 1/d^2 is moderate; the
+// Laplacian's rounding error is carried by the short secants, whose terms (of
+// size 1/d) cancel between neighbours, so pairs with d below a sixteenth of
+// the largest ||x - mean|| keep FP64 arithmetic throughout.  Measured against
+// 64 bits the vectors' and values' errors are those of the FP64 form (the
+// short secants' rounding dominates both).
+//
+// A pair's 8 bytes hold either the FP64 w (sign bit 0; 0.0: excluded) or,
+// sign bit 1, the FP32 pair: -wh in the high word, wl in the low one.
+
+__device__ __forceinline__ void two_diff(float a, float b, float &s, float &e)
+{
+    s = __fsub_rn(a, b);
+    const float bb = __fsub_rn(s, a);
+    e = __fsub_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fadd_rn(b, bb));
+}
+__device__ __forceinline__ void add_pair(float &hi, float &lo, float p, float pe)
+{
+    const float s = __fadd_rn(hi, p);
+    const float bb = __fsub_rn(s, hi);
+    const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(p, bb));
+    hi = s;
+    lo = __fadd_rn(lo, __fadd_rn(e, pe));
+}
+
+__global__ void __launch_bounds__(256) w_pair_kernel(const float *X, int N, int n, const int2 *tiles, double eps2,
+                                                     double d2cut, unsigned long long *w)
+{
+    __shared__ float xi[PC][PT + 4], xj[PC][PT + 4];
+    const int2 IJ = tiles[blockIdx.x];
+    const int i0 = IJ.x * PT, j0 = IJ.y * PT;
+    const int tr = threadIdx.x >> 4, tc = threadIdx.x & 15;  // 4 x 4 pairs each
+    float hi[4][4], lo[4][4];
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) hi[p][q] = lo[p][q] = 0.f;
+    for (int c0 = 0; c0 < n; c0 += PC) {
+        __syncthreads();
+        for (int idx = threadIdx.x; idx < PT * PC; idx += 256) {
+            const int r = idx / PC, l = idx % PC;
+            const bool inl = c0 + l < n;
+            xi[l][r] = (i0 + r < N && inl) ? X[(size_t)(i0 + r) * n + c0 + l] : 0.f;
+            xj[l][r] = (j0 + r < N && inl) ? X[(size_t)(j0 + r) * n + c0 + l] : 0.f;
+        }
+        __syncthreads();
+        const int lc = min(PC, n - c0);
+#pragma unroll 2
+        for (int l = 0; l < lc; ++l) {
+            const float4 a4 = *reinterpret_cast<const float4 *>(&xi[l][tr * 4]);
+            const float4 b4 = *reinterpret_cast<const float4 *>(&xj[l][tc * 4]);
+            const float a[4] = {a4.x, a4.y, a4.z, a4.w}, b[4] = {b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+            for (int p = 0; p < 4; ++p)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    float s, e;
+                    two_diff(a[p], b[q], s, e);
+                    const float sq = __fmul_rn(s, s);
+                    float r = fmaf(s, s, -sq);
+                    r = fmaf(__fadd_rn(s, s), e, r);
+                    add_pair(hi[p][q], lo[p][q], sq, r);
+                }
+        }
+    }
+    unsigned long long *out = w + (size_t)blockIdx.x * PT * PT;
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int i = i0 + tr * 4 + p, j = j0 + tc * 4 + q;
+            unsigned long long v = 0ull;
+            if (i < j && j < N) {
+                double d = (double)hi[p][q] + (double)lo[p][q];
+                const bool far_ = d >= d2cut;
+                // short secants, the threshold's neighbourhood (the exclusion
+                // is decided in FP64) and lengths outside FP32's safe range
+                if (!far_ || !(hi[p][q] < 1e30f) || fabs(d - eps2) <= 1e-9 * eps2) {
+                    d = 0.0;
+                    for (int l = 0; l < n; ++l) {
+                        const double D = (double)X[(size_t)i * n + l] - (double)X[(size_t)j * n + l];
+                        d = fma(D, D, d);
+                    }
+                }
+                if (d != 0.0 && !(d < eps2)) {
+                    const double wv = 1.0 / d;
+                    const float wh = (float)wv;
+                    if (far_ && wh < 1e30f && wh > 1e-25f) {
+                        const float wl = (float)(wv - (double)wh);
+                        v = ((unsigned long long)(__float_as_uint(wh) | 0x80000000u) << 32) | __float_as_uint(wl);
+                    } else {
+                        v = (unsigned long long)__double_as_longlong(wv);
+                    }
+                }
+            }
+            out[(tr * 4 + p) * PT + tc * 4 + q] = v;
+        }
+}
+
+// R_i as in lap_rows_kernel: the FP32 pairs' sums over one block of columns,
+// then added in FP64 (partial sums stay small, so their 2^-48 do too).
+__global__ void __launch_bounds__(256) lap_pair_kernel(const float *X, int N, int n, const unsigned long long *w, int nb,
+                                                       double *R)
+{
+    __shared__ uint2 wt[PT][PT + 1];
+    __shared__ float xs[PT][PC];
+    const int I = blockIdx.x, c0 = blockIdx.y * PC;
+    const int r = threadIdx.x & (PT - 1), g = threadIdx.x >> 6;  // 4 groups of 8 coordinates
+    const int i = I * PT + r;
+    float xi[8];
+    double acc[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const int l = c0 + g * 8 + q;
+        xi[q] = (i < N && l < n) ? X[(size_t)i * n + l] : 0.f;
+        acc[q] = 0.0;
+    }
+    for (int J = 0; J < nb; ++J) {
+        __syncthreads();
+        const uint2 *tw = reinterpret_cast<const uint2 *>(w + tile_of(min(I, J), max(I, J), nb) * (PT * PT));
+        for (int idx = threadIdx.x; idx < PT * PT; idx += 256) {
+            const int a = idx / PT, b = idx % PT;  // the stored tile's row and column
+            const uint2 v = tw[idx];
+            if (I < J) wt[a][b] = v;
+            else if (I > J) wt[b][a] = v;
+            else if (a < b) { wt[a][b] = v; wt[b][a] = v; }
+            else if (a == b) wt[a][a] = make_uint2(0u, 0u);
+        }
+        for (int idx = threadIdx.x; idx < PT * PC; idx += 256) {
+            const int b = idx / PC, l = idx % PC;
+            const int j = J * PT + b;
+            xs[b][l] = (j < N && c0 + l < n) ? X[(size_t)j * n + c0 + l] : 0.f;
+        }
+        __syncthreads();
+        float hi[8], lo[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) hi[q] = lo[q] = 0.f;
+#pragma unroll 2
+        for (int b = 0; b < PT; ++b) {
+            const uint2 v = wt[r][b];
+            const float4 u0 = *reinterpret_cast<const float4 *>(&xs[b][g * 8]);
+            const float4 u1 = *reinterpret_cast<const float4 *>(&xs[b][g * 8 + 4]);
+            const float xb[8] = {u0.x, u0.y, u0.z, u0.w, u1.x, u1.y, u1.z, u1.w};
+            if ((int)v.y < 0) {
+                const float wh = __uint_as_float(v.y & 0x7fffffffu), wl = __uint_as_float(v.x);
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    float s, e;
+                    two_diff(xi[q], xb[q], s, e);
+                    const float p = __fmul_rn(wh, s);
+                    float t = fmaf(wh, s, -p);
+                    t = fmaf(wh, e, t);
+                    t = fmaf(wl, s, t);
+                    add_pair(hi[q], lo[q], p, t);
+                }
+            } else if (v.x | v.y) {
+                const double wv = __hiloint2double((int)v.y, (int)v.x);
+#pragma unroll
+                for (int q = 0; q < 8; ++q) acc[q] = fma(wv, (double)xi[q] - (double)xb[q], acc[q]);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 8; ++q) acc[q] += widen(hi[q]) + widen(lo[q]);
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const int l = c0 + g * 8 + q;
+        if (i < N && l < n) R[(size_t)i * n + l] = acc[q];
+    }
+}
+
+// Band z of C[a][b] = sum_i (x_ia - mean_a) R_ib over a 16 x 16 block of (a,
+// b): the rows are cut into bands (with all rows in one block the 49 blocks
+// of n = 100 left most SMs idle: 0.92 ms), added in order by band_sum_kernel.
+constexpr int kGramBands = 16;
 template <typename TX>
 __global__ void __launch_bounds__(256) gram_kernel(const TX *X, const double *mean, const double *R, int N, int n,
-                                                   double *C)
+                                                   double *Cp)
 {
     __shared__ double xa[32][17], rb[32][17];
     const int a0 = blockIdx.x * 16, b0 = blockIdx.y * 16;
     const int ta = threadIdx.x >> 4, tb = threadIdx.x & 15;
     double acc = 0.0;
-    for (int i0 = 0; i0 < N; i0 += 32) {
+    const int rows = (N + 32 * kGramBands - 1) / (32 * kGramBands) * 32, r1 = min(N, ((int)blockIdx.z + 1) * rows);
+    for (int i0 = blockIdx.z * rows; i0 < r1; i0 += 32) {
         __syncthreads();
         for (int idx = threadIdx.x; idx < 32 * 16; idx += 256) {
             const int q = idx / 16, c = idx % 16;
             const int i = i0 + q;
-            xa[q][c] = (i < N && a0 + c < n) ? ldx(X, (size_t)i * n + a0 + c) - mean[a0 + c] : 0.0;
-            rb[q][c] = (i < N && b0 + c < n) ? R[(size_t)i * n + b0 + c] : 0.0;
+            xa[q][c] = (i < r1 && a0 + c < n) ? ldx(X, (size_t)i * n + a0 + c) - mean[a0 + c] : 0.0;
+            rb[q][c] = (i < r1 && b0 + c < n) ? R[(size_t)i * n + b0 + c] : 0.0;
         }
         __syncthreads();
 #pragma unroll 8
         for (int q = 0; q < 32; ++q) acc = fma(xa[q][ta], rb[q][tb], acc);
     }
-    if (a0 + ta < n && b0 + tb < n) C[(size_t)(a0 + ta) * n + b0 + tb] = acc;
+    if (a0 + ta < n && b0 + tb < n) Cp[((size_t)blockIdx.z * n + a0 + ta) * n + b0 + tb] = acc;
+}
+
+__global__ void band_sum_kernel(const double *Cp, int n, double *C)
+{
+    const long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x, nn = (long long)n * n;
+    if (idx >= nn) return;
+    double acc = 0.0;
+    for (int z = 0; z < kGramBands; ++z) acc += Cp[z * nn + idx];
+    C[idx] = acc;
 }
 
 // C <- (C + C^T) / 2 (the two halves differ only by rounding).
@@ -285,14 +477,14 @@ __global__ void jacobi_norms_kernel(const double *A, int n, double *out)
 
 struct Scratch {
     double *w = nullptr, *R = nullptr, *mean = nullptr, *C = nullptr, *C2 = nullptr, *V = nullptr, *V2 = nullptr,
-           *norms = nullptr, *part = nullptr;
+           *norms = nullptr, *part = nullptr, *Cp = nullptr;
     double2 *fg = nullptr;
     int2 *tiles = nullptr;
     int *partner = nullptr;
     ~Scratch()
     {
         for (void *p : {(void *)w, (void *)R, (void *)mean, (void *)C, (void *)C2, (void *)V, (void *)V2,
-                        (void *)norms, (void *)part, (void *)fg, (void *)tiles, (void *)partner})
+                        (void *)norms, (void *)part, (void *)Cp, (void *)fg, (void *)tiles, (void *)partner})
             if (p) cudaFree(p);
     }
 };
@@ -328,25 +520,32 @@ sap_status secant_pca(sap_handle h, int k, double *U_out, double *sigma_out)
     PCK(cudaMalloc(&sc.part, colmean_scratch(N, n) * sizeof(double)));
     PCK(cudaMalloc(&sc.C, (size_t)n * n * sizeof(double)));
     PCK(cudaMalloc(&sc.C2, (size_t)n * n * sizeof(double)));
+    PCK(cudaMalloc(&sc.Cp, (size_t)kGramBands * n * n * sizeof(double)));
     PCK(cudaMalloc(&sc.V, (size_t)n * n * sizeof(double)));
     PCK(cudaMalloc(&sc.V2, (size_t)n * n * sizeof(double)));
     PCK(cudaMalloc(&sc.norms, 2 * sizeof(double)));
     PCK(cudaMalloc(&sc.fg, (size_t)n * sizeof(double2)));
     PCK(cudaMalloc(&sc.partner, (size_t)n * sizeof(int)));
     const double eps2 = handle_eps2(h);
-    const dim3 lgrid(nb, (n + PC - 1) / PC), ggrid((n + 15) / 16, (n + 15) / 16);
+    const dim3 lgrid(nb, (n + PC - 1) / PC), ggrid((n + 15) / 16, (n + 15) / 16, kGramBands);
     if (X64) {
         w64_kernel<double><<<(unsigned)ntiles, 256, 0, s>>>(X64, N, n, sc.tiles, eps2, sc.w);
         lap_rows_kernel<double><<<lgrid, 256, 0, s>>>(X64, N, n, sc.w, nb, sc.R);
         PCK(launch_colmean(X64, N, n, sc.part, sc.mean, s));
-        gram_kernel<double><<<ggrid, 256, 0, s>>>(X64, sc.mean, sc.R, N, n, sc.C);
+        gram_kernel<double><<<ggrid, 256, 0, s>>>(X64, sc.mean, sc.R, N, n, sc.Cp);
     } else {
-        w64_kernel<float><<<(unsigned)ntiles, 256, 0, s>>>(X32, N, n, sc.tiles, eps2, sc.w);
-        lap_rows_kernel<float><<<lgrid, 256, 0, s>>>(X32, N, n, sc.w, nb, sc.R);
+        std::vector<float> nu(N);
+        PCK(cudaMemcpyAsync(nu.data(), handle_nu(h), (size_t)N * sizeof(float), cudaMemcpyDeviceToHost, s));
+        PCK(cudaStreamSynchronize(s));
+        const double numax = *std::max_element(nu.begin(), nu.end());
+        unsigned long long *wp = reinterpret_cast<unsigned long long *>(sc.w);
+        w_pair_kernel<<<(unsigned)ntiles, 256, 0, s>>>(X32, N, n, sc.tiles, eps2, numax * numax / 256.0, wp);
+        lap_pair_kernel<<<lgrid, 256, 0, s>>>(X32, N, n, wp, nb, sc.R);
         PCK(launch_colmean(X32, N, n, sc.part, sc.mean, s));
-        gram_kernel<float><<<ggrid, 256, 0, s>>>(X32, sc.mean, sc.R, N, n, sc.C);
+        gram_kernel<float><<<ggrid, 256, 0, s>>>(X32, sc.mean, sc.R, N, n, sc.Cp);
     }
     PCK(cudaGetLastError());
+    band_sum_kernel<<<(unsigned)(((long long)n * n + 255) / 256), 256, 0, s>>>(sc.Cp, n, sc.C);
     symmetrize_kernel<<<(unsigned)(((long long)n * n + 255) / 256), 256, 0, s>>>(sc.C, n);
     PCK(cudaGetLastError());
     // cyclic Jacobi sweeps: A (= C) towards diag(lambda), V accumulating the

@@ -59,7 +59,8 @@ int handle_sms(sap_handle h);
 ProbState *handle_state(sap_handle h);
 const float *handle_x32(sap_handle h);
 const float *handle_u32(sap_handle h);
-int restructured_pass_grid(sap_handle h);  // blocks of the all-pairs pass
+int restructured_pass_grid(sap_handle h, bool shared);  // blocks of the all-pairs pass
+bool handle_shared(sap_handle h);  // its passes run beside other datasets' and do not all fit
 Partial *handle_partials(sap_handle h);
 double *handle_u64(sap_handle h);
 const float *handle_u32lo(sap_handle h);
@@ -95,6 +96,7 @@ struct BasisView {
     long long cap;            // capacity of each list
     const double *U64;        // n x k FP64 basis, column-major (tiers inside the pass)
     Partial *partials;        // per-block best pairs (tiers inside the pass)
+    bool shared = false;      // its pass runs beside others that together want more than all SMs
 };
 
 // Filter operands of a product: the buffer and the bases' widths.
