@@ -29,12 +29,16 @@
 #include "colmean.cuh"
 #include "../../include/sap.h"
 
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
 #include <string>
 #include <vector>
+
+namespace cg = cooperative_groups;
 
 namespace sap {
 
@@ -164,7 +168,7 @@ __global__ void __launch_bounds__(256) lap_rows_kernel(const TX *X, int N, int n
 // bound by it (12.6 ms and 39 ms at N = 8192, n = 100).  With FP32 points the
 // difference of two coordinates is an exact FP32 pair s + e, so lengths and
 // weighted differences can be formed with error-free FP32 steps (18
-// operations instead of two FP64 ones: @@ ms and @@ ms), accurate to a few
+// operations instead of two FP64 ones: 2.2 ms and 8.2 ms), accurate to a few
 // 2^-48 of the running sums.  That is enough where w = 1/d^2 is moderate; the
 // Laplacian's rounding error is carried by the short secants, whose terms (of
 // size 1/d) cancel between neighbours, so pairs with d below a sixteenth of
@@ -475,6 +479,167 @@ __global__ void jacobi_norms_kernel(const double *A, int n, double *out)
     }
 }
 
+// The whole eigensolver for n <= kClusterN in one launch: a cluster of 16
+// blocks runs the rounds behind cluster barriers (two launches per round took
+// 11 us, most of it gaps: 9 ms for the 792 rounds of n = 100).  Every block
+// computes all rotations of a round itself (no exchange) from A in L2; the
+// 2 x 2 blocks of (row pair, column pair) entries are dealt to the blocks,
+// 16 FP64 operations per four entries; V's rows stay in the blocks' shared
+// memory, since rotations combine its columns only.  The rotation of (p, q)
+// with d = a_qq - a_pp, b = a_pq comes from two reciprocal square roots: r =
+// 1/sqrt(d^2 + 4 b^2), c^2 = (1 + |d| r) / 2, s = |b| r / c, the same plane
+// rotation as the quotient form above.  Above kClusterN the matrix is large
+// enough for all SMs and the launches above.
+constexpr int kClusterN = 256;
+constexpr int kJacobiBlocks = 16;
+constexpr int kJacobiThreads = 256;
+
+__device__ __forceinline__ int2 rr_pair(int t, int r, int m, int n)
+{
+    int x, y;
+    if (t == 0) {
+        x = m - 1;
+        y = r;
+    } else {
+        x = r + t;
+        if (x >= m - 1) x -= m - 1;
+        y = r - t;
+        if (y < 0) y += m - 1;
+    }
+    const int p = min(x, y), q = max(x, y);
+    return make_int2(p, q < n ? q : -1);  // an odd n's extra index pairs with nobody
+}
+
+__global__ void __launch_bounds__(kJacobiThreads) jacobi_cluster_kernel(double *A, double *A2, double *V, int n, double tol,
+                                                                        int max_sweeps, double *out)
+{
+    extern __shared__ double vrow[];  // this block's rows of V
+    __shared__ int2 pq[kClusterN / 2];
+    __shared__ double2 cs[kClusterN / 2];
+    __shared__ double part[2], red[2][kJacobiThreads / 32];
+    cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank(), C = (int)cluster.num_blocks();
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int m = n + (n & 1), np = m / 2;
+    const int rows = (n + C - 1) / C, v0 = rank * rows, nv = max(0, min(rows, n - v0));
+    for (int idx = tid; idx < nv * n; idx += kJacobiThreads) vrow[idx] = (idx % n) == v0 + idx / n ? 1.0 : 0.0;
+    bool done = n == 1;
+    int sweep = 0;
+    for (; sweep < max_sweeps && !done; ++sweep) {
+        for (int r = 0; r < m - 1; ++r) {
+            __syncthreads();  // the previous round's rotations have been used
+            for (int t = tid; t < np; t += kJacobiThreads) {
+                const int2 x = rr_pair(t, r, m, n);
+                double2 v = make_double2(1.0, 0.0);
+                if (x.y >= 0) {
+                    const double b = __ldcg(A + (size_t)x.x * n + x.y);
+                    const double d = __ldcg(A + (size_t)x.y * n + x.y) - __ldcg(A + (size_t)x.x * n + x.x);
+                    const double h = fma(4.0 * b, b, d * d);
+                    if (b != 0.0 && h > 0.0) {
+                        const double ih = rsqrt(h);
+                        const double c2 = 0.5 * fma(fabs(d), ih, 1.0);
+                        const double ic = rsqrt(c2);
+                        double sn = fabs(b) * ih * ic, cn = c2 * ic;
+                        // one Newton step towards c^2 + s^2 = 1
+                        const double f = fma(-0.5, fma(cn, cn, fma(sn, sn, -1.0)), 1.0);
+                        cn *= f;
+                        sn *= f;
+                        v = make_double2(cn, (d >= 0.0) == (b >= 0.0) ? sn : -sn);
+                    }
+                }
+                pq[t] = x;
+                cs[t] = v;
+            }
+            __syncthreads();
+            // A2 = J^T A J: column p' = c p - s q, q' = s p + c q, rows alike
+            for (int e = rank + C * tid; e < np * np; e += C * kJacobiThreads) {
+                const int tr = e / np, tc = e - tr * np;
+                const int2 R = pq[tr], S = pq[tc];
+                const double2 jr = cs[tr], jc = cs[tc];
+                const bool hq = R.y >= 0, hs = S.y >= 0;
+                const double a00 = __ldcg(A + (size_t)R.x * n + S.x);
+                const double a01 = hs ? __ldcg(A + (size_t)R.x * n + S.y) : 0.0;
+                const double a10 = hq ? __ldcg(A + (size_t)R.y * n + S.x) : 0.0;
+                const double a11 = hq && hs ? __ldcg(A + (size_t)R.y * n + S.y) : 0.0;
+                const double b00 = fma(jc.x, a00, -(jc.y * a01)), b01 = fma(jc.y, a00, jc.x * a01);
+                const double b10 = fma(jc.x, a10, -(jc.y * a11)), b11 = fma(jc.y, a10, jc.x * a11);
+                A2[(size_t)R.x * n + S.x] = fma(jr.x, b00, -(jr.y * b10));
+                if (hs) A2[(size_t)R.x * n + S.y] = fma(jr.x, b01, -(jr.y * b11));
+                if (hq) A2[(size_t)R.y * n + S.x] = fma(jr.y, b00, jr.x * b10);
+                if (hq && hs) A2[(size_t)R.y * n + S.y] = fma(jr.y, b01, jr.x * b11);
+            }
+            for (int e = tid; e < nv * np; e += kJacobiThreads) {
+                const int i = e / np, t = e - i * np;
+                const int2 S = pq[t];
+                if (S.y < 0) continue;
+                const double2 j = cs[t];
+                const double x = vrow[i * n + S.x], y = vrow[i * n + S.y];
+                vrow[i * n + S.x] = fma(j.x, x, -(j.y * y));
+                vrow[i * n + S.y] = fma(j.y, x, j.x * y);
+            }
+            double *t2 = A;
+            A = A2;
+            A2 = t2;
+            cluster.sync();  // the round's A is complete
+        }
+        // off-diagonal and whole sums of squares, the blocks' parts added in order
+        double off = 0.0, all = 0.0;
+        for (int idx = tid; idx < nv * n; idx += kJacobiThreads) {
+            const int i = v0 + idx / n, j = idx % n;
+            const double v = __ldcg(A + (size_t)i * n + j);
+            all = fma(v, v, all);
+            if (i != j) off = fma(v, v, off);
+        }
+        off = warp_sum(off);
+        all = warp_sum(all);
+        if (lane == 0) {
+            red[0][w] = off;
+            red[1][w] = all;
+        }
+        __syncthreads();
+        if (tid == 0) {
+            double o = 0.0, a = 0.0;
+            for (int q = 0; q < kJacobiThreads / 32; ++q) {
+                o += red[0][q];
+                a += red[1][q];
+            }
+            part[0] = o;
+            part[1] = a;
+        }
+        cluster.sync();
+        double o = 0.0, a = 0.0;
+        for (int q = 0; q < C; ++q) {
+            o += *cluster.map_shared_rank(&part[0], q);
+            a += *cluster.map_shared_rank(&part[1], q);
+        }
+        done = !(o > tol * tol * a);  // the same in every block
+        cluster.sync();  // the parts have been read
+    }
+    for (int idx = tid; idx < nv * n; idx += kJacobiThreads) V[(size_t)v0 * n + idx] = vrow[idx];
+    if (rank == 0)
+        for (int i = tid; i < n; i += kJacobiThreads) out[2 + i] = __ldcg(A + (size_t)i * n + i);
+    if (rank == 0 && tid == 0) out[0] = done ? 1.0 : 0.0;
+}
+
+cudaError_t launch_jacobi_cluster(double *A, double *A2, double *V, int n, double tol, double *out, cudaStream_t s)
+{
+    cudaError_t e = cudaFuncSetAttribute(jacobi_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kJacobiBlocks);
+    cfg.blockDim = dim3(kJacobiThreads);
+    cfg.dynamicSmemBytes = (size_t)((n + kJacobiBlocks - 1) / kJacobiBlocks) * n * sizeof(double);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = kJacobiBlocks;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, jacobi_cluster_kernel, A, A2, V, n, tol, 40, out);
+}
+
 struct Scratch {
     double *w = nullptr, *R = nullptr, *mean = nullptr, *C = nullptr, *C2 = nullptr, *V = nullptr, *V2 = nullptr,
            *norms = nullptr, *part = nullptr, *Cp = nullptr;
@@ -523,7 +688,7 @@ sap_status secant_pca(sap_handle h, int k, double *U_out, double *sigma_out)
     PCK(cudaMalloc(&sc.Cp, (size_t)kGramBands * n * n * sizeof(double)));
     PCK(cudaMalloc(&sc.V, (size_t)n * n * sizeof(double)));
     PCK(cudaMalloc(&sc.V2, (size_t)n * n * sizeof(double)));
-    PCK(cudaMalloc(&sc.norms, 2 * sizeof(double)));
+    PCK(cudaMalloc(&sc.norms, (size_t)(n + 2) * sizeof(double)));
     PCK(cudaMalloc(&sc.fg, (size_t)n * sizeof(double2)));
     PCK(cudaMalloc(&sc.partner, (size_t)n * sizeof(int)));
     const double eps2 = handle_eps2(h);
@@ -550,40 +715,50 @@ sap_status secant_pca(sap_handle h, int k, double *U_out, double *sigma_out)
     PCK(cudaGetLastError());
     // cyclic Jacobi sweeps: A (= C) towards diag(lambda), V accumulating the
     // rotations (its columns become the eigenvectors)
-    const unsigned nn_blocks = (unsigned)(((long long)n * n + 255) / 256);
-    jacobi_init_kernel<<<nn_blocks, 256, 0, s>>>(sc.V, n);
-    PCK(cudaGetLastError());
-    const int m = n + (n & 1);
     double *A = sc.C, *A2 = sc.C2, *V = sc.V, *V2 = sc.V2;
-    const double u = std::ldexp(1.0, -53);
+    const double tol = 4.0 * n * std::ldexp(1.0, -53);
     bool converged = n == 1;
-    for (int sweep = 0; sweep < 40 && !converged; ++sweep) {
-        for (int r = 0; r < m - 1; ++r) {
-            jacobi_angles_kernel<<<(n + 127) / 128, 128, 0, s>>>(A, n, m, r, sc.fg, sc.partner);
-            jacobi_apply_kernel<<<nn_blocks, 256, 0, s>>>(A, V, n, sc.fg, sc.partner, A2, V2);
-            std::swap(A, A2);
-            std::swap(V, V2);
-        }
-        PCK(cudaGetLastError());
-        jacobi_norms_kernel<<<1, 1024, 0, s>>>(A, n, sc.norms);
-        double nrm[2] = {0.0, 0.0};
-        PCK(cudaMemcpyAsync(nrm, sc.norms, sizeof(nrm), cudaMemcpyDeviceToHost, s));
+    std::vector<double> lam(n), Vh((size_t)n * n);
+    if (n <= kClusterN) {
+        PCK(launch_jacobi_cluster(A, A2, V, n, tol, sc.norms, s));
+        std::vector<double> o(n + 2);
+        PCK(cudaMemcpyAsync(o.data(), sc.norms, o.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
+        PCK(cudaMemcpyAsync(Vh.data(), V, Vh.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
         PCK(cudaStreamSynchronize(s));
-        const double tol = 4.0 * n * u;
-        converged = !(nrm[0] > tol * tol * nrm[1]);
+        converged = o[0] != 0.0;
+        for (int c = 0; c < n; ++c) lam[c] = o[2 + c];
+    } else {
+        const unsigned nn_blocks = (unsigned)(((long long)n * n + 255) / 256);
+        jacobi_init_kernel<<<nn_blocks, 256, 0, s>>>(sc.V, n);
+        PCK(cudaGetLastError());
+        const int m = n + (n & 1);
+        for (int sweep = 0; sweep < 40 && !converged; ++sweep) {
+            for (int r = 0; r < m - 1; ++r) {
+                jacobi_angles_kernel<<<(n + 127) / 128, 128, 0, s>>>(A, n, m, r, sc.fg, sc.partner);
+                jacobi_apply_kernel<<<nn_blocks, 256, 0, s>>>(A, V, n, sc.fg, sc.partner, A2, V2);
+                std::swap(A, A2);
+                std::swap(V, V2);
+            }
+            PCK(cudaGetLastError());
+            jacobi_norms_kernel<<<1, 1024, 0, s>>>(A, n, sc.norms);
+            double nrm[2] = {0.0, 0.0};
+            PCK(cudaMemcpyAsync(nrm, sc.norms, sizeof(nrm), cudaMemcpyDeviceToHost, s));
+            PCK(cudaStreamSynchronize(s));
+            converged = !(nrm[0] > tol * tol * nrm[1]);
+        }
+        std::vector<double> Ah((size_t)n * n);
+        PCK(cudaMemcpyAsync(Ah.data(), A, Ah.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
+        PCK(cudaMemcpyAsync(Vh.data(), V, Vh.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
+        PCK(cudaStreamSynchronize(s));
+        for (int c = 0; c < n; ++c) lam[c] = Ah[(size_t)c * n + c];
     }
     if (!converged) return handle_fail(h, SAP_E_CUDA, "Jacobi eigensolver did not converge in 40 sweeps");
-    PCK(cudaStreamSynchronize(s));  // the copies below run on the legacy stream
-    // the k largest eigenvalues (diagonal of A) and their columns of V,
-    // largest first; each vector signed so that its entry of largest
-    // magnitude is positive
-    std::vector<double> Ah((size_t)n * n), Vh((size_t)n * n);
-    PCK(cudaMemcpy(Ah.data(), A, Ah.size() * sizeof(double), cudaMemcpyDeviceToHost));
-    PCK(cudaMemcpy(Vh.data(), V, Vh.size() * sizeof(double), cudaMemcpyDeviceToHost));
+    // the k largest eigenvalues and their columns of V, largest first; each
+    // vector signed so that its entry of largest magnitude is positive
     std::vector<int> order(n);
     for (int c = 0; c < n; ++c) order[c] = c;
     std::stable_sort(order.begin(), order.end(),
-                     [&](int a, int b) { return Ah[(size_t)a * n + a] > Ah[(size_t)b * n + b]; });
+                     [&](int a, int b) { return lam[a] > lam[b]; });
     for (int c = 0; c < k; ++c) {
         const int col = order[c];
         int am = 0;
@@ -591,7 +766,7 @@ sap_status secant_pca(sap_handle h, int k, double *U_out, double *sigma_out)
             if (std::fabs(Vh[(size_t)l * n + col]) > std::fabs(Vh[(size_t)am * n + col])) am = l;
         const double sg = Vh[(size_t)am * n + col] < 0 ? -1.0 : 1.0;
         for (int l = 0; l < n; ++l) U_out[(size_t)c * n + l] = sg * Vh[(size_t)l * n + col];
-        if (sigma_out) sigma_out[c] = std::sqrt(std::max(Ah[(size_t)col * n + col], 0.0));
+        if (sigma_out) sigma_out[c] = std::sqrt(std::max(lam[col], 0.0));
     }
     return SAP_OK;
 #undef PCK
