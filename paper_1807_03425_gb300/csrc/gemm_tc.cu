@@ -333,7 +333,7 @@ size_t gemm_smem_bytes(int KPG, int stages)
 
 // Ring depth: up to 4 stages, but where the grid does not fit one CTA per SM
 // few enough that two CTAs share one (156 CTAs at N = 19939 were a second
-// wave of four: @@ -> @@ us).
+// wave of four: 12.4 -> 9.5 us).
 int gemm_pick_stages(int KPG, int nkb, int ctas, int sms)
 {
     int s = 4;

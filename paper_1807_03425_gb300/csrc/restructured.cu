@@ -343,6 +343,14 @@ struct PassArgs {
     int n_near = 0;
     Partial *partials = nullptr;
     Cert cert32;
+    // double-float tier (no X): the stored FP32 w narrows the emission, and
+    // the near pairs that Y cannot rule out go to a list of their own
+    const float *w32 = nullptr;   // FP32 1/d^2 tiles (row-major 128 x 128)
+    int nb = 0;                   // point blocks per side
+    long long tile0 = 0;          // global index of the first stored tile
+    float rho32 = 0.f;            // relative error with the FP32 w
+    int2 *near_out = nullptr;     // near_cap entries; st->cntn counts all
+    int near_cap = 0;
 };
 
 // One ring stage: the BF16 1/d^2 tile (32 KB), the row block's A image and
@@ -662,7 +670,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) restr_pass_kernel(const __gri
     const int nearG = (int)gridDim.x * kConsumerWarps, near0 = (int)blockIdx.x * kConsumerWarps + warp;
     int2 npr = make_int2(0, 0);
     float nw = INFINITY;
-    if (EXPL && near0 + lane * nearG < a.n_near) {
+    if (near0 + lane * nearG < a.n_near) {
         npr = __ldcg(a.near + near0 + lane * nearG);
         nw = __ldcg(a.near_w + near0 + lane * nearG);
     }
@@ -780,7 +788,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) restr_pass_kernel(const __gri
     // The near pairs, one per lane: their ratio from Y with their own (large)
     // bound rules most of them out in O(k); it also bounds the minimum.
     auto near_pairs = [&]() {
-        if constexpr (EXPL) {
+        {
             for (long long base = 0; base < a.n_near; base += 32ll * nearG) {
                 const long long idx = base + near0 + (long long)lane * nearG;
                 int2 pr = npr;
@@ -794,12 +802,20 @@ __global__ void __launch_bounds__(kPassThreads, 1) restr_pass_kernel(const __gri
                         const float *yi = a.Y + (size_t)(pr.x >> 7) * a.Ykt * T + (pr.x & (T - 1));
                         const float *yj = a.Y + (size_t)(pr.y >> 7) * a.Ykt * T + (pr.y & (T - 1));
                         float zz = 0.f;
+                        if constexpr (EXPL) {
 #pragma unroll
-                        for (int c = 0; c < K; ++c)
-                            if (c < k) {
+                            for (int c = 0; c < K; ++c)
+                                if (c < k) {
+                                    const float e = __ldcg(yi + c * T) - __ldcg(yj + c * T);
+                                    zz = fmaf(e, e, zz);
+                                }
+                        } else {
+#pragma unroll 8
+                            for (int c = 0; c < k; ++c) {
                                 const float e = __ldcg(yi + c * T) - __ldcg(yj + c * T);
                                 zz = fmaf(e, e, zz);
                             }
+                        }
                         if (nw < INFINITY) {
                             const float r = sqrt_up(zz * nw);
                             const float b = pair_bound(a.beta, __ldg(a.nu + pr.x), __ldg(a.nu + pr.y), nw);
@@ -813,11 +829,21 @@ __global__ void __launch_bounds__(kPassThreads, 1) restr_pass_kernel(const __gri
                 ub = warp_min(ub);
                 const float U = bound_now();
                 if (ub < U) lower_bound_to(ub);
-                append(pr.x, pr.y, lo, lo <= fminf(U, ub) * 1.000001f && lo < INFINITY);
+                const bool keep = lo <= fminf(U, ub) * 1.000001f && lo < INFINITY;
+                if constexpr (EXPL) {
+                    append(pr.x, pr.y, lo, keep);
+                } else {
+                    const unsigned int m = __ballot_sync(0xffffffffu, keep);
+                    if (!m) continue;
+                    unsigned int at = 0;
+                    if (lane == 0) at = atomicAdd((unsigned int *)&a.st->cntn, (unsigned int)__popc(m));
+                    at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & ((1u << lane) - 1u));
+                    if (keep && at < (unsigned int)a.near_cap) a.near_out[at] = pr;
+                }
             }
         }
     };
-    near_pairs();  // while the first stages' copies land
+    if (EXPL) near_pairs();  // while the first stages' copies land
     // ring position and barrier phases, advanced without integer division
     int s = 0;
     uint32_t phase = 0;
@@ -886,6 +912,9 @@ __global__ void __launch_bounds__(kPassThreads, 1) restr_pass_kernel(const __gri
         const float *gI = a.Y + (size_t)IJ.x * a.Ykt * T, *gJ = a.Y + (size_t)IJ.y * a.Ykt * T;
         const uint16_t *hs = reinterpret_cast<const uint16_t *>(stage);
         const float *nuI = reinterpret_cast<const float *>(stage + o_nu), *nuJ = nuI + T;
+        const float *w32t = nullptr;  // the tile's FP32 w
+        if (!EXPL && a.w32)
+            w32t = a.w32 + ((long long)IJ.x * a.nb - (long long)IJ.x * (IJ.x - 1) / 2 + (IJ.y - IJ.x) - a.tile0) * (T * T);
         // r~^2 of pair (r, c), its w in w
         auto pair_q = [&](int r, int c, float &w) {
             w = __uint_as_float((uint32_t)hs[((c >> 3) * T + r) * 8 + (c & 7)] << 16) * wsc;
@@ -924,6 +953,11 @@ __global__ void __launch_bounds__(kPassThreads, 1) restr_pass_kernel(const __gri
                 float w;
                 const float r = sqrt_up(pair_q(row, pcol, w));
                 if (r < U) ub = (r + pair_bound(a.beta, nuI[row], nuJ[pcol], w)) * inv_up;
+                if (!EXPL && w32t && ub < INFINITY) {
+                    const float w32 = __ldg(w32t + row * T + pcol);
+                    ub = fminf(ub, (r * sqrt_up(w32 / w) + pair_bound(a.beta, nuI[row], nuJ[pcol], w)) *
+                                       (1.000003f / (1.0f - a.rho32)));
+                }
             }
             ub = __shfl_sync(0xffffffffu, ub, src);
             if (ub < U) {
@@ -972,10 +1006,18 @@ __global__ void __launch_bounds__(kPassThreads, 1) restr_pass_kernel(const __gri
                 const int e = __ffs(flag) - 1;
                 flag &= flag - 1u;
                 float w;
-                const float q = pair_q(row, col0 + e, w);
+                float q = pair_q(row, col0 + e, w);
                 if (q <= thc2) {
-                    const float th = (ut + pair_bound(a.beta, nuI[row], nuJ[col0 + e], w)) * 1.000001f;
-                    if (q <= th * th * 1.000001f) emit |= 1u << e;
+                    const float bp = pair_bound(a.beta, nuI[row], nuJ[col0 + e], w);
+                    float th = (ut + bp) * 1.000001f;
+                    if (q > th * th * 1.000001f) continue;
+                    if (w32t) {
+                        // the FP32 w: an eighth of the BF16 rounding's window
+                        q = q / w * __ldg(w32t + row * T + col0 + e);
+                        th = (U * (1.0f + a.rho32) + bp) * 1.000002f;
+                        if (q > th * th * 1.000001f) continue;
+                    }
+                    emit |= 1u << e;
                 }
             }
             const int cnt = __popc(emit);
@@ -999,6 +1041,15 @@ __global__ void __launch_bounds__(kPassThreads, 1) restr_pass_kernel(const __gri
                 else atomicOr(&a.st->status, ST_OVERFLOW);
                 ++pos;
             }
+        }
+    }
+    if constexpr (!EXPL) {
+        if (a.n_near > 0) {
+            // the near pairs against the grid's bound, now tight
+            if (lane == 0) atomicMin(&sub, __float_as_uint(load_pos_float(&a.st->run_ub1)));
+            __syncwarp();
+            near_pairs();
+            if (lane == 0) atomic_min_pos_float(&a.st->run_ub1, bound_now());
         }
     }
     if constexpr (EXPL) {
@@ -1446,7 +1497,23 @@ struct YdfArgs {
     int Npad;
     float *Yh, *Yl;          // KY x Npad each, component-major; rows >= N zero
     int KY;
+    // pair mode (st set, no more than pair_max pairs left by the pass)
+    ProbState *st = nullptr;
+    long long pair_max = -1;
+    const int2 *cand1 = nullptr, *near_list = nullptr;
+    Cert cert;               // of the extended-precision explicit evaluation
+    int k = 0;
+    unsigned long long *cand2 = nullptr;
+    long long cap2 = 0;
 };
+
+// The pass left few pairs: they are evaluated one by one (pair mode) and the
+// whole double-float Y is not needed.
+__device__ __forceinline__ bool pair_mode(const ProbState *st, long long pair_max)
+{
+    const long long c = (long long)*(volatile const unsigned int *)&st->cnt1 + *(volatile const unsigned int *)&st->cntn;
+    return c <= pair_max;
+}
 
 __device__ __forceinline__ void df_merge_norm(float &hi, float &lo, float h2, float l2)
 {
@@ -1457,6 +1524,14 @@ __device__ __forceinline__ void df_merge_norm(float &hi, float &lo, float h2, fl
     lo = __fsub_rn(l, __fsub_rn(hi, s));
 }
 
+// Pair mode: a Y row costs n k error-free steps whether or not a candidate
+// needs it, and N rows for a basis are 4 GFLOP of FP32 steps at N = n = 4096, k =
+// 20 (0.3-0.5 ms beside the other bases' kernels); a pair costs n (k + 1).
+// With fewer pairs than points a warp takes a pair instead, its differences
+// in place of the row's coordinates and |D|^2 as one more component, and emits
+// what the bound does not exclude for the FP64 tier (the error model of the
+// extended-precision explicit tier).
+//
 // A block of 16 warps computes 32 rows at a time, two per warp; the lanes of
 // a warp split the coordinates (l = lane, lane + 32, ...), and their partial
 // sums are merged by a 5-level shuffle tree at the end (within the error
@@ -1478,6 +1553,71 @@ __global__ void __launch_bounds__(kYdfWarps * 32) ydf_warp_kernel(YdfArgs a)
     __shared__ float us[2 * K][CH];  // [c][l] hi, [K + c][l] lo
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nchunks = (a.n + CH - 1) / CH;
+    if (a.st && pair_mode(a.st, a.pair_max)) {
+        const int cn = *(volatile const int *)&a.st->cntn, total = *(volatile const int *)&a.st->cnt1 + cn;
+        const float seed = load_pos_float(&a.st->seed_ub);
+        for (int pbase = blockIdx.x * kYdfWarps; pbase < total; pbase += gridDim.x * kYdfWarps) {
+            const int p = pbase + warp;
+            int2 pr = make_int2(0, 0);
+            bool valid = p < total;
+            if (valid) {
+                pr = p < cn ? __ldcg(a.near_list + p) : __ldcg(a.cand1 + (p - cn));
+                valid = SAP_PAIR_OK(a.st, pr, a.N);
+                if (!valid) pr = make_int2(0, 0);
+            }
+            const float *xi = a.X + (size_t)pr.x * a.n, *xj = a.X + (size_t)pr.y * a.n;
+            float hi[K + 1], lo[K + 1];
+#pragma unroll
+            for (int c = 0; c <= K; ++c) hi[c] = lo[c] = 0.f;
+            for (int ch = 0; ch < nchunks; ++ch) {
+                const int c0 = ch * CH, nc = min(CH, a.n - c0);
+                __syncthreads();
+                for (int idx = threadIdx.x; idx < K * CH; idx += kYdfWarps * 32) {
+                    const int c = idx / CH, l = idx % CH;
+                    const bool in = l < nc;
+                    us[c][l] = in ? a.U32[(size_t)(c0 + l) * a.KP + c] : 0.f;
+                    us[K + c][l] = in ? a.U32lo[(size_t)(c0 + l) * a.KP + c] : 0.f;
+                }
+                __syncthreads();
+                if (valid)
+#pragma unroll 2
+                    for (int l = lane; l < nc; l += 32) {
+                        const float D = xi[c0 + l] - xj[c0 + l];
+#pragma unroll
+                        for (int c = 0; c < K; ++c) df_step(hi[c], lo[c], D, us[c][l], us[K + c][l]);
+                        df_step(hi[K], lo[K], D, D, 0.f);
+                    }
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                for (int c = 0; c <= K; ++c) {
+                    const float h2 = __shfl_xor_sync(0xffffffffu, hi[c], o);
+                    const float l2 = __shfl_xor_sync(0xffffffffu, lo[c], o);
+                    df_merge_norm(hi[c], lo[c], h2, l2);
+                }
+            if (lane == 0 && valid) {
+                const float dd = hi[K];
+                float zz = 0.f;
+#pragma unroll
+                for (int c = 0; c < K; ++c) zz = fmaf(hi[c], hi[c], zz);
+                float lb = 0.f;  // too short for FP32: the FP64 tier decides
+                float U = fminf(seed, fminf(load_pos_float(&a.st->run_ub1), load_pos_float(&a.st->run_ub2)));
+                if (!(dd < 1e-30f)) {
+                    const float rr = sqrtf(zz / dd), ub = cert_upper(rr, a.cert);
+                    if (ub < U) atomic_min_pos_float(&a.st->run_ub2, ub);
+                    U = fminf(U, ub);
+                    lb = fmaxf((rr - a.cert.A) / (1.0f + a.cert.rho) * 0.999998f, 0.f);
+                }
+                if (lb <= U * 1.000001f) {
+                    const unsigned int at = atomicAdd((unsigned int *)&a.st->cnt2, 1u);
+                    if ((long long)at < a.cap2) a.cand2[at] = pack_cand(pr.x, pr.y, lb, lb == 0.f);
+                    else atomicOr(&a.st->status, ST_OVERFLOW);
+                }
+            }
+        }
+        return;
+    }
     for (int rbase = blockIdx.x * (kYdfWarps * kYdfRpw); rbase < a.Npad;
          rbase += gridDim.x * (kYdfWarps * kYdfRpw)) {
         float hi[kYdfRpw][K], lo[kYdfRpw][K];
@@ -1551,6 +1691,7 @@ struct RefineArgs {
     unsigned long long *cand2;  // packed (i, j, lower bound of the ratio)
     long long cap2;
     int pdl;
+    long long pair_max;      // the double-float kernel took the pairs itself up to this many
 };
 
 // One thread per pair; K = compute width (Y's pad components are zero).
@@ -1559,19 +1700,16 @@ template <int K>
 __global__ void __launch_bounds__(256) refine_kernel(RefineArgs a)
 {
     const int lane = threadIdx.x & 31;
-    const float seed = load_pos_float(&a.st->seed_ub);
     const float rho = a.cert.rho;
-    // With programmatic launch the near list is evaluated first (it needs
-    // only the previous iteration's results), the pass's candidates after
-    // the wait; otherwise one range covers both.
-    for (int seg = 0; seg < (a.pdl ? 2 : 1); ++seg) {
+    grid_dep_wait();
+    grid_dep_launch();
+    if (pair_mode(a.st, a.pair_max)) return;
+    const float seed = load_pos_float(&a.st->seed_ub);
+    {
         long long nn = a.n_near, total = a.n_near;
-        if (seg == 1 || !a.pdl) {
-            grid_dep_wait();
-            grid_dep_launch();
+        {
             unsigned int c1 = *(volatile const unsigned int *)&a.st->cnt1;
             if (c1 > a.cap1) c1 = a.cap1;
-            nn = a.pdl ? 0 : a.n_near;
             total = nn + c1;
         }
         const long long stride = (long long)gridDim.x * blockDim.x;
@@ -1768,6 +1906,14 @@ Cert cert_pass(int n, int k, double b_cap)
     // rest as for explicit differences
     c.rho = (float)((std::ldexp(1.0, -9) + g(n + 2) + g(k) + 8 * u) * 1.05);
     return c;
+}
+
+// Relative error of the pass's ratios with the FP32 w in place of the BF16 one.
+float cert_pass32(int n, int k)
+{
+    const double u = std::ldexp(1.0, -24);
+    auto g = [&](double m) { return m * u / (1.0 - m * u); };
+    return (float)((g(n + 2) + g(k) + 8 * u) * 1.05);
 }
 
 // Extended-precision tier: 2^-24 absolute from the rounding of D (U
@@ -2021,6 +2167,8 @@ sap_status restructured_basis_alloc(sap_handle h)
     const size_t op_bytes = (size_t)(r.Npad / T) * 2 * op_image_bytes(k);
     RCK(cudaMalloc(&r.ops, op_bytes));
     RCK(cudaMemsetAsync(r.ops, 0, op_bytes, s));  // pad halves stay zero
+    dfree(r.near_list);
+    RCK(cudaMalloc(&r.near_list, (size_t)handle_n_points(h) * sizeof(int2)));
     dfree(r.Ydh);
     dfree(r.Ydl);
     RCK(cudaMalloc(&r.Ydh, (size_t)r.Npad * r.KY * sizeof(float)));
@@ -2164,12 +2312,25 @@ sap_status restructured_enqueue_basis(sap_handle h, const BasisView &b, cudaStre
             p.partials = b.partials;
             p.cert32 = cert_explicit(n, b.k);
         }
+        if (tier == 1 && b.near_list) {
+            p.N = (int)handle_n_points(h);
+            p.near = r.near;
+            p.near_w = r.near_w;
+            p.n_near = r.n_near;
+            p.near_out = b.near_list;
+            p.near_cap = (int)handle_n_points(h);
+            p.w32 = r.w;
+            p.nb = r.Npad / T;
+            p.tile0 = r.tile0;
+            p.rho32 = cert_pass32(n, b.k);
+        }
         handle_count_launch(h, 1, &ea, &eb);
         if (ea) cudaEventRecord(ea, s);
         RCK(launch_pass(p, restructured_pass_grid(h, b.shared), s));
         if (eb) cudaEventRecord(eb, s);
         handle_push_timing(h, 1, ea, eb);
     }
+    const long long pair_max = tier == 1 && b.k <= 24 && b.near_list ? handle_n_points(h) : -1;
     if (tier == 2 || tier == 3 || tier == 5) {
         // the explicit tier runs inside the FP64 recheck (restructured_fuse_args)
         // or (5) inside the pass
@@ -2211,7 +2372,16 @@ sap_status restructured_enqueue_basis(sap_handle h, const BasisView &b, cudaStre
         y.Yh = b.Ydh;
         y.Yl = b.Ydl;
         y.KY = b.KY;
+        y.st = b.st;
+        y.pair_max = pair_max;
+        y.cand1 = b.cand1;
+        y.near_list = b.near_list;
+        y.cert = cert_explicit_df(n, b.k);
+        y.k = b.k;
+        y.cand2 = reinterpret_cast<unsigned long long *>(b.cand2);
+        y.cap2 = b.cap;
         RefineArgs x;
+        x.pair_max = pair_max;
         x.Yh = b.Ydh;
         x.Yl = b.Ydl;
         x.Npad = r.Npad;
@@ -2266,6 +2436,7 @@ sap_status restructured_enqueue(sap_handle h, double alpha)
     b.ops = r.ops;
     b.ops_stride = 2 * op_image_bytes(b.k);
     b.shared = handle_shared(h);
+    b.near_list = r.near_list;
     b.Ydh = r.Ydh;
     b.Ydl = r.Ydl;
     b.st = handle_state(h);
@@ -2381,8 +2552,7 @@ int restructured_tier(sap_handle h) { return restructured_tier_for(h, handle_k(h
 // takes every SM it can use.  Beside other passes that together want more
 // than the SMs there are, blocks of fewer than about 8 tiles would mostly
 // serialise those fixed costs: 16 scenes of 500..12000 points took 246 us per
-// iteration with a block per tile and @@ us with at least 8 tiles each, the 20
-// bases of a sweep over 4096 points @@ and @@ us.
+// iteration with a block per tile and 205 us with at least 8 tiles each.
 int restructured_pass_grid(sap_handle h, bool shared)
 {
     const int t = restr_state(h).nwtiles, sms = handle_sms(h);
@@ -2448,7 +2618,7 @@ void restructured_free(sap_handle h)
     RestrState &r = restr_state(h);
     dfree(r.Xhi); dfree(r.Xlo); dfree(r.center); dfree(r.colpart); dfree(r.nu); dfree(r.w); dfree(r.wtiles);
     dfree(r.near); dfree(r.counters); dfree(r.Uhi); dfree(r.Ulo); dfree(r.Y); dfree(r.ops); dfree(r.Ypart);
-    dfree(r.near_w); dfree(r.xn); dfree(r.Ydh); dfree(r.Ydl); dfree(r.wb);
+    dfree(r.near_w); dfree(r.near_list); dfree(r.xn); dfree(r.Ydh); dfree(r.Ydl); dfree(r.wb);
 }
 
 void restructured_stats(sap_handle h, sap_stats *out)

@@ -44,6 +44,7 @@ struct RestrState {
     float *Y = nullptr;       // block-major [Npad/128][KY][128]
     unsigned char *ops = nullptr;  // the pass's filter operands: per 128-point block, A and B images
     float yscale = 1.f;       // power of two: |y| * yscale <= 64 for any orthonormal basis
+    int2 *near_list = nullptr;  // near pairs the pass could not rule out (N entries)
     float *Ydh = nullptr, *Ydl = nullptr;  // double-float Y of the refine tier, KY x Npad each
     int KY = 0;               // k rounded up to 4
     int ksplit = 1;           // K slices of the product (shorter accumulation chains)
@@ -96,6 +97,7 @@ struct BasisView {
     long long cap;            // capacity of each list
     const double *U64;        // n x k FP64 basis, column-major (tiers inside the pass)
     Partial *partials;        // per-block best pairs (tiers inside the pass)
+    int2 *near_list = nullptr; // near pairs the pass could not rule out (N entries)
     bool shared = false;      // its pass runs beside others that together want more than all SMs
 };
 

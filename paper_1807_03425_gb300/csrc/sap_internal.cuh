@@ -123,6 +123,7 @@ struct ProbState {
     unsigned int run_ub2;   // float bits: running upper bound, explicit recheck
     int cnt1;               // entries emitted by the all-pairs pass
     int cnt2;               // entries emitted by the explicit recheck
+    int cntn;               // near pairs the pass could not rule out (double-float tier)
     int iter;               // evaluations recorded in the history
     int status;             // StatusBits
     int watch_n;            // filled entries of watch[]

@@ -613,7 +613,9 @@ __global__ void __launch_bounds__(SB) select_update_kernel(SelectUpdateArgs a)
             // pair that can still be the argmin under the final running bound
             // is evaluated (the tier emitted against earlier, looser values)
             float th = INFINITY;
-            if (packed) th = cert_emit_threshold(fminf(load_pos_float(&st->seed_ub), load_pos_float(&st->run_ub2)), a.cert2);
+            if (packed)
+                th = cert_emit_threshold(fminf(load_pos_float(&st->seed_ub), fminf(load_pos_float(&st->run_ub1), load_pos_float(&st->run_ub2))),
+                                         a.cert2);
             bool by_block = false;
             if constexpr (sizeof(TX) == 4) by_block = n > kSliceN;
             if (by_block) {
@@ -756,6 +758,7 @@ __global__ void __launch_bounds__(SB) select_update_kernel(SelectUpdateArgs a)
             st->cnt1 = 0;
             st->tile_next = 0;
             st->cnt2 = 0;
+            st->cntn = 0;
             st->ticket = 0;
             st->run_ub1 = 0x7f800000u;
             st->run_ub2 = 0x7f800000u;
@@ -782,6 +785,7 @@ __global__ void __launch_bounds__(SB) select_update_kernel(SelectUpdateArgs a)
         st->cnt1 = 0;
         st->tile_next = 0;
         st->cnt2 = 0;
+            st->cntn = 0;
         st->ticket = 0;
         st->run_ub1 = 0x7f800000u;
         st->run_ub2 = 0x7f800000u;

@@ -125,6 +125,7 @@ sap_status alloc_impl(sap_handle h, SweepState *&swp, int kmax, int hist_need)
         WCK(cudaMemsetAsync(b.U32lo, 0, (size_t)n * b.KP * sizeof(float), s0));
         WCK(cudaMalloc(&b.work, (size_t)(kMaxK + 1) * n * sizeof(double)));
         WCK(cudaMalloc(&b.st, sizeof(ProbState)));
+        WCK(cudaMalloc(&b.near_list, (size_t)N * sizeof(int2)));
         WCK(cudaMalloc(&b.cand1, (size_t)sw.cap * sizeof(int2)));
         WCK(cudaMalloc(&b.cand2, (size_t)sw.cap * sizeof(int2)));
         WCK(cudaMalloc(&b.partials, (size_t)kRecheckBlocks * sizeof(Partial)));
@@ -241,6 +242,7 @@ sap_status enqueue_iteration(sap_handle h, SweepState &sw, double alpha, int eva
         v.cap = sw.cap;
         v.U64 = b.U64;
         v.partials = b.partials;
+        v.near_list = b.near_list;
         v.shared = sweep_shared(h, sw);
         st = restructured_enqueue_basis(h, v, b.stream);
         if (st != SAP_OK) return st;
@@ -409,7 +411,7 @@ void sweep_free(SweepState *&s)
     s->graphs.clear();
     for (SweepBasis &b : s->b) {
         wfree(b.U64); wfree(b.U32); wfree(b.U32lo); wfree(b.work); wfree(b.st); wfree(b.Ydh); wfree(b.Ydl);
-        wfree(b.cand1); wfree(b.cand2); wfree(b.partials); wfree(b.hist); wfree(b.am);
+        wfree(b.cand1); wfree(b.near_list); wfree(b.cand2); wfree(b.partials); wfree(b.hist); wfree(b.am);
         if (b.stream) cudaStreamDestroy(b.stream);
         if (b.done) cudaEventDestroy(b.done);
     }

@@ -18,7 +18,7 @@ struct SweepBasis {
     float *U32 = nullptr, *U32lo = nullptr;
     double *work = nullptr;
     ProbState *st = nullptr;
-    int2 *cand1 = nullptr, *cand2 = nullptr;
+    int2 *cand1 = nullptr, *cand2 = nullptr, *near_list = nullptr;
     Partial *partials = nullptr;
     double *hist = nullptr;
     int2 *am = nullptr;
