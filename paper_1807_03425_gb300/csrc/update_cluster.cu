@@ -107,7 +107,7 @@ __global__ void __launch_bounds__(UB, 1) update_cluster_kernel(SelectUpdateArgs 
     float *Qs = reinterpret_cast<float *>(smb + Lay::o_Q);
     float *rows = reinterpret_cast<float *>(smb + Lay::o_rows);
     __shared__ float red[UW * (K + 1)];
-    __shared__ float cvec[K + 1], cw[K];
+    __shared__ float cvec[K + 1], cw[K], qd[K + 1];
     __shared__ Partial best_sh;
     __shared__ int2 watch[kWatch];
     __shared__ int watch_n, watch_pos, iter, hist_cap, cnt1, cnt2, alive0_sh;
@@ -249,20 +249,21 @@ __global__ void __launch_bounds__(UB, 1) update_cluster_kernel(SelectUpdateArgs 
 
     // ---- 3-4. pivot, modified Gram-Schmidt on [c, e_l (l != t)] and the
     // rotation coefficients: warp 0, lane m holding vector m
+    // (a direction travels from its lane through shared memory: as K shuffles
+    // per step this section took 42 K of the kernel's 71 K cycles at n = 200,
+    // k = 10; now 17 K)
     if (w == 0) {
         const float d = sqrtf(cvec[K]);
-        float x[K];
-        float r2 = 0.f, cmax = -1.f;
+        if (lane < K) cw[lane] = lane < kk ? cvec[lane] / d : 0.f;
+        __syncwarp();
+        float x[K], r2 = 0.f, cmax = -1.f;
         int t = 0;
 #pragma unroll
         for (int q = 0; q < K; ++q) {
-            x[q] = q < kk ? cvec[q] / d : 0.f;
+            x[q] = cw[q];
             r2 = fmaf(x[q], x[q], r2);
             if (q < kk && fabsf(x[q]) > cmax) { cmax = fabsf(x[q]); t = q; }
         }
-        if (lane == 0)
-#pragma unroll
-            for (int q = 0; q < K; ++q) cw[q] = x[q];
         if (lane != 0) {
             const int lm = (lane - 1) < t ? (lane - 1) : lane;  // list entry m >= 1 is column lm
 #pragma unroll
@@ -270,23 +271,26 @@ __global__ void __launch_bounds__(UB, 1) update_cluster_kernel(SelectUpdateArgs 
         }
 #pragma unroll 1
         for (int p = 0; p < kk; ++p) {
-            float nn = 0.f;
-#pragma unroll
-            for (int q = 0; q < K; ++q) nn = fmaf(x[q], x[q], nn);
-            const bool alive = nn > 0.f;
             if (lane == p) {
+                float nn = 0.f;
+#pragma unroll
+                for (int q = 0; q < K; ++q) nn = fmaf(x[q], x[q], nn);
+                const bool alive = nn > 0.f;
                 const float inv = alive ? 1.f / sqrtf(nn) : 0.f;
 #pragma unroll
-                for (int q = 0; q < K; ++q) x[q] = x[q] * inv;
+                for (int q = 0; q < K; ++q) qd[q] = x[q] = x[q] * inv;
+                qd[K] = alive ? 1.f : 0.f;
                 if (p == 0) alive0_sh = alive ? 1 : 0;
             }
-            if (!__shfl_sync(0xffffffffu, alive ? 1 : 0, p)) continue;
-            float h = 0.f, qp[K];
+            __syncwarp();
+            float qp[K], h = 0.f;
 #pragma unroll
-            for (int q = 0; q < K; ++q) {
-                qp[q] = __shfl_sync(0xffffffffu, x[q], p);
-                h = fmaf(qp[q], x[q], h);
-            }
+            for (int q = 0; q < K; ++q) qp[q] = qd[q];
+            const bool alive = qd[K] != 0.f;  // the same in every lane
+            __syncwarp();                     // read before the next step writes
+            if (!alive) continue;
+#pragma unroll
+            for (int q = 0; q < K; ++q) h = fmaf(qp[q], x[q], h);
             if (lane > p)
 #pragma unroll
                 for (int q = 0; q < K; ++q) x[q] = fmaf(-h, qp[q], x[q]);
@@ -532,59 +536,55 @@ __global__ void __launch_bounds__(UB, 1) update_cluster_kernel(SelectUpdateArgs 
     __syncthreads();
 
     // ---- 6. the block's rows of U'', in every form the kernels read
+    // (one entry per thread and turn, lanes over rows: a row per thread left
+    // most threads idle, 12.6 K cycles at n = 200, k = 10; now 2.4 K)
     const double s00 = small ? G[0] : 0.0;
 #pragma unroll 1
-    for (int r = tid; r < nr; r += UB) {
-        const int l = l0 + r;
-        float *row = rows + (size_t)r * KS;
-        float x[K];
-#pragma unroll
-        for (int p = 0; p < K; ++p) x[p] = p < kk ? row[p] : 0.f;
-#pragma unroll 1
-        for (int m = 0; m < kk; ++m) {
-            double s;
-            if (small) {
-                if (m == 0) {
-                    s = widen(x[0]) * s00;
-                } else {
-                    // x_m + sum_p x_p S_pm: two chains of error-free steps
-                    float h0 = 0.f, e0 = 0.f, h1 = 0.f, e1 = 0.f;
-#pragma unroll
-                    for (int p = 0; p < K; p += 2) {
-                        if (p <= m) xs_fma(h0, e0, x[p], Shi[p * K + m], Slo[p * K + m]);
-                        if (p + 1 < K && p + 1 <= m) xs_fma(h1, e1, x[p + 1], Shi[(p + 1) * K + m], Slo[(p + 1) * K + m]);
-                    }
-                    float hs, es;
-                    xs_two_sum(h0, h1, hs, es);
-                    es = __fadd_rn(es, __fadd_rn(e0, e1));
-                    s = widen(row[m]) + (widen(hs) + widen(es));
-                }
+    for (int e = tid; e < nr * kk; e += UB) {
+        const int m = e / nr, r = e - m * nr, l = l0 + r;
+        const float *row = rows + (size_t)r * KS;
+        double s;
+        float hi = 0.f, rest = 0.f;  // x_m + correction as an FP32 pair (when available)
+        if (small && m > 0) {
+            // x_m + sum_p x_p S_pm: two chains of error-free steps
+            float h0 = 0.f, e0 = 0.f, h1 = 0.f, e1 = 0.f;
+#pragma unroll 2
+            for (int p = 0; p <= m; p += 2) {
+                xs_fma(h0, e0, row[p], Shi[p * K + m], Slo[p * K + m]);
+                if (p + 1 <= m) xs_fma(h1, e1, row[p + 1], Shi[(p + 1) * K + m], Slo[(p + 1) * K + m]);
+            }
+            float hs, es;
+            xs_two_sum(h0, h1, hs, es);
+            es = __fadd_rn(es, __fadd_rn(e0, e1));
+            s = widen(row[m]) + (widen(hs) + widen(es));
+            xs_two_sum(row[m], hs, hi, rest);
+            rest = __fadd_rn(rest, es);
+        } else if (small) {
+            s = widen(row[0]) * s00;
+        } else {
+            s = 0.0;
+            for (int p = 0; p <= m; ++p) s = fma(widen(row[p]), Ri[p * K + m], s);
+        }
+        a.U64[(size_t)m * n + l] = s;
+        const float sf = (float)s;
+        a.U32[(size_t)l * a.KP + m] = sf;
+        // the residual from the FP32 pair where sf is its high part (FP64
+        // operations are the scarce resource here)
+        if (a.U32lo) a.U32lo[(size_t)l * a.KP + m] = (small && m > 0 && sf == hi) ? rest : (float)(s - (double)sf);
+        if (a.Uhi) {
+            // hi + lo * 2^-s of the FP32 value (the FP32 rounding adds 2^-24
+            // relative to the split residual)
+            const size_t idx = (size_t)m * a.NP + l;
+            if (a.split_bf16) {
+                const __nv_bfloat16 h = __float2bfloat16_rn(sf);
+                static_cast<__nv_bfloat16 *>(a.Uhi)[idx] = h;
+                static_cast<__nv_bfloat16 *>(a.Ulo)[idx] =
+                    __float2bfloat16_rn((sf - __bfloat162float(h)) * a.split_scale);
             } else {
-                s = 0.0;
-#pragma unroll
-                for (int p = 0; p < K; ++p)
-                    if (p <= m) s = fma(widen(x[p]), Ri[p * K + m], s);
+                const __half h = __float2half_rn(sf);
+                static_cast<__half *>(a.Uhi)[idx] = h;
+                static_cast<__half *>(a.Ulo)[idx] = __float2half_rn((sf - __half2float(h)) * a.split_scale);
             }
-            a.U64[(size_t)m * n + l] = s;
-            const float sf = (float)s;
-            a.U32[(size_t)l * a.KP + m] = sf;
-            if (a.U32lo) a.U32lo[(size_t)l * a.KP + m] = (float)(s - (double)sf);
-            if (a.Uhi) {
-                // hi + lo * 2^-s of the FP32 value (the FP32 rounding adds 2^-24
-                // relative to the split residual)
-                const size_t idx = (size_t)m * a.NP + l;
-                if (a.split_bf16) {
-                    const __nv_bfloat16 h = __float2bfloat16_rn(sf);
-                    static_cast<__nv_bfloat16 *>(a.Uhi)[idx] = h;
-                    static_cast<__nv_bfloat16 *>(a.Ulo)[idx] =
-                        __float2bfloat16_rn((sf - __bfloat162float(h)) * a.split_scale);
-                } else {
-                    const __half h = __float2half_rn(sf);
-                    static_cast<__half *>(a.Uhi)[idx] = h;
-                    static_cast<__half *>(a.Ulo)[idx] = __float2half_rn((sf - __half2float(h)) * a.split_scale);
-                }
-            }
-            row[m] = sf;  // for the seeds (x holds the old row)
         }
     }
     if (a.seeds_in_product) {
@@ -605,11 +605,16 @@ __global__ void __launch_bounds__(UB, 1) update_cluster_kernel(SelectUpdateArgs 
             const float *wi = X + (size_t)pr.x * n + l0, *wj = X + (size_t)pr.y * n + l0;
             for (int r = lane; r < nr; r += 32) {
                 const float D = wi[r] - wj[r];
-                const float *row = rows + (size_t)r * KS;
+                const float *row = a.U32 + (size_t)(l0 + r) * a.KP;  // written by this block above
                 v[K] = fmaf(D, D, v[K]);
 #pragma unroll
-                for (int c = 0; c < K; ++c)
-                    if (c < kk) v[c] = fmaf(row[c], D, v[c]);
+                for (int c = 0; c < KP4; c += 4) {
+                    const float4 u = __ldcg(reinterpret_cast<const float4 *>(row + c));
+                    v[c] = fmaf(u.x, D, v[c]);
+                    if (c + 1 < K) v[c + 1 < K ? c + 1 : 0] = fmaf(u.y, D, v[c + 1 < K ? c + 1 : 0]);
+                    if (c + 2 < K) v[c + 2 < K ? c + 2 : 0] = fmaf(u.z, D, v[c + 2 < K ? c + 2 : 0]);
+                    if (c + 3 < K) v[c + 3 < K ? c + 3 : 0] = fmaf(u.w, D, v[c + 3 < K ? c + 3 : 0]);
+                }
             }
         }
         warp_sum_multi<float, K + 1>(v);
