@@ -49,8 +49,8 @@ CFG_NAME = "c2"
 # DRAM traffic of one restructured-pass launch from the ncu capture of this
 # kernel on this workload, valid only while the pass kernel's source is
 # unchanged (hash below, kernel_source_sha).
-PASS_TRAFFIC_BYTES = 71932416   # 71.120 MB read + 0.812 MB written
-PASS_SOURCE_SHA = "774558e356117a0b"
+PASS_TRAFFIC_BYTES = 70184960   # 69.627 MB read + 0.558 MB written
+PASS_SOURCE_SHA = "0296d2d8edf7f5d2"
 
 
 def kernel_source_sha() -> str:
@@ -1010,7 +1010,7 @@ def run_pca(args):
     fp64_flops = 2.0 * P * n * 2 + 2.0 * N * n * n  # Laplacian rows (both halves) + Xc^T R
     line = _common(args, cfg["workload"] + "_secant_pca", 1.0 / wall, "PCA starts/s", 1e3 * wall, reps, 1, "f64",
                    {"N": N, "n": n, "k": k, "alpha": alpha,
-                    "l2": "FP64 lengths 268 MB (larger than L2), written once and read by every row block"})
+                    "l2": "inverse lengths 268 MB (8 B per pair, larger than L2), written once and read by every row block"})
     line.update({
         "seconds_per_start": wall,
         "singular_values": [float(v) for v in sv],
@@ -1020,10 +1020,11 @@ def run_pca(args):
             "naive_first_three_coordinates": r_naive, "pca_start": r_epca, "sap_100_from_pca": float(he[-1]),
             "paper_printed": {"naive": 0.1013, "pca": 0.0466, "sap_100": 0.1677},
             "closed_form_naive_limit": 1.0 / np.sqrt(55.0)},
-        "roofline": {"kernel": "Laplacian rows + Gram (FP64)", "bound": "fp64",
+        "roofline": {"kernel": "lengths, Laplacian rows (FP32 pairs) + Gram (FP64)", "bound": "alu",
                      "achieved": fp64_flops / wall / 1e12, "unit": "TFLOP/s", "peak": None, "frac": None,
                      "traffic": None,
-                     "note": "whole start incl. the Jacobi eigensolver; FP64 rate of this part measured near 1.0 TFLOP/s"},
+                     "note": "whole start incl. the Jacobi eigensolver, counted in FP64 operations; the lengths and the "
+                             "Laplacian run as pairs of FP32 numbers (FP64 rate of this part: near 1.0 TFLOP/s)"},
         "e2e": {"value": 1.0 / wall, "unit": "PCA starts/s", "h2d_bytes_per_step": 0,
                 "d2h_bytes_per_step": n * k * 8},
     })

@@ -161,16 +161,17 @@ sap_status sap_set_basis(sap_handle h, const double *U, int32_t k,
  * (distinct points, Sec. II; d >= eps after sap_set_min_secant_length,
  * Sec. VII), i.e. the eigenvectors of S S^T = sum_{i<j} s s^T with the k
  * largest eigenvalues, each signed so that its entry of largest magnitude is
- * positive.  S S^T is formed in FP64 on the device as Xc^T L X (L the
- * 1/d^2-weighted graph Laplacian of the pairs, lengths from explicit FP64
- * differences), never storing S; the n x n symmetric eigenproblem is solved
+ * positive.  S S^T is formed on the device as Xc^T L X (L the 1/d^2-weighted
+ * graph Laplacian of the pairs, lengths from explicit differences; FP64, for
+ * FP32 and BF16 data the lengths and L X as pairs of FP32 numbers with
+ * error-free products and sums), never storing S; the n x n symmetric eigenproblem is solved
  * on the device by the cyclic Jacobi method in FP64 (round-robin parallel
  * ordering, sweeps until the off-diagonal norm is below 4 n 2^-53 of the
  * whole; SAP_E_CUDA if 40 sweeps do not get there).  U_out (nullable, host, n x k
  * column-major) receives the basis, sigma_out (nullable, k) the singular
  * values sqrt(lambda) in descending order.  1 <= k <= min(n, 32).  Resets
  * the iteration counter, like sap_set_basis.  Work memory: 8 B per pair
- * (the FP64 lengths) plus 8 N n + 8 n^2 bytes, freed before returning.
+ * (the lengths) plus 8 N n + 160 n^2 bytes, freed before returning.
  * Synchronises.
  */
 sap_status sap_secant_pca(sap_handle h, int32_t k, double *U_out, double *sigma_out);
@@ -384,12 +385,12 @@ typedef struct {
                                        fused into the FP64 recheck (one launch fewer; k <= 8, else
                                        as 0), 4 explicit differences in extended precision whose
                                        list carries each pair's ratio, so the FP64 recheck takes
-                                       only the pairs within the final bound, 5 explicit
-                                       differences in extended precision inside the all-pairs
-                                       pass: each emitted pair, and each near pair, is rechecked
-                                       at once by the warp that found it, and evaluated in FP64
-                                       there if it can still be the argmin; one block then takes
-                                       the argmin and updates (two launches fewer, no lists;
+                                       only the pairs within the final bound, 5 inside the
+                                       all-pairs pass: the pairs it emits and the near pairs wait
+                                       with their block, and those that can still be the argmin
+                                       when its tiles are done are evaluated there in FP64 (first
+                                       from explicit FP32 differences where they are many); the
+                                       update then takes the argmin (two launches fewer, no lists;
                                        k <= 16, else as 0), -1 chosen by n and k (double-float
                                        above n = 256, else 5 for k <= 16, else 0) */
     double us_per_iteration;        /* measured by sap_autotune; 0 when set by hand */

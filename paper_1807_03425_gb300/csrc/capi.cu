@@ -4,8 +4,10 @@
 //
 // One iteration (Algorithm 1 of Kvinge et al., arXiv:1807.03425):
 //   plain form:         plain pass -> FP64 recheck -> update
-//   restructured form:  Y = X U (tensor cores) -> restructured pass ->
-//                       explicit-difference recheck -> FP64 recheck -> update
+//   restructured form:  Y = X U (tensor cores) -> restructured pass, with the
+//                       second and FP64 tiers inside it (n <= 256, k <= 16)
+//                       -> update; otherwise second tier -> FP64 recheck ->
+//                       update
 // Nothing returns to the host inside the loop; sap_run replays captured
 // graphs of `chunk` iterations.
 #include "sap_internal.cuh"

@@ -16,7 +16,10 @@
 // issues TMA loads of 64-wide K blocks (128-byte swizzle) into a ring of
 // shared-memory stages; warp 1 lane 0 issues the MMAs (M = 128, N = KPG,
 // K = 16 per instruction) and releases each stage with tcgen05.commit; after
-// the last commit all four warps read their 32 TMEM lanes and write Y.
+// the last commit all four warps read their 32 TMEM lanes and write Y. Where
+// the all-pairs pass follows, the same epilogue rounds each row's components
+// to the 16-bit operand images of the pass's filter (gemm_tc.cuh): the pass
+// reads them with plain bulk copies and Y is not read again to build them.
 #include "sap_internal.cuh"
 #include "tc_ptx.cuh"
 #include "gemm_tc.cuh"

@@ -4,7 +4,7 @@
 //     r_ij^2 = ||y_i - y_j||^2 * w_ij,   w_ij = 1 / ||x_i - x_j||^2.
 // The lengths are computed once per dataset (and threshold eps, Sec. VII)
 // from explicit FP32 differences; each iteration then costs one tensor-core
-// product and one pass over the stored w (4 bytes per pair).
+// product and one pass over the stored w (2 bytes per pair: BF16).
 //
 // Precision.  The rows of Y carry absolute errors of order eps_Y ||x - mean||
 // (split-operand product, FP32 accumulation), so y_i - y_j cancels for close
@@ -14,12 +14,13 @@
 // pass skips them (w = NaN) and every iteration re-evaluates them from
 // explicit differences instead.  All other pairs are certified to within the
 // cap, so the pass emits every pair that can still be the argmin (selection
-// scheme of sap_internal.cuh); the explicit-difference tier narrows the list
-// and the FP64 tier decides.
+// scheme of sap_internal.cuh); a second tier narrows them and the FP64 tier
+// decides (for n <= 256 and k <= 16 both inside the pass, restr_pass_kernel).
 //
 // Layout.  w is stored tile-major over the upper triangle: tile t = (I, J),
-// I <= J, holds the 128 x 128 pairs (I*128 + a, J*128 + b) row-major at
-// w + t*128*128; entries with i >= j, with an index beyond N, excluded pairs
+// I <= J, holds the 128 x 128 pairs (I*128 + a, J*128 + b) at t*128*128 --
+// the FP32 w row-major, the BF16 w that the pass streams in groups of 8
+// columns, the order its consumers read --; entries with i >= j, with an index beyond N, excluded pairs
 // and near pairs hold NaN.
 #include "restructured.cuh"
 #include "colmean.cuh"
@@ -323,13 +324,12 @@ struct PassArgs {
     int pdl;
     int k = 0;
     // second and third tiers inside the pass (non-null X; k <= 16): the
-    // near pairs that Y cannot rule out and every emitted pair are evaluated
-    // by the warp that holds them, from explicit FP32 differences (the
-    // explicit tier's arithmetic and error model, cert32), which tightens
-    // the bounds; the survivors wait in the warp's list and, once its tiles
-    // are done, those that can still be the argmin under the bound as it is
-    // then are evaluated in FP64 (the FP64 recheck's arithmetic).  Every
-    // block leaves its best (q = r^2, i, j) in partials[blockIdx.x] for the
+    // near pairs that Y cannot rule out and every emitted pair wait in their
+    // warp's list; once its tiles are done, those that can still be the
+    // argmin under the bound as it is then are evaluated, where many are left
+    // first from explicit FP32 differences (the explicit tier's arithmetic
+    // and error model, cert32), the survivors in FP64 (the FP64 recheck's
+    // arithmetic).  Every block leaves its best (q = r^2, i, j) in partials[blockIdx.x] for the
     // update.  No list is written; st->cnt1 counts the emitted pairs,
     // st->cnt2 the FP64 evaluations.
     const float *X = nullptr;  // N x n FP32 points

@@ -1,6 +1,8 @@
 // select_update.cu -- the FP64 argmin over the certified candidate list and
 // the basis update of one SAP iteration (Algorithm 1 and Sec. IV of Kvinge
-// et al., arXiv:1807.03425), fused into one launch.
+// et al., arXiv:1807.03425), fused into one launch.  For FP32 and BF16 data
+// with k > 8 or n > 128 only phase 1 runs here (or nothing, after a pass that
+// holds the FP64 tier): the update is update_cluster.cu's.
 //
 // Phase 1 (all blocks): one warp per candidate forms the explicit FP64
 // difference D = x_i - x_j, d^2 = |D|^2 and z = U^T D, applies the exclusion

@@ -6,8 +6,8 @@
 // so that list is a superset of each smaller k's).  One iteration is one
 // tensor-core product Y = X [U_1 .. U_kmax] for all bases at once (their
 // padded widths sum to 256 at k_max = 20: a single MMA N), then, per basis
-// and on its own stream, the all-pairs pass, the explicit-difference tier
-// and the FP64 recheck fused with the update.  A chunk of iterations is
+// and on its own stream, the all-pairs pass, its second tier, the FP64
+// recheck and the update (sap_internal.cuh, launch_select_update).  A chunk of iterations is
 // captured once as a CUDA graph with one branch per basis and replayed;
 // the bases' chains overlap on the GPU.
 #include "sweep.cuh"
