@@ -168,7 +168,7 @@ __global__ void __launch_bounds__(256) lap_rows_kernel(const TX *X, int N, int n
 // bound by it (12.6 ms and 39 ms at N = 8192, n = 100).  With FP32 points the
 // difference of two coordinates is an exact FP32 pair s + e, so lengths and
 // weighted differences can be formed with error-free FP32 steps (18
-// operations instead of two FP64 ones: 2.2 ms and 8.2 ms), accurate to a few
+// operations instead of two FP64 ones: 2.2 ms and 7.2 ms), accurate to a few
 // 2^-48 of the running sums.  That is enough where w = 1/d^2 is moderate; the
 // Laplacian's rounding error is carried by the short secants, whose terms (of
 // size 1/d) cancel between neighbours, so pairs with d below a sixteenth of
@@ -269,8 +269,13 @@ __global__ void __launch_bounds__(256) w_pair_kernel(const float *X, int N, int 
 }
 
 // R_i as in lap_rows_kernel: the FP32 pairs' sums over one block of columns,
-// then added in FP64 (partial sums stay small, so their 2^-48 do too).
-__global__ void __launch_bounds__(256) lap_pair_kernel(const float *X, int N, int n, const unsigned long long *w, int nb,
+// then added in FP64 (partial sums stay small, so their 2^-48 do too).  Warps
+// whose coordinates are padding only stage (n = 100: 3 of 16 groups of 8), and
+// three blocks per SM instead of two (80 registers) let the blocks of the
+// last coordinates run beside the others: 8.2 -> 7.2 ms at N = 8192, n = 100
+// (the whole start 13.7 with two blocks per SM, 13.4 with three, 14.1 with
+// four, which spill).
+__global__ void __launch_bounds__(256, 3) lap_pair_kernel(const float *X, int N, int n, const unsigned long long *w, int nb,
                                                        double *R)
 {
     __shared__ uint2 wt[PT][PT + 1];
@@ -306,6 +311,7 @@ __global__ void __launch_bounds__(256) lap_pair_kernel(const float *X, int N, in
         float hi[8], lo[8];
 #pragma unroll
         for (int q = 0; q < 8; ++q) hi[q] = lo[q] = 0.f;
+        if (c0 + g * 8 >= n) continue;  // only padding
 #pragma unroll 2
         for (int b = 0; b < PT; ++b) {
             const uint2 v = wt[r][b];
