@@ -787,7 +787,7 @@ __global__ void __launch_bounds__(SB) select_update_kernel(SelectUpdateArgs a)
         st->cnt1 = 0;
         st->tile_next = 0;
         st->cnt2 = 0;
-            st->cntn = 0;
+        st->cntn = 0;
         st->ticket = 0;
         st->run_ub1 = 0x7f800000u;
         st->run_ub2 = 0x7f800000u;

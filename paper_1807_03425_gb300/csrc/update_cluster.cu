@@ -27,10 +27,11 @@
 //     product with S (as FP32 hi + lo) is formed with error-free FP32 steps,
 //     accurate to 2^-46 |S| -- far below the FP64 rounding of U'' -- and two
 //     FP64 additions per entry remain instead of k.
-// Measured against the one-block update it replaces: 67 -> 20 us at n = 224,
-// k = 10 (alone on the GPU); 1705 -> 106 us at n = 4096, k = 17..20, 1201 ->
-// 81 us at k = 13..16 and 618 -> 70 us at k = 9..12 (averages inside the
-// dimension sweep, beside the other bases' kernels).
+// Measured against the one-block update it replaces: 67 -> 16.5 us at n =
+// 224, k = 10 (alone on the GPU); 1705 -> 129 us at n = 4096, k = 17..20,
+// 1201 -> 92 us at k = 13..16 and 618 -> 66 us at k = 9..12 (averages inside
+// the dimension sweep, beside the other bases' kernels, which have become
+// shorter and overlap them more than when the first form took 106, 81 and 70).
 #include "update_cluster.cuh"
 
 #include <cooperative_groups.h>
