@@ -1065,7 +1065,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) restr_pass_kernel(const __gri
         if (direct && warp < k)
 #pragma unroll
             for (int t = 0; t < kSliceN / 32; ++t)
-                ur[t] = lane + 32 * t < a.n ? __ldg(a.U64 + (size_t)warp * a.n + lane + 32 * t) : 0.0;
+                ur[t] = lane + 32 * t < a.n ? __ldcg(a.U64 + (size_t)warp * a.n + lane + 32 * t) : 0.0;
         meet();
         if (warp == 0 && lane == 0) {
             const float g = load_pos_float(&a.st->run_ub1), mine = bound_now();

@@ -295,11 +295,20 @@ __device__ __forceinline__ void warp_ratio_parts(double (&v)[K + 1], int lane, d
 constexpr int kSliceN = 256;
 constexpr int kFp64Slices = 8;
 
+// RO: called from a kernel that may be resident (programmatic launch) while
+// the previous update still writes the basis.  The points never change, so
+// they may come through the non-coherent path; the basis is read from the L2.
 template <typename TX, bool RO>
 __device__ __forceinline__ double ld_fp64(const TX *p)
 {
     if constexpr (RO) return (double)__ldg(p);
     return (double)*p;
+}
+template <bool RO>
+__device__ __forceinline__ double ld_basis(const double *p)
+{
+    if constexpr (RO) return __ldcg(p);
+    return *p;
 }
 
 // One slice's warp totals: lane L returns the total of entry rs_index<S>(L)
@@ -317,7 +326,7 @@ __device__ __forceinline__ double fp64_slice(const TX *xi, const TX *xj, const d
         v[K] = fma(D, D, v[K]);
 #pragma unroll
         for (int c = 0; c < K; ++c)
-            if (c < k) v[c] = fma(ld_fp64<double, RO>(U64 + (size_t)c * n + l), D, v[c]);
+            if (c < k) v[c] = fma(ld_basis<RO>(U64 + (size_t)c * n + l), D, v[c]);
     }
     constexpr int M = K + 1;
     constexpr int S = M <= 8 ? 8 : M <= 16 ? 16 : 32;
@@ -348,7 +357,7 @@ __device__ __forceinline__ void fp64_pair_parts(const TX *X, const double *U64, 
             v[K] = fma(D, D, v[K]);
 #pragma unroll
             for (int c = 0; c < K; ++c)
-                if (c < k) v[c] = fma(ld_fp64<double, RO>(U64 + (size_t)c * n + l), D, v[c]);
+                if (c < k) v[c] = fma(ld_basis<RO>(U64 + (size_t)c * n + l), D, v[c]);
         }
         warp_ratio_parts<K>(v, lane, zz, d2);
         return;
@@ -430,7 +439,7 @@ __device__ __forceinline__ double fp64_entry(const double *D, const double *U64,
     for (int s = 0; s < slices; ++s) {
         double v = 0.0;
 #pragma unroll 4
-        for (int l = 32 * s + lane; l < n; l += 32 * slices) v = fma(c < k ? ld_fp64<double, RO>(u + l) : D[l], D[l], v);
+        for (int l = 32 * s + lane; l < n; l += 32 * slices) v = fma(c < k ? ld_basis<RO>(u + l) : D[l], D[l], v);
         v = warp_sum(v);
         t = slices == 1 ? v : t + v;
     }
