@@ -82,6 +82,7 @@ struct sap_ctx {
     int2 *cand1 = nullptr, *cand2 = nullptr;
     long long cap = 0;
     Partial *partials = nullptr;
+    std::vector<double> basis_host;  // source of the basis's upload, kept while the copy may read it
     long long *pack = nullptr;   // results gathered for one copy to the host
     size_t pack_cap = 0;
     RunView *views = nullptr;    // batch: the datasets' result buffers
@@ -1045,9 +1046,13 @@ sap_status sap_set_basis(sap_handle h, const double *U, int32_t k, int u_is_devi
             if (s != SAP_OK) return s;
         }
     }
-    // one copy (staged by the runtime before it returns), then every other
-    // form and the reset state by one kernel
-    CK(cudaMemcpyAsync(h->U64, Uh.data(), Uh.size() * sizeof(double), cudaMemcpyHostToDevice, h->stream));
+    // one copy, then every other form and the reset state by one kernel.  The
+    // copy may read its source after this call has returned (a pageable one is
+    // not always staged first): the handle keeps it, and the next call waits
+    // for the stream, above, before it replaces it.
+    h->basis_host.swap(Uh);
+    CK(cudaMemcpyAsync(h->U64, h->basis_host.data(), h->basis_host.size() * sizeof(double), cudaMemcpyHostToDevice,
+                       h->stream));
     CK(basis_forms(h, h->U64, true));
     if (h->dt != SAP_F64) {
         sap_status s = restructured_basis_changed(h);

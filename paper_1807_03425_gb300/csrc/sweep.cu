@@ -344,10 +344,12 @@ sap_status sweep_run(sap_handle h, const double *U0, int kmax, int iters, double
     st = restructured_classify(h, kmax);
     if (st != SAP_OK) return st;
     st = upload(h, sw, U0);
-    if (st != SAP_OK) return st;
-    st = run_graph(h, sw, alpha, 0, iters);
+    if (st == SAP_OK) st = run_graph(h, sw, alpha, 0, iters);
     if (st == SAP_OK) st = run_graph(h, sw, 0.0, 1, 1);
-    if (st != SAP_OK) return st;
+    if (st != SAP_OK) {
+        cudaStreamSynchronize(s0);  // the upload may still read the caller's U0
+        return st;
+    }
     // every basis's status and final ratio (and the product's status) in one
     // copy
     std::vector<RunView> views(kmax + 1);
