@@ -239,7 +239,7 @@ sap_status sync_and_status(sap_handle h)
     int status = 0;
     CK(cudaMemcpy(&status, &h->st->status, sizeof(int), cudaMemcpyDeviceToHost));
     if (status) {
-        CK(cudaMemset(&h->st->status, 0, sizeof(int)));
+        CK(cudaMemsetAsync(&h->st->status, 0, sizeof(int), h->stream));
         return status_error(h, status);
     }
     return SAP_OK;
@@ -390,7 +390,8 @@ sap_status ensure_hist(sap_handle h, int need)
     CK(dalloc(&h->hist, cap));
     CK(dalloc(&h->am, cap));
     h->hist_cap = cap;
-    CK(cudaMemcpy(&h->st->hist_cap, &cap, sizeof(int), cudaMemcpyHostToDevice));
+    CK(cudaMemcpyAsync(&h->st->hist_cap, &cap, sizeof(int), cudaMemcpyHostToDevice, h->stream));
+    CK(cudaStreamSynchronize(h->stream));
     return SAP_OK;
 }
 
@@ -424,7 +425,8 @@ sap_status build_tiles(sap_handle h, int edge)
         for (int J = I; J < nb; ++J) t.push_back(make_int2(I, J));
     dfree(h->tiles);
     CK(dalloc(&h->tiles, t.size()));
-    CK(cudaMemcpy(h->tiles, t.data(), t.size() * sizeof(int2), cudaMemcpyHostToDevice));
+    CK(cudaMemcpyAsync(h->tiles, t.data(), t.size() * sizeof(int2), cudaMemcpyHostToDevice, h->stream));
+    CK(cudaStreamSynchronize(h->stream));
     h->ntiles = (int)t.size();
     return SAP_OK;
 }
@@ -671,6 +673,7 @@ static sap_status create_impl(const void *X, int64_t N, int32_t n, sap_dtype dt,
             uint16_t *tmp = nullptr;
             chk(dalloc(&tmp, cnt));
             if (st == SAP_OK) chk(cudaMemcpy(tmp, X, cnt * sizeof(uint16_t), kind));
+            if (st == SAP_OK) chk(cudaStreamSynchronize(cudaStreamLegacy));
             if (st == SAP_OK) {
                 bf16_to_f32_kernel<<<4 * h->sms, 256, 0, h->stream>>>(tmp, h->X32, cnt);
                 chk(cudaGetLastError());
@@ -680,6 +683,9 @@ static sap_status create_impl(const void *X, int64_t N, int32_t n, sap_dtype dt,
         }
         h->path = SAP_RESTRUCTURED;
     }
+    // X comes by the legacy stream, in order with the caller's work there; the
+    // handle's non-blocking stream does not wait for it by itself
+    if (st == SAP_OK) chk(cudaStreamSynchronize(cudaStreamLegacy));
     const long long P = (long long)N * (N - 1) / 2;
     h->cap = std::min<long long>(P + 64, 1ll << 26);
     chk(dalloc(&h->cand1, (size_t)h->cap));

@@ -2087,7 +2087,8 @@ sap_status restructured_prepare(sap_handle h)
         r.tile0 = t0;
         r.nwtiles = (int)t.size();
         RCK(cudaMalloc(&r.wtiles, t.size() * sizeof(int2)));
-        RCK(cudaMemcpy(r.wtiles, t.data(), t.size() * sizeof(int2), cudaMemcpyHostToDevice));
+        RCK(cudaMemcpyAsync(r.wtiles, t.data(), t.size() * sizeof(int2), cudaMemcpyHostToDevice, s));
+        RCK(cudaStreamSynchronize(s));
         RCK(cudaMalloc(&r.w, (size_t)r.nwtiles * T * T * sizeof(float)));
         RCK(cudaMalloc(&r.wb, (size_t)r.nwtiles * T * T * sizeof(uint16_t)));
         const long long P = (long long)N * (N - 1) / 2;

@@ -1205,9 +1205,7 @@ sap_status ensure_buffers(sap_handle h, bool need_bwd)
         SCK(cudaMalloc(&ss.Yl, (size_t)k * r.Npad * sizeof(float)));
         SCK(cudaMalloc(&ss.G, (size_t)k * n * sizeof(double)));
         SCK(cudaMalloc(&ss.dev, sizeof(SoftDev)));
-        SoftDev d;
-        std::memset(&d, 0, sizeof(d));
-        SCK(cudaMemcpy(ss.dev, &d, sizeof(d), cudaMemcpyHostToDevice));
+        SCK(cudaMemsetAsync(ss.dev, 0, sizeof(SoftDev), handle_stream(h)));
         ss.k = k;
         ss.grid_far = std::min(r.nwtiles, sms);
         ss.n_near = -1;
@@ -1426,10 +1424,11 @@ sap_status softmin_ascent(sap_handle h, double tau, double eta, int steps, doubl
         SCK(cudaMalloc(&ss.hist, (size_t)cap * sizeof(double)));
         ss.hist_cap = cap;
     }
-    SoftDev d;
-    std::memset(&d, 0, sizeof(d));
-    d.hist_cap = ss.hist_cap;
-    SCK(cudaMemcpy(ss.dev, &d, sizeof(d), cudaMemcpyHostToDevice));
+    // on the handle's stream, ahead of the kernels that read it (a copy on the
+    // legacy stream is not ordered with a non-blocking stream's kernels)
+    ss.init = SoftDev{};
+    ss.init.hist_cap = ss.hist_cap;
+    SCK(cudaMemcpyAsync(ss.dev, &ss.init, sizeof(SoftDev), cudaMemcpyHostToDevice, s));
     // one step = forward (records L), backward, update; captured once and
     // replayed `steps` times
     if (steps > 0 && handle_profiling(h)) {
@@ -1470,6 +1469,7 @@ sap_status softmin_ascent(sap_handle h, double tau, double eta, int steps, doubl
     // the value at the final basis
     st = enqueue_forward(h, tau, true);
     if (st != SAP_OK) return st;
+    SoftDev d;
     st = read_dev(h, &d);
     if (st != SAP_OK) return st;
     if (hist) SCK(cudaMemcpy(hist, ss.hist, (size_t)(steps + 1) * sizeof(double), cudaMemcpyDeviceToHost));

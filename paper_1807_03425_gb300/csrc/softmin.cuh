@@ -35,6 +35,7 @@ struct SoftState {
     int gp_cap = 0;
     double *G = nullptr;        // k x n (the n x k column-major gradient)
     SoftDev *dev = nullptr;
+    SoftDev init = {};          // source of dev's initial value, kept while the copy may read it
     double *hist = nullptr;
     int hist_cap = 0;
     int grid_far = 0;           // persistent pass grid
