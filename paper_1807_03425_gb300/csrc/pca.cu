@@ -245,8 +245,11 @@ __global__ void __launch_bounds__(256) w_pair_kernel(const float *X, int N, int 
                 double d = (double)hi[p][q] + (double)lo[p][q];
                 const bool far_ = d >= d2cut;
                 // short secants, the threshold's neighbourhood (the exclusion
-                // is decided in FP64) and lengths outside FP32's safe range
-                if (!far_ || !(hi[p][q] < 1e30f) || fabs(d - eps2) <= 1e-9 * eps2) {
+                // is decided in FP64) and lengths outside FP32's safe range:
+                // squares overflow above it, and below it their residuals are
+                // subnormal (each off by up to 2^-149: n 2^-149 / d^2 stays
+                // below 2^-50 down to d^2 = 1e-25 at the largest n, 16384)
+                if (!far_ || !(hi[p][q] > 1e-25f && hi[p][q] < 1e30f) || fabs(d - eps2) <= 1e-9 * eps2) {
                     d = 0.0;
                     for (int l = 0; l < n; ++l) {
                         const double D = (double)X[(size_t)i * n + l] - (double)X[(size_t)j * n + l];
