@@ -171,10 +171,25 @@ __global__ void __launch_bounds__(256) lap_rows_kernel(const TX *X, int N, int n
 // operations instead of two FP64 ones: 2.2 ms and 7.2 ms), accurate to a few
 // 2^-48 of the running sums.  That is enough where w = 1/d^2 is moderate; the
 // Laplacian's rounding error is carried by the short secants, whose terms (of
-// size 1/d) cancel between neighbours, so pairs with d below a sixteenth of
-// the largest ||x - mean|| keep FP64 arithmetic throughout.  Measured against
-// 64 bits the vectors' and values' errors are those of the FP64 form (the
-// short secants' rounding dominates both).
+// size 1/d) cancel between neighbours: a rounding of R_i reaches S S^T times
+// x_i, so the pairs whose d is below a sixteenth of the larger of their own
+// ||x - mean|| keep FP64 arithmetic throughout.  (A cut against the largest
+// norm of all points let one point a hundred times farther out make every
+// secant short: 87 ms instead of 13.)  Measured against the
+// compensated sum of the secants' outer products, over ten families of curves
+// and scenes (700 to 8192 points, n = 8 .. 160, 4 to 10 draws each), the
+// vectors' errors are 0.4 to 1.1 times those of the FP64 form (geometric means
+// of the largest entry; 8.1e-14 against 7.8e-14 at N = 8192, n = 100, where
+// both come from the product with Xc), the values' 0.2 to 1.2 times.
+// N = 8192, n = 100, whole start, FP64 form -> this: a smooth curve 62.2 ->
+// 13.4 ms, with one point a hundred times farther out 62.3 -> 13.4, fifty
+// tight clusters 65.3 -> 43.9, two tight clusters 62.2 -> 50.4.
+//
+// The FP64 operations of the short secants: the difference of two FP32
+// numbers is an exact FP32 sum and remainder, widened by integer operations,
+// so a term takes one FP64 addition and one multiply-add (one multiply-add
+// where the difference is exact in FP32, as it is for close numbers), not
+// more than the FP64 kernels above take.
 //
 // A pair's 8 bytes hold either the FP64 w (sign bit 0; 0.0: excluded) or,
 // sign bit 1, the FP32 pair: -wh in the high word, wl in the low one.
@@ -194,8 +209,16 @@ __device__ __forceinline__ void add_pair(float &hi, float &lo, float p, float pe
     lo = __fadd_rn(lo, __fadd_rn(e, pe));
 }
 
+// x - y in FP64 from the two_diff parts (an overflow of the FP32 difference
+// takes the conversions).
+__device__ __forceinline__ double diff64(float x, float y, float s, float e)
+{
+    if (!(fabsf(s) < INFINITY)) return (double)x - (double)y;
+    return e == 0.f ? widen(s) : widen(s) + widen(e);
+}
+
 __global__ void __launch_bounds__(256) w_pair_kernel(const float *X, int N, int n, const int2 *tiles, double eps2,
-                                                     double d2cut, unsigned long long *w)
+                                                     const float *nu, unsigned long long *w)
 {
     __shared__ float xi[PC][PT + 4], xj[PC][PT + 4];
     const int2 IJ = tiles[blockIdx.x];
@@ -235,6 +258,12 @@ __global__ void __launch_bounds__(256) w_pair_kernel(const float *X, int N, int 
         }
     }
     unsigned long long *out = w + (size_t)blockIdx.x * PT * PT;
+    float nui[4], nuj[4];
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+        nui[p] = nu[min(i0 + tr * 4 + p, N - 1)];
+        nuj[p] = nu[min(j0 + tc * 4 + p, N - 1)];
+    }
 #pragma unroll
     for (int p = 0; p < 4; ++p)
 #pragma unroll
@@ -243,7 +272,10 @@ __global__ void __launch_bounds__(256) w_pair_kernel(const float *X, int N, int 
             unsigned long long v = 0ull;
             if (i < j && j < N) {
                 double d = (double)hi[p][q] + (double)lo[p][q];
-                const bool far_ = d >= d2cut;
+                // d >= max(nu_i, nu_j) / 16; the square overflows or underflows
+                // only outside the range below
+                const float m = fmaxf(nui[p], nuj[q]) * 0.0625f;
+                const bool far_ = hi[p][q] >= m * m;
                 // short secants, the threshold's neighbourhood (the exclusion
                 // is decided in FP64) and lengths outside FP32's safe range:
                 // squares overflow above it, and below it their residuals are
@@ -251,8 +283,13 @@ __global__ void __launch_bounds__(256) w_pair_kernel(const float *X, int N, int 
                 // below 2^-50 down to d^2 = 1e-25 at the largest n, 16384)
                 if (!far_ || !(hi[p][q] > 1e-25f && hi[p][q] < 1e30f) || fabs(d - eps2) <= 1e-9 * eps2) {
                     d = 0.0;
+                    const float *xr = X + (size_t)i * n, *yr = X + (size_t)j * n;
+#pragma unroll 4
                     for (int l = 0; l < n; ++l) {
-                        const double D = (double)X[(size_t)i * n + l] - (double)X[(size_t)j * n + l];
+                        const float x = xr[l], y = yr[l];
+                        float s, e;
+                        two_diff(x, y, s, e);
+                        const double D = diff64(x, y, s, e);
                         d = fma(D, D, d);
                     }
                 }
@@ -336,7 +373,11 @@ __global__ void __launch_bounds__(256, 3) lap_pair_kernel(const float *X, int N,
             } else if (v.x | v.y) {
                 const double wv = __hiloint2double((int)v.y, (int)v.x);
 #pragma unroll
-                for (int q = 0; q < 8; ++q) acc[q] = fma(wv, (double)xi[q] - (double)xb[q], acc[q]);
+                for (int q = 0; q < 8; ++q) {
+                    float s, e;
+                    two_diff(xi[q], xb[q], s, e);
+                    acc[q] = fma(wv, diff64(xi[q], xb[q], s, e), acc[q]);
+                }
             }
         }
 #pragma unroll
@@ -708,12 +749,8 @@ sap_status secant_pca(sap_handle h, int k, double *U_out, double *sigma_out)
         PCK(launch_colmean(X64, N, n, sc.part, sc.mean, s));
         gram_kernel<double><<<ggrid, 256, 0, s>>>(X64, sc.mean, sc.R, N, n, sc.Cp);
     } else {
-        std::vector<float> nu(N);
-        PCK(cudaMemcpyAsync(nu.data(), handle_nu(h), (size_t)N * sizeof(float), cudaMemcpyDeviceToHost, s));
-        PCK(cudaStreamSynchronize(s));
-        const double numax = *std::max_element(nu.begin(), nu.end());
         unsigned long long *wp = reinterpret_cast<unsigned long long *>(sc.w);
-        w_pair_kernel<<<(unsigned)ntiles, 256, 0, s>>>(X32, N, n, sc.tiles, eps2, numax * numax / 256.0, wp);
+        w_pair_kernel<<<(unsigned)ntiles, 256, 0, s>>>(X32, N, n, sc.tiles, eps2, handle_nu(h), wp);
         lap_pair_kernel<<<lgrid, 256, 0, s>>>(X32, N, n, wp, nb, sc.R);
         PCK(launch_colmean(X32, N, n, sc.part, sc.mean, s));
         gram_kernel<float><<<ggrid, 256, 0, s>>>(X32, sc.mean, sc.R, N, n, sc.Cp);
