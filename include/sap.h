@@ -171,7 +171,8 @@ sap_status sap_set_basis(sap_handle h, const double *U, int32_t k,
  * column-major) receives the basis, sigma_out (nullable, k) the singular
  * values sqrt(lambda) in descending order.  1 <= k <= min(n, 32).  Resets
  * the iteration counter, like sap_set_basis.  Work memory: 8 B per pair
- * (the lengths) plus 8 N n + 160 n^2 bytes, freed before returning.
+ * (the lengths) plus 8 N n + 32 n^2 bytes (up to 160 n^2 below n = 385),
+ * freed before returning.
  * Synchronises.
  */
 sap_status sap_secant_pca(sap_handle h, int32_t k, double *U_out, double *sigma_out);

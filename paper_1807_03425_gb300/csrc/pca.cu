@@ -49,6 +49,7 @@ int handle_n_dim(sap_handle h);
 const float *handle_x32(sap_handle h);
 const double *handle_x64(sap_handle h);
 double handle_eps2(sap_handle h);
+int handle_sms(sap_handle h);
 const float *handle_nu(sap_handle h);  // ||x_i - mean||, rounded up (FP32/BF16 data)
 sap_status handle_fail(sap_handle h, sap_status s, const char *msg);
 
@@ -393,7 +394,15 @@ __global__ void __launch_bounds__(256, 3) lap_pair_kernel(const float *X, int N,
 // Band z of C[a][b] = sum_i (x_ia - mean_a) R_ib over a 16 x 16 block of (a,
 // b): the rows are cut into bands (with all rows in one block the 49 blocks
 // of n = 100 left most SMs idle: 0.92 ms), added in order by band_sum_kernel.
+// Bands cost n^2 words each, so there are only as many as it takes to give
+// every SM eight blocks (16 at n = 100, one from n = 385 on, which then writes
+// C itself), and none without rows.
 constexpr int kGramBands = 16;
+inline int gram_bands(int N, int n, int sms)
+{
+    const long long blocks = (long long)((n + 15) / 16) * ((n + 15) / 16);
+    return (int)std::max(1ll, std::min({(long long)kGramBands, 8ll * sms / blocks, (N + 31ll) / 32}));
+}
 template <typename TX>
 __global__ void __launch_bounds__(256) gram_kernel(const TX *X, const double *mean, const double *R, int N, int n,
                                                    double *Cp)
@@ -402,7 +411,8 @@ __global__ void __launch_bounds__(256) gram_kernel(const TX *X, const double *me
     const int a0 = blockIdx.x * 16, b0 = blockIdx.y * 16;
     const int ta = threadIdx.x >> 4, tb = threadIdx.x & 15;
     double acc = 0.0;
-    const int rows = (N + 32 * kGramBands - 1) / (32 * kGramBands) * 32, r1 = min(N, ((int)blockIdx.z + 1) * rows);
+    const int step = 32 * (int)gridDim.z;
+    const int rows = (N + step - 1) / step * 32, r1 = min(N, ((int)blockIdx.z + 1) * rows);
     for (int i0 = blockIdx.z * rows; i0 < r1; i0 += 32) {
         __syncthreads();
         for (int idx = threadIdx.x; idx < 32 * 16; idx += 256) {
@@ -418,12 +428,12 @@ __global__ void __launch_bounds__(256) gram_kernel(const TX *X, const double *me
     if (a0 + ta < n && b0 + tb < n) Cp[((size_t)blockIdx.z * n + a0 + ta) * n + b0 + tb] = acc;
 }
 
-__global__ void band_sum_kernel(const double *Cp, int n, double *C)
+__global__ void band_sum_kernel(const double *Cp, int bands, int n, double *C)
 {
     const long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x, nn = (long long)n * n;
     if (idx >= nn) return;
     double acc = 0.0;
-    for (int z = 0; z < kGramBands; ++z) acc += Cp[z * nn + idx];
+    for (int z = 0; z < bands; ++z) acc += Cp[z * nn + idx];
     C[idx] = acc;
 }
 
@@ -735,28 +745,30 @@ sap_status secant_pca(sap_handle h, int k, double *U_out, double *sigma_out)
     PCK(cudaMalloc(&sc.part, colmean_scratch(N, n) * sizeof(double)));
     PCK(cudaMalloc(&sc.C, (size_t)n * n * sizeof(double)));
     PCK(cudaMalloc(&sc.C2, (size_t)n * n * sizeof(double)));
-    PCK(cudaMalloc(&sc.Cp, (size_t)kGramBands * n * n * sizeof(double)));
+    const int bands = gram_bands(N, n, handle_sms(h));
+    if (bands > 1) PCK(cudaMalloc(&sc.Cp, (size_t)bands * n * n * sizeof(double)));
+    double *Cp = bands > 1 ? sc.Cp : sc.C;
     PCK(cudaMalloc(&sc.V, (size_t)n * n * sizeof(double)));
     PCK(cudaMalloc(&sc.V2, (size_t)n * n * sizeof(double)));
     PCK(cudaMalloc(&sc.norms, (size_t)(n + 2) * sizeof(double)));
     PCK(cudaMalloc(&sc.fg, (size_t)n * sizeof(double2)));
     PCK(cudaMalloc(&sc.partner, (size_t)n * sizeof(int)));
     const double eps2 = handle_eps2(h);
-    const dim3 lgrid(nb, (n + PC - 1) / PC), ggrid((n + 15) / 16, (n + 15) / 16, kGramBands);
+    const dim3 lgrid(nb, (n + PC - 1) / PC), ggrid((n + 15) / 16, (n + 15) / 16, bands);
     if (X64) {
         w64_kernel<double><<<(unsigned)ntiles, 256, 0, s>>>(X64, N, n, sc.tiles, eps2, sc.w);
         lap_rows_kernel<double><<<lgrid, 256, 0, s>>>(X64, N, n, sc.w, nb, sc.R);
         PCK(launch_colmean(X64, N, n, sc.part, sc.mean, s));
-        gram_kernel<double><<<ggrid, 256, 0, s>>>(X64, sc.mean, sc.R, N, n, sc.Cp);
+        gram_kernel<double><<<ggrid, 256, 0, s>>>(X64, sc.mean, sc.R, N, n, Cp);
     } else {
         unsigned long long *wp = reinterpret_cast<unsigned long long *>(sc.w);
         w_pair_kernel<<<(unsigned)ntiles, 256, 0, s>>>(X32, N, n, sc.tiles, eps2, handle_nu(h), wp);
         lap_pair_kernel<<<lgrid, 256, 0, s>>>(X32, N, n, wp, nb, sc.R);
         PCK(launch_colmean(X32, N, n, sc.part, sc.mean, s));
-        gram_kernel<float><<<ggrid, 256, 0, s>>>(X32, sc.mean, sc.R, N, n, sc.Cp);
+        gram_kernel<float><<<ggrid, 256, 0, s>>>(X32, sc.mean, sc.R, N, n, Cp);
     }
     PCK(cudaGetLastError());
-    band_sum_kernel<<<(unsigned)(((long long)n * n + 255) / 256), 256, 0, s>>>(sc.Cp, n, sc.C);
+    if (bands > 1) band_sum_kernel<<<(unsigned)(((long long)n * n + 255) / 256), 256, 0, s>>>(Cp, bands, n, sc.C);
     symmetrize_kernel<<<(unsigned)(((long long)n * n + 255) / 256), 256, 0, s>>>(sc.C, n);
     PCK(cudaGetLastError());
     // cyclic Jacobi sweeps: A (= C) towards diag(lambda), V accumulating the
