@@ -210,6 +210,14 @@ __device__ __forceinline__ void add_pair(float &hi, float &lo, float p, float pe
     lo = __fadd_rn(lo, __fadd_rn(e, pe));
 }
 
+// Shared-memory rows that are read 16 bytes at a time: the array and every
+// row start on such a boundary.
+template <int ROWS, int COLS>
+struct __align__(16) Staged {
+    float v[ROWS][COLS];
+    static_assert(COLS * sizeof(float) % 16 == 0, "rows are read as float4");
+};
+
 // x - y in FP64 from the two_diff parts (an overflow of the FP32 difference
 // takes the conversions).
 __device__ __forceinline__ double diff64(float x, float y, float s, float e)
@@ -221,7 +229,8 @@ __device__ __forceinline__ double diff64(float x, float y, float s, float e)
 __global__ void __launch_bounds__(256) w_pair_kernel(const float *X, int N, int n, const int2 *tiles, double eps2,
                                                      const float *nu, unsigned long long *w)
 {
-    __shared__ float xi[PC][PT + 4], xj[PC][PT + 4];
+    __shared__ Staged<PC, PT + 4> xi_, xj_;
+    auto &xi = xi_.v, &xj = xj_.v;
     const int2 IJ = tiles[blockIdx.x];
     const int i0 = IJ.x * PT, j0 = IJ.y * PT;
     const int tr = threadIdx.x >> 4, tc = threadIdx.x & 15;  // 4 x 4 pairs each
@@ -320,7 +329,8 @@ __global__ void __launch_bounds__(256, 3) lap_pair_kernel(const float *X, int N,
                                                        double *R)
 {
     __shared__ uint2 wt[PT][PT + 1];
-    __shared__ float xs[PT][PC];
+    __shared__ Staged<PT, PC> xs_;
+    auto &xs = xs_.v;
     const int I = blockIdx.x, c0 = blockIdx.y * PC;
     const int r = threadIdx.x & (PT - 1), g = threadIdx.x >> 6;  // 4 groups of 8 coordinates
     const int i = I * PT + r;
