@@ -1710,11 +1710,13 @@ sap_status sap_run_batch(sap_handle h, double alpha, int32_t iters, double *hist
     std::vector<long long> w(words);
     CK(cudaMemcpyAsync(w.data(), h->pack, words * sizeof(long long), cudaMemcpyDeviceToHost, h->stream));
     CK(cudaStreamSynchronize(h->stream));
-    for (int b = 0; b < B; ++b)
-        if (w[b]) return kid_result(h, b, h->kids[b], status_error(h->kids[b], (int)w[b]));
-    if (hist) std::memcpy(hist, w.data() + B, (size_t)B * cnt * sizeof(double));
-    if (pairs) std::memcpy(argmins, w.data() + B + (size_t)B * cnt, 2 * (size_t)B * cnt * sizeof(int64_t));
-    return SAP_OK;
+    // the first dataset that failed is reported; the results of those before
+    // it are delivered
+    int good = 0;
+    while (good < B && !w[good]) ++good;
+    if (hist) std::memcpy(hist, w.data() + B, (size_t)good * cnt * sizeof(double));
+    if (pairs) std::memcpy(argmins, w.data() + B + (size_t)B * cnt, 2 * (size_t)good * cnt * sizeof(int64_t));
+    return good < B ? kid_result(h, good, h->kids[good], status_error(h->kids[good], (int)w[good])) : SAP_OK;
 }
 
 } // extern "C"
