@@ -382,11 +382,15 @@ sap_status reset_state(sap_handle h)
 sap_status ensure_hist(sap_handle h, int need)
 {
     if (h->hist_cap >= need) return SAP_OK;
+    const int cap = std::max(need, 1024);
     CK(cudaStreamSynchronize(h->stream));
+    // the buffer through which a history of this length is read
+    const sap_status s = ensure_words(h, &h->pack, &h->pack_cap, gather_words(1, cap, true));
+    if (s != SAP_OK) return s;
     drop_graphs(h);
     dfree(h->hist);
     dfree(h->am);
-    int cap = std::max(need, 1024);
+    h->hist_cap = 0;
     CK(dalloc(&h->hist, cap));
     CK(dalloc(&h->am, cap));
     h->hist_cap = cap;
@@ -1654,6 +1658,12 @@ sap_status sap_run_batch(sap_handle h, double alpha, int32_t iters, double *hist
             cudaStreamWaitEvent(h->stream, h->kid_done[b], 0) != cudaSuccess)
             return fail(h, SAP_E_CUDA, "dataset stream");
     }
+    const int B = (int)h->kids.size(), cnt = iters + 1;
+    const bool pairs = argmins != nullptr;
+    const size_t words = gather_words(B, cnt, pairs);
+    if (!h->views) CK(dalloc(&h->views, B));
+    sap_status st = ensure_words(h, &h->pack, &h->pack_cap, words);
+    if (st != SAP_OK) return st;
     // the batch's graphs replay the datasets' buffers: rebuild them once any
     // dataset dropped its own graphs (new basis, lengths, history buffers ...)
     long long gen = 0;
@@ -1685,7 +1695,6 @@ sap_status sap_run_batch(sap_handle h, double alpha, int32_t iters, double *hist
         return SAP_OK;
     };
     const int chunk = std::min(iters, 16);
-    sap_status st = SAP_OK;
     if (chunk > 0) {
         st = run(chunk, 0, iters / chunk);
         if (st == SAP_OK && iters % chunk) st = run(iters % chunk, 0, 1);
@@ -1693,18 +1702,12 @@ sap_status sap_run_batch(sap_handle h, double alpha, int32_t iters, double *hist
     if (st == SAP_OK) st = run(1, 1, 1);
     if (st != SAP_OK) return st;
     // every dataset's status, ratios and pairs in one copy
-    const int B = (int)h->kids.size(), cnt = iters + 1;
     std::vector<RunView> views(B);
     for (int b = 0; b < B; ++b) {
         sap_handle kid = h->kids[b];
         kid->last_iters = iters;
         views[b] = RunView{kid->hist, kid->am, kid->st};
     }
-    if (!h->views) CK(dalloc(&h->views, B));
-    const bool pairs = argmins != nullptr;
-    const size_t words = gather_words(B, cnt, pairs);
-    st = ensure_words(h, &h->pack, &h->pack_cap, words);
-    if (st != SAP_OK) return st;
     CK(cudaMemcpyAsync(h->views, views.data(), (size_t)B * sizeof(RunView), cudaMemcpyHostToDevice, h->stream));
     CK(launch_gather(h->views, views[0], B, cnt, pairs, h->pack, h->stream));
     std::vector<long long> w(words);
