@@ -108,7 +108,7 @@ struct sap_ctx {
 
     // uneven batch: one ordinary handle per dataset, run together
     bool is_batch = false;
-    bool shared = false;     // a dataset of a batch whose passes together want more SMs than there are
+    int share = 1;           // batch: least tiles per block of the datasets' passes (pass_share)
     std::vector<sap_handle> kids;
     std::vector<cudaEvent_t> kid_done;
     cudaEvent_t fork = nullptr;
@@ -301,7 +301,9 @@ SelectUpdateArgs su_args(sap_handle h, double alpha, int eval_only, const int2 *
     return u;
 }
 
-sap_status enqueue_iteration(sap_handle h, double alpha, int eval_only, Partial *shard_rec = nullptr)
+// share: least tiles per block of the pass (pass_share); 1 where the handle
+// runs alone
+sap_status enqueue_iteration(sap_handle h, double alpha, int eval_only, Partial *shard_rec = nullptr, int share = 1)
 {
     cudaStream_t s = h->stream;
     const Cert c32 = cert_plain_f32(h->n, h->k);
@@ -329,7 +331,7 @@ sap_status enqueue_iteration(sap_handle h, double alpha, int eval_only, Partial 
             CK(launch_plain_f32(a, s));
         }
     } else {
-        sap_status st = restructured_enqueue(h, alpha);
+        sap_status st = restructured_enqueue(h, share);
         if (st != SAP_OK) return st;
         which = 2;
         list = h->cand2;
@@ -343,7 +345,7 @@ sap_status enqueue_iteration(sap_handle h, double alpha, int eval_only, Partial 
             bv.k = h->k;
             bv.cand1 = h->cand1;
             bv.cand2 = h->cand2;
-            bv.shared = h->shared;
+            bv.share = share;
             restructured_fuse_args(h, bv, u);
         }
         Timed t(h, K_UPDATE);
@@ -499,7 +501,6 @@ TuneKey handle_tune_key(sap_handle h)
     std::memcpy(&t.eps_bits, &h->eps, sizeof(double));
     return t;
 }
-bool handle_shared(sap_handle h) { return h->shared; }
 bool &handle_tuning_flag(sap_handle h) { return h->tuning; }
 void handle_shard(sap_handle h, long long *t0, long long *t1)
 {
@@ -1496,9 +1497,9 @@ sap_status sap_create_batch(const void *const *Xs, const int64_t *Ns, int32_t B,
         if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) return cleanup_fail(SAP_E_CUDA);
         h->kid_done.push_back(e);
     }
-    long long want = 0;
-    for (sap_handle kid : h->kids) want += std::min(kid->rs.nwtiles, h->sms);
-    for (sap_handle kid : h->kids) kid->shared = want > h->sms;
+    long long tiles = 0;
+    for (sap_handle kid : h->kids) tiles += kid->rs.nwtiles;
+    h->share = pass_share(tiles, h->sms);
     *out = h;
     return SAP_OK;
 }
@@ -1616,7 +1617,8 @@ static sap_status batch_graph(sap_handle h, double alpha, int eval_only, int chu
     for (size_t b = 0; b < h->kids.size() && s == SAP_OK && e == cudaSuccess; ++b) {
         sap_handle kid = h->kids[b];
         e = cudaStreamWaitEvent(kid->stream, h->fork, 0);
-        for (int c = 0; c < chunk && s == SAP_OK && e == cudaSuccess; ++c) s = enqueue_iteration(kid, alpha, eval_only);
+        for (int c = 0; c < chunk && s == SAP_OK && e == cudaSuccess; ++c) 
+            s = enqueue_iteration(kid, alpha, eval_only, nullptr, h->share);
         if (s == SAP_OK && e == cudaSuccess) e = cudaEventRecord(h->kid_done[b], kid->stream);
         if (s == SAP_OK && e == cudaSuccess) e = cudaStreamWaitEvent(h->stream, h->kid_done[b], 0);
         if (s != SAP_OK) h->err = "dataset " + std::to_string(b) + ": " + kid->err;

@@ -2327,7 +2327,7 @@ sap_status restructured_enqueue_basis(sap_handle h, const BasisView &b, cudaStre
         }
         handle_count_launch(h, 1, &ea, &eb);
         if (ea) cudaEventRecord(ea, s);
-        RCK(launch_pass(p, restructured_pass_grid(h, b.shared), s));
+        RCK(launch_pass(p, restructured_pass_grid(h, b.share), s));
         if (eb) cudaEventRecord(eb, s);
         handle_push_timing(h, 1, ea, eb);
     }
@@ -2417,9 +2417,8 @@ sap_status restructured_enqueue_basis(sap_handle h, const BasisView &b, cudaStre
     return SAP_OK;
 }
 
-sap_status restructured_enqueue(sap_handle h, double alpha)
+sap_status restructured_enqueue(sap_handle h, int share)
 {
-    (void)alpha;
     RestrState &r = restr_state(h);
     cudaStream_t s = handle_stream(h);
     const int k = handle_k(h);
@@ -2436,7 +2435,7 @@ sap_status restructured_enqueue(sap_handle h, double alpha)
     b.Ykt = r.KY;
     b.ops = r.ops;
     b.ops_stride = 2 * op_image_bytes(b.k);
-    b.shared = handle_shared(h);
+    b.share = share;
     b.near_list = r.near_list;
     b.Ydh = r.Ydh;
     b.Ydl = r.Ydl;
@@ -2550,14 +2549,22 @@ int restructured_tier(sap_handle h) { return restructured_tier_for(h, handle_k(h
 
 // A block of the pass occupies its SM (shared memory) and spends 4-5 us on its
 // start and its survivors before and after 0.7 us per tile.  Alone, a pass
-// takes every SM it can use.  Beside other passes that together want more
-// than the SMs there are, blocks of fewer than about 8 tiles would mostly
-// serialise those fixed costs: 16 scenes of 500..12000 points took 246 us per
-// iteration with a block per tile and 205 us with at least 8 tiles each.
-int restructured_pass_grid(sap_handle h, bool shared)
+// takes every SM it can use.  Passes side by side that together have more
+// tiles than there are SMs take as many tiles per block as it needs for all
+// their blocks to be resident at once, up to 8, past which the fixed costs no
+// longer count; an excess of an eighth of the SMs is left to the first blocks
+// that finish.  us per iteration with one tile per block, this rule, and 8 at
+// once: 8 bases over 21 tiles each 48.7, 48.7, 54.0; 4 bases over 45 tiles
+// 34.9, 31.4, 37.8; 4 over 300 tiles 55.9, 39.9, 39.9; 11 datasets of 15 tiles
+// 33.3, 33.3, 39.7; 16 scenes of 500..12000 points 184, 152, 152.
+int pass_share(long long tiles, int sms)
 {
-    const int t = restr_state(h).nwtiles, sms = handle_sms(h);
-    return std::min(shared ? (t + 7) / 8 : t, sms);
+    return (int)std::max(1ll, std::min(8ll, (tiles + sms - 1 - sms / 8) / sms));
+}
+
+int restructured_pass_grid(sap_handle h, int share)
+{
+    return std::min((restr_state(h).nwtiles + share - 1) / share, handle_sms(h));
 }
 
 bool restructured_uses_refine(sap_handle h) { return restructured_tier(h) == 1; }
@@ -2571,7 +2578,7 @@ void restructured_fuse_args(sap_handle h, const BasisView &b, SelectUpdateArgs &
     const int tier = restructured_tier_for(h, b.k);
     if (tier == 5) {
         // the pass left its blocks' best pairs: one block takes the argmin
-        u.pass_parts = restructured_pass_grid(h, b.shared);
+        u.pass_parts = restructured_pass_grid(h, b.share);
         u.grid = 1;
         return;
     }

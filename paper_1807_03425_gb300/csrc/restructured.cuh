@@ -60,8 +60,8 @@ int handle_sms(sap_handle h);
 ProbState *handle_state(sap_handle h);
 const float *handle_x32(sap_handle h);
 const float *handle_u32(sap_handle h);
-int restructured_pass_grid(sap_handle h, bool shared);  // blocks of the all-pairs pass
-bool handle_shared(sap_handle h);  // its passes run beside other datasets' and do not all fit
+int restructured_pass_grid(sap_handle h, int share);  // blocks of the all-pairs pass
+int pass_share(long long tiles, int sms);  // least tiles per block for passes side by side, `tiles` in all
 Partial *handle_partials(sap_handle h);
 double *handle_u64(sap_handle h);
 const float *handle_u32lo(sap_handle h);
@@ -98,7 +98,7 @@ struct BasisView {
     const double *U64;        // n x k FP64 basis, column-major (tiers inside the pass)
     Partial *partials;        // per-block best pairs (tiers inside the pass)
     int2 *near_list = nullptr; // near pairs the pass could not rule out (N entries)
-    bool shared = false;      // its pass runs beside others that together want more than all SMs
+    int share = 1;            // least tiles per block of its pass (pass_share)
 };
 
 // Filter operands of a product: the buffer and the bases' widths.
@@ -124,7 +124,7 @@ sap_status restructured_classify(sap_handle h, int k);  // near list for width k
 sap_status restructured_prepare(sap_handle h);          // X split, norms, lengths, near list
 sap_status restructured_basis_alloc(sap_handle h);      // U operands and Y for k
 sap_status restructured_basis_changed(sap_handle h);    // after the basis's operands were rewritten
-sap_status restructured_enqueue(sap_handle h, double alpha);
+sap_status restructured_enqueue(sap_handle h, int share);
 int restructured_kernels_per_iteration(sap_handle h);
 // Second tier of the restructured form: 0 explicit differences (own
 // launch), 1 double-float Y + refine, 2 explicit differences fused into the

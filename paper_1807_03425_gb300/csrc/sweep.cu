@@ -161,10 +161,10 @@ sap_status upload(sap_handle h, SweepState &sw, const double *U0)
     return SAP_OK;
 }
 
-// The bases' passes run side by side: do they want more SMs than there are?
-bool sweep_shared(sap_handle h, const SweepState &sw)
+// The bases' passes run side by side.
+int sweep_share(sap_handle h, const SweepState &sw)
 {
-    return (long long)sw.kmax * std::min(restr_state(h).nwtiles, handle_sms(h)) > handle_sms(h);
+    return pass_share((long long)sw.kmax * restr_state(h).nwtiles, handle_sms(h));
 }
 
 SelectUpdateArgs update_args(sap_handle h, SweepState &sw, SweepBasis &b, double alpha, int eval_only)
@@ -206,7 +206,7 @@ SelectUpdateArgs update_args(sap_handle h, SweepState &sw, SweepBasis &b, double
     v.k = b.k;
     v.cand1 = b.cand1;
     v.cand2 = b.cand2;
-    v.shared = sweep_shared(h, sw);
+    v.share = sweep_share(h, sw);
     restructured_fuse_args(h, v, u);
     return u;
 }
@@ -243,7 +243,7 @@ sap_status enqueue_iteration(sap_handle h, SweepState &sw, double alpha, int eva
         v.U64 = b.U64;
         v.partials = b.partials;
         v.near_list = b.near_list;
-        v.shared = sweep_shared(h, sw);
+        v.share = sweep_share(h, sw);
         st = restructured_enqueue_basis(h, v, b.stream);
         if (st != SAP_OK) return st;
         const SelectUpdateArgs u = update_args(h, sw, b, alpha, eval_only);

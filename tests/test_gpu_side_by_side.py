@@ -1,0 +1,54 @@
+"""Passes side by side (a sweep's bases, a batch's datasets): how many tiles a
+block takes grows with the tiles there are, and is a property of the call, so
+a dataset evaluated alone runs as on a handle of its own.  Results do not
+depend on it."""
+import time
+
+import numpy as np
+import pytest
+
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def scene(N, n, seed):
+    return W.hyperspectral(N, seed, W.endmembers(1, n), noise=0.02, bf16=False)
+
+
+@pytest.mark.parametrize("N,B", [(260, 3), (763, 8), (763, 9), (1147, 4), (2171, 4)])
+def test_batch_matches_lone_handles(N, B):
+    import paper_1807_03425_gb300 as P
+    n, k, T = 60, 4, 6
+    Xs = [scene(N - 7 * b, n, b) for b in range(B)]
+    with P.SapBatch(Xs) as s:
+        for b in range(B):
+            s.set_basis(b, W.random_basis(n, k, b))
+        first = [s.min_secant(b) for b in range(B)]
+        hist, am = s.run(0.01, T)
+        U = [s.get_basis(b) for b in range(B)]
+    for b in range(B):
+        with P.Sap(Xs[b]) as s:
+            s.set_basis(W.random_basis(n, k, b))
+            assert s.min_secant() == first[b]
+            h, a = s.run(0.01, T)
+            assert np.array_equal(h, hist[b]) and np.array_equal(a, am[b]) and np.array_equal(s.get_basis(), U[b])
+
+
+def test_one_tile_more_does_not_slow_a_batch():
+    """Eleven datasets of 15 tiles each have 13 tiles more than the GPU has
+    SMs: an iteration took 19 % longer than with blocks of one tile each, where
+    ten datasets fit; 1.12 allows for the eleventh and the timing's spread."""
+    import paper_1807_03425_gb300 as P
+    best = []
+    for B in (10, 11):
+        with P.SapBatch([scene(635, 100, b) for b in range(B)]) as s:
+            for b in range(B):
+                s.set_basis(b, W.random_basis(100, 5, b))
+            t = []
+            for _ in range(25):
+                t0 = time.perf_counter()
+                s.run(0.01, 32)
+                t.append(time.perf_counter() - t0)
+        best.append(min(t[1:]))
+    assert best[1] < 1.12 * best[0], best
