@@ -416,6 +416,7 @@ __device__ __forceinline__ float pair_bound(float beta, float nui, float nuj, fl
 constexpr int kConsumerWarps = 16;
 constexpr int kPassThreads = (kConsumerWarps + 2) * 32;
 constexpr int kTmemCols = 256;          // two 128-column accumulators
+constexpr unsigned int kDense = 6;      // flagged columns per lane above which all 32 are evaluated
 constexpr float kFilter = 1.0081f;      // (1 + 2^-7) (1 + 2.8e-4): odd columns' w, FP32 roundings
 
 // A warp's pending pairs, packed with a lower bound of their ratio (pack_cand).
@@ -967,13 +968,77 @@ __global__ void __launch_bounds__(kPassThreads, 1) restr_pass_kernel(const __gri
                 thc2 = thc * thc * 1.000001f;
             }
         }
-        // emission: the uniform test, then each survivor against its own bound
-        const float ut = U * (1.0f + a.cert.rho);
         uint32_t flag = 0u, emit = 0u;
         if (mymin <= thc2 * kFilter)
 #pragma unroll
             for (int e = 0; e < 32; ++e)
                 if (v[e] <= thc2 * kFilter) flag |= 1u << e;
+        // Where the filter tells little (its error is relative to the points'
+        // distances from the mean, and absolute at the scale of the farthest
+        // one: a point far out leaves most pairs flagged, and the lowest bound
+        // says nothing about where the minimum is) the lane's 32 columns are
+        // evaluated eight at a time instead of a pair per lane and turn, with
+        // pair_q's operations, and the true minimum tightens the bound (once
+        // more if that still leaves many).  Per iteration, with one point
+        // 10^4 times farther out: 4116 -> 174 us at N = 3000, n = 100, k = 20
+        // (109 without the point), 158 -> 82 at N = 8192, k = 5 (41), 141 ->
+        // 73 at N = 3000, n = 300, k = 6 (63).  From 7 flagged columns in a
+        // lane on: with 13 and 21 the same took 171 and 187, 86 and 94, 70
+        // and 71 us, and with noise at k = 5 (58) 83 and 96.
+        for (int rep = 0; rep < 2 && __reduce_max_sync(0xffffffffu, (unsigned int)__popc(flag)) > kDense; ++rep) {
+            const bool staged = (EXPL && K <= 12) || ybytes;  // (pass_stages_y)
+            const float *yI = staged ? sI : gI, *yJ = staged ? sJ : gJ;
+            float mn = INFINITY;
+            int mc = col0;
+            flag = 0u;
+#pragma unroll 1
+            for (int c = 0; c < 32; c += 8) {
+                uint64_t q2[4] = {0ull, 0ull, 0ull, 0ull};
+#pragma unroll 4
+                for (int m = 0; m < k; ++m) {
+                    const float yi = staged ? yI[m * T + row] : __ldcg(yI + m * T + row);
+                    const ulonglong2 *g = reinterpret_cast<const ulonglong2 *>(yJ + m * T + col0 + c);
+                    const ulonglong2 ya = staged ? g[0] : __ldcg(g), yb = staged ? g[1] : __ldcg(g + 1);
+                    const uint64_t yy = tc::pk2(yi, yi);
+                    const uint64_t d0 = tc::sub2(yy, ya.x), d1 = tc::sub2(yy, ya.y);
+                    const uint64_t d2 = tc::sub2(yy, yb.x), d3 = tc::sub2(yy, yb.y);
+                    q2[0] = tc::fma2(d0, d0, q2[0]);
+                    q2[1] = tc::fma2(d1, d1, q2[1]);
+                    q2[2] = tc::fma2(d2, d2, q2[2]);
+                    q2[3] = tc::fma2(d3, d3, q2[3]);
+                }
+                const uint4 w4 = *(reinterpret_cast<const uint4 *>(stage) + ((col0 + c) >> 3) * T + row);
+                const uint32_t ww[4] = {w4.x, w4.y, w4.z, w4.w};
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const float2 t = tc::upk2(q2[e >> 1]);
+                    const float w = __uint_as_float((e & 1) ? ww[e >> 1] & 0xffff0000u : ww[e >> 1] << 16) * wsc;
+                    const float q = ((e & 1) ? t.y : t.x) * w;
+                    if (q < mn) {
+                        mn = q;
+                        mc = col0 + c + e;
+                    }
+                    if (q <= thc2) flag |= 1u << (c + e);
+                }
+            }
+            const float qmin = warp_min(mn);
+            if (!(qmin <= thc2)) break;
+            const int src = __ffs(__ballot_sync(0xffffffffu, mn == qmin)) - 1;
+            float ub = INFINITY;
+            if (lane == src) {
+                const float w = __uint_as_float((uint32_t)hs[((mc >> 3) * T + row) * 8 + (mc & 7)] << 16) * wsc;
+                const float r = sqrt_up(qmin);
+                if (r < U) ub = (r + pair_bound(a.beta, nuI[row], nuJ[mc], w)) * inv_up;
+            }
+            ub = __shfl_sync(0xffffffffu, ub, src);
+            if (!(ub < U)) break;
+            lower_bound_to(ub);
+            U = ub;
+            thc = cert_emit_threshold(U, a.cert);
+            thc2 = thc * thc * 1.000001f;
+        }
+        // emission: the uniform test, then each survivor against its own bound
+        const float ut = U * (1.0f + a.cert.rho);
         const int i0 = IJ.x * T, j0 = IJ.y * T;
         if constexpr (EXPL) {
             int total = 0;
