@@ -2334,12 +2334,26 @@ sap_status restructured_enqueue_product(sap_handle h, const CUtensorMap *mhi, co
     return SAP_OK;
 }
 
+// Does the pass of the double-float tier look at the near pairs itself, so that
+// the pairs left can be evaluated one by one (pair mode)?  That takes the pass
+// a gather of 2 k words per near pair, and pays only if it leaves at most N
+// pairs.  us per iteration without and with it: 20 bases side by side over N =
+// 4000 points, n = 2000, 4 000 near pairs 1754, 885; 159 000 1853, 1442; 319 000
+// 1912, 1971; 799 000 2093, 3351; N = 1500 = n, 112 000 673, 538; 563 000 853,
+// 1002; one basis (k = 6) over N = 3000, n = 300, 90 000 70, 68; 181 000 72, 78;
+// 2 249 000 113, 261.  Hence at most 80 per point and a tenth of N n.
+bool pairs_pay(long long N, int n, int k, long long n_near)
+{
+    return k <= 24 && n_near <= 80 * N && 10 * n_near <= N * n;
+}
+
 sap_status restructured_enqueue_basis(sap_handle h, const BasisView &b, cudaStream_t s)
 {
     RestrState &r = restr_state(h);
     const int n = handle_n_dim(h);
     cudaEvent_t ea, eb;
     const int tier = restructured_tier_for(h, b.k);
+    const bool pairs = tier == 1 && b.near_list && pairs_pay(handle_n_points(h), n, b.k, r.n_near);
     {
         PassArgs p;
         p.wb = r.wb;
@@ -2380,11 +2394,13 @@ sap_status restructured_enqueue_basis(sap_handle h, const BasisView &b, cudaStre
         }
         if (tier == 1 && b.near_list) {
             p.N = (int)handle_n_points(h);
-            p.near = r.near;
-            p.near_w = r.near_w;
-            p.n_near = r.n_near;
-            p.near_out = b.near_list;
-            p.near_cap = (int)handle_n_points(h);
+            if (pairs) {
+                p.near = r.near;
+                p.near_w = r.near_w;
+                p.n_near = r.n_near;
+                p.near_out = b.near_list;
+                p.near_cap = (int)handle_n_points(h);
+            }
             p.w32 = r.w;
             p.nb = r.Npad / T;
             p.tile0 = r.tile0;
@@ -2396,7 +2412,7 @@ sap_status restructured_enqueue_basis(sap_handle h, const BasisView &b, cudaStre
         if (eb) cudaEventRecord(eb, s);
         handle_push_timing(h, 1, ea, eb);
     }
-    const long long pair_max = tier == 1 && b.k <= 24 && b.near_list ? handle_n_points(h) : -1;
+    const long long pair_max = pairs ? handle_n_points(h) : -1;
     if (tier == 2 || tier == 3 || tier == 5) {
         // the explicit tier runs inside the FP64 recheck (restructured_fuse_args)
         // or (5) inside the pass
