@@ -1567,7 +1567,6 @@ struct YdfArgs {
     long long pair_max = -1;
     const int2 *cand1 = nullptr, *near_list = nullptr;
     Cert cert;               // of the extended-precision explicit evaluation
-    int k = 0;
     unsigned long long *cand2 = nullptr;
     long long cap2 = 0;
 };
@@ -1980,11 +1979,6 @@ float cert_pass32(int n, int k)
     auto g = [&](double m) { return m * u / (1.0 - m * u); };
     return (float)((g(n + 2) + g(k) + 8 * u) * 1.05);
 }
-
-// Extended-precision tier: 2^-24 absolute from the rounding of D (U
-// orthonormal), n^1.5 2^-46 from the hi + lo accumulation; relative: the
-// rounding of d, the FP32 squares and sum of the k components, the division
-// and the square root.
 
 // Explicit tier in extended precision for large n (the FP32 tier's
 // gamma_{n+3} bound grows with n).
@@ -2459,7 +2453,6 @@ sap_status restructured_enqueue_basis(sap_handle h, const BasisView &b, cudaStre
         y.cand1 = b.cand1;
         y.near_list = b.near_list;
         y.cert = cert_explicit_df(n, b.k);
-        y.k = b.k;
         y.cand2 = reinterpret_cast<unsigned long long *>(b.cand2);
         y.cap2 = b.cap;
         RefineArgs x;
