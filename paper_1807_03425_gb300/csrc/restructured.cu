@@ -985,7 +985,17 @@ __global__ void __launch_bounds__(kPassThreads, 1) restr_pass_kernel(const __gri
         // 73 at N = 3000, n = 300, k = 6 (63).  From 7 flagged columns in a
         // lane on: with 13 and 21 the same took 171 and 187, 86 and 94, 70
         // and 71 us, and with noise at k = 5 (58) 83 and 96.
-        for (int rep = 0; rep < 2 && __reduce_max_sync(0xffffffffu, (unsigned int)__popc(flag)) > kDense; ++rep) {
+        bool many = __reduce_max_sync(0xffffffffu, (unsigned int)__popc(flag)) > kDense;
+        if (many) {
+            // The lanes read the bound each for itself and other warps lower
+            // it meanwhile, so it may differ between them.  What follows
+            // leaves its loop by comparisons with it and meets in warp-wide
+            // operations: one value for the warp (any lane's is valid).
+            U = __shfl_sync(0xffffffffu, U, 0);
+            thc = cert_emit_threshold(U, a.cert);
+            thc2 = thc * thc * 1.000001f;
+        }
+        for (int rep = 0; rep < 2 && many; ++rep) {
             const bool staged = (EXPL && K <= 12) || ybytes;  // (pass_stages_y)
             const float *yI = staged ? sI : gI, *yJ = staged ? sJ : gJ;
             float mn = INFINITY;
@@ -1036,6 +1046,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) restr_pass_kernel(const __gri
             U = ub;
             thc = cert_emit_threshold(U, a.cert);
             thc2 = thc * thc * 1.000001f;
+            many = __reduce_max_sync(0xffffffffu, (unsigned int)__popc(flag)) > kDense;
         }
         // emission: the uniform test, then each survivor against its own bound
         const float ut = U * (1.0f + a.cert.rho);
